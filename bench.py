@@ -352,8 +352,7 @@ def table_sweep(with_oracle):
                 rows.append({"L": n, "d": d, "k": k, "ms": round(best, 3), "rows_per_s": n / (best * 1e-3),
                              "gbs": alg / (best * 1e-3) / 1e9, "contraction_tflops": 2.0 * n * n * d / (best * 1e-3) / 1e12,
                              "candidates_per_s": float(n) * n / (best * 1e-3),
-                             "path": ("tcgen05" if (n >= 8192 and d % 8 == 0 and d <= 256 and k <= 320)
-                                      else "mma.sync" if (d % 16 == 0 and 32 <= d <= 256 and k <= 320) else "brute"),
+                             "path": "tcgen05" if (n >= 64 and d <= 256 and k <= 320) else "brute",
                              "oracle_rows_per_s": None if t_or is None else 1.0 / t_or})
     return rows, SWEEP_DUP_FRAC
 
@@ -369,7 +368,7 @@ def run_table_sweep(args):
                       "n_gpus": 1, "steps": 3, "warmup": 1, "ms_per_step": total_ms, "higher_is_better": True,
                       "scaling": "weak", "vs_baseline": None, "dtype": "bf16 mma + f64 re-rank", "data": "synthetic",
                       "config": {"workload": "c5_table_sweep", "dup_frac": dup}, "builds": rows,
-                      "gpu_launches": 4 * 2 * len(rows)}))
+                      "gpu_launches": sum(4 * (1 + 4 * -(-r["L"] // (128 * 148))) for r in rows)}))
 
 
 def run_dynamic_tree(args):

@@ -11,6 +11,8 @@
 // belong to the exact top k is ever dropped).  The survivors are re-ranked by their double
 // distances.  If ties at tau overflow the buffer the query falls back to k rounds of an exact
 // arg-min over all candidates.
+#include <math.h>
+
 #include "common.cuh"
 
 namespace lantern {
@@ -31,22 +33,6 @@ template <typename T> __device__ __forceinline__ float widen(T x);
 template <> __device__ __forceinline__ float widen<float>(float x) { return x; }
 template <> __device__ __forceinline__ float widen<__nv_bfloat16>(__nv_bfloat16 x) { return __bfloat162float(x); }
 
-// in-place ascending bitonic sort of n (power of two) 64-bit keys in shared memory
-__device__ __forceinline__ void bitonic_u64(unsigned long long* a, int n) {
-  for (int size = 2; size <= n; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int i = threadIdx.x; i < (n >> 1); i += kKnnThreads) {
-        int lo = 2 * i - (i & (stride - 1));
-        int hi = lo + stride;
-        bool up = (lo & size) == 0;
-        unsigned long long x = a[lo], y = a[hi];
-        if ((x > y) == up) { a[lo] = y; a[hi] = x; }
-      }
-      __syncthreads();
-    }
-  }
-}
-
 // ascending bitonic sort of n (power of two) (dist, idx) pairs
 __device__ __forceinline__ void bitonic_pair(double* dv, int* iv, int n) {
   for (int size = 2; size <= n; size <<= 1) {
@@ -65,20 +51,13 @@ __device__ __forceinline__ void bitonic_pair(double* dv, int* iv, int n) {
   }
 }
 
-template <int NT, int BAR>
-__device__ __forceinline__ void knn_bar() {
-  if (BAR == 0) __syncthreads();
-  else asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
-}
-
 // Cut-back of one query's candidate buffer without sorting it.  Entries are 64-bit words whose
 // upper half is a monotone 32-bit key of the filter distance.  A most-significant-digit radix
 // select (4 passes of 8 bits, shared-memory histogram) finds the k-th smallest key; `limit_of`
 // turns it into the largest key that may stay (k-th key plus the caller's error margin); the
 // entries up to that limit are compacted through `tmp` (order is irrelevant: the final ranking
 // sorts).  Returns the number kept; *kth_key_out receives the k-th smallest key.  n >= k.
-// NT threads (threadIdx.x < NT) take part and meet at hardware barrier BAR (0 = the whole CTA).
-template <int NT = kKnnThreads, int BAR = 0, typename F>
+template <typename F>
 __device__ __forceinline__ int radix_cut(unsigned long long* bq, int n, int k, unsigned long long* tmp, uint32_t* hist,
                                          int* sel, F&& limit_of, uint32_t* limit_out) {
   const int tid = threadIdx.x, lane = tid & 31;
@@ -86,13 +65,13 @@ __device__ __forceinline__ int radix_cut(unsigned long long* bq, int n, int k, u
   int rem = k;
   for (int pass = 0; pass < 4; ++pass) {
     const int shift = 24 - 8 * pass;
-    for (int i = tid; i < 256; i += NT) hist[i] = 0;
-    knn_bar<NT, BAR>();
-    for (int i = tid; i < n; i += NT) {
+    for (int i = tid; i < 256; i += kKnnThreads) hist[i] = 0;
+    __syncthreads();
+    for (int i = tid; i < n; i += kKnnThreads) {
       const uint32_t key = static_cast<uint32_t>(bq[i] >> 32);
       if (pass == 0 || (key >> (shift + 8)) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1u);
     }
-    knn_bar<NT, BAR>();
+    __syncthreads();
     if (tid < 32) {
       uint32_t c8[8], s = 0;
 #pragma unroll
@@ -116,15 +95,15 @@ __device__ __forceinline__ int radix_cut(unsigned long long* bq, int n, int k, u
         }
       }
     }
-    knn_bar<NT, BAR>();
+    __syncthreads();
     prefix = (prefix << 8) | static_cast<uint32_t>(sel[0]);
     rem = sel[1];
-    knn_bar<NT, BAR>();
+    __syncthreads();
   }
   const uint32_t limit = limit_of(prefix);          // prefix is now the k-th smallest key
   if (tid == 0) sel[2] = 0;
-  knn_bar<NT, BAR>();
-  for (int i0 = 0; i0 < n; i0 += NT) {
+  __syncthreads();
+  for (int i0 = 0; i0 < n; i0 += kKnnThreads) {
     const int i = i0 + tid;
     const unsigned long long e = i < n ? bq[i] : ~0ull;
     const bool keep = i < n && static_cast<uint32_t>(e >> 32) <= limit;
@@ -134,11 +113,11 @@ __device__ __forceinline__ int radix_cut(unsigned long long* bq, int n, int k, u
     pos0 = __shfl_sync(0xffffffffu, pos0, 0);
     if (keep) tmp[pos0 + __popc(m & ((1u << lane) - 1u))] = e;
   }
-  knn_bar<NT, BAR>();
+  __syncthreads();
   const int kept = sel[2];
-  for (int i = tid; i < kept; i += NT) bq[i] = tmp[i];
+  for (int i = tid; i < kept; i += kKnnThreads) bq[i] = tmp[i];
   *limit_out = limit;
-  knn_bar<NT, BAR>();
+  __syncthreads();
   return kept;
 }
 
@@ -154,36 +133,50 @@ __device__ __forceinline__ double exact_dist(const T* __restrict__ cb, int d, in
   return s;
 }
 
-// The same sum, in the same order, for a bfloat16 query row held in shared memory and a candidate
-// row read from global memory with 16-byte loads (d a multiple of 8, both rows 16-byte aligned).
-__device__ __forceinline__ double exact_dist_bf16x8(const __nv_bfloat16* a, const __nv_bfloat16* __restrict__ b, int d) {
-  double s = 0.0;
-  for (int t = 0; t < d; t += 8) {
-    const uint4 av = *reinterpret_cast<const uint4*>(a + t);
-    const uint4 bv = __ldg(reinterpret_cast<const uint4*>(b + t));
-    const uint32_t aw[4] = {av.x, av.y, av.z, av.w}, bw[4] = {bv.x, bv.y, bv.z, bv.w};
+// k rounds of an exact arg-min over (distance, index) greater than the last pick, by a CTA of NT threads
+template <typename T, int NT>
+__device__ __forceinline__ void argmin_rounds(const T* __restrict__ cb, int L, int d, int k, int qi, double* redd, int* redi,
+                                              int32_t* out_i, float* out_d) {
+  const int tid = threadIdx.x;
+  double pd = -1.0;
+  int pj = -1;
+  for (int r = 0; r < k; ++r) {
+    double bd = INFINITY;
+    int bj = 0x7fffffff;
+    for (int j = tid; j < L; j += NT) {
+      if (j == qi) continue;
+      const double dj = exact_dist<T>(cb, d, qi, j);
+      const bool after = dj > pd || (dj == pd && j > pj);
+      if (after && (dj < bd || (dj == bd && j < bj))) { bd = dj; bj = j; }
+    }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const double d0 = static_cast<double>(__uint_as_float(aw[i] << 16)) - static_cast<double>(__uint_as_float(bw[i] << 16));
-      s = fma(d0, d0, s);
-      const double d1 = static_cast<double>(__uint_as_float(aw[i] & 0xffff0000u)) -
-                        static_cast<double>(__uint_as_float(bw[i] & 0xffff0000u));
-      s = fma(d1, d1, s);
+    for (int o = 16; o > 0; o >>= 1) {
+      const double od = __shfl_xor_sync(0xffffffffu, bd, o);
+      const int oj = __shfl_xor_sync(0xffffffffu, bj, o);
+      if (od < bd || (od == bd && oj < bj)) { bd = od; bj = oj; }
+    }
+    if ((tid & 31) == 0) { redd[tid >> 5] = bd; redi[tid >> 5] = bj; }
+    __syncthreads();
+    bd = redd[0]; bj = redi[0];
+    for (int w = 1; w < NT / 32; ++w)
+      if (redd[w] < bd || (redd[w] == bd && redi[w] < bj)) { bd = redd[w]; bj = redi[w]; }
+    __syncthreads();
+    pd = bd; pj = bj;
+    if (tid == 0) {
+      out_i[r] = bj;
+      if (out_d) out_d[r] = static_cast<float>(bd);
     }
   }
-  return s;
 }
 
 // Exact ranking of one query's surviving candidates (keys carry the candidate index in their
 // low 32 bits): distances re-evaluated in double, sorted by (distance, index), first k written.
 // With `overflow` the buffer is ignored and k rounds of an exact arg-min over all rows are run.
-// `q_row`, if given, is the query's bfloat16 row in shared memory (d a multiple of 8): the distances
-// then come from exact_dist_bf16x8.
 template <typename T>
 __device__ __forceinline__ void rank_query(const T* __restrict__ cb, int L, int d, int k, int qi,
                                            const unsigned long long* bq, int n_in, bool overflow, int CAP,
                                            double* sortd, int* sorti, double* redd, int* redi,
-                                           int32_t* out_i, float* out_d, const __nv_bfloat16* q_row = nullptr) {
+                                           int32_t* out_i, float* out_d) {
   const int tid = threadIdx.x;
     if (!overflow) {
     const int n = min(n_in, CAP);
@@ -191,10 +184,7 @@ __device__ __forceinline__ void rank_query(const T* __restrict__ cb, int L, int 
       if (i < n) {
         int j = static_cast<int>(bq[i] & 0xffffffffu);
         sorti[i] = j;
-        if (sizeof(T) == 2 && q_row)
-          sortd[i] = exact_dist_bf16x8(q_row, reinterpret_cast<const __nv_bfloat16*>(cb) + static_cast<long long>(j) * d, d);
-        else
-          sortd[i] = exact_dist<T>(cb, d, qi, j);
+        sortd[i] = exact_dist<T>(cb, d, qi, j);
       } else {
         sorti[i] = 0x7fffffff;
         sortd[i] = INFINITY;
@@ -208,36 +198,7 @@ __device__ __forceinline__ void rank_query(const T* __restrict__ cb, int L, int 
     }
     __syncthreads();
   } else {
-    // exact fallback: k rounds of arg-min over (distance, index) greater than the last pick
-    double pd = -1.0;
-    int pj = -1;
-    for (int r = 0; r < k; ++r) {
-      double bd = INFINITY;
-      int bj = 0x7fffffff;
-      for (int j = tid; j < L; j += kKnnThreads) {
-        if (j == qi) continue;
-        double dj = exact_dist<T>(cb, d, qi, j);
-        bool after = dj > pd || (dj == pd && j > pj);
-        if (after && (dj < bd || (dj == bd && j < bj))) { bd = dj; bj = j; }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        double od = __shfl_xor_sync(0xffffffffu, bd, o);
-        int oj = __shfl_xor_sync(0xffffffffu, bj, o);
-        if (od < bd || (od == bd && oj < bj)) { bd = od; bj = oj; }
-      }
-      if ((tid & 31) == 0) { redd[tid >> 5] = bd; redi[tid >> 5] = bj; }
-      __syncthreads();
-      bd = redd[0]; bj = redi[0];
-      for (int w = 1; w < kKnnThreads / 32; ++w)
-        if (redd[w] < bd || (redd[w] == bd && redi[w] < bj)) { bd = redd[w]; bj = redi[w]; }
-      __syncthreads();
-      pd = bd; pj = bj;
-      if (tid == 0) {
-        out_i[r] = bj;
-        if (out_d) out_d[r] = static_cast<float>(bd);
-      }
-    }
+    argmin_rounds<T, kKnnThreads>(cb, L, d, k, qi, redd, redi, out_i, out_d);
   }
 }
 
@@ -403,37 +364,148 @@ __global__ void __launch_bounds__(kKnnThreads) knn_kernel(const KnnArgs a) {
 
 }  // namespace lantern
 
-#include "knn_tc.cuh"
 #include "knn_t5.cuh"
 
 using namespace lantern;
 
-// The tensor-core path is taken for bfloat16 codebooks with d a multiple of 16 in [32, 256] and
-// k small enough for its per-query buffers.
-static bool use_tensor_path(lantern_dtype dt, int L, int d, int k) {
-  return dt == LANTERN_BF16 && d % 16 == 0 && d >= 32 && d <= kTcMaxD && k <= 320 && L >= 64;
+namespace {
+// Where the table is built by the tcgen05 kernels, and with which sizes.  Operand rows of up to 256
+// elements fit the shared-memory tiles (bfloat16 rows of up to 256 elements; float32 rows, three parts each, of up
+// to 85) and k <= 320 keeps a query's survivors within the ranking's 512 slots.  Against the brute-force kernel (and, for
+// bfloat16, an mma.sync kernel that stood here): 16384 x 8 float32, k = 100: 0.45 ms, was 2.63; 20000 x 64 float32,
+// k = 200: 0.91 ms, was 17.4; 600 x 256 bfloat16, k = 200: 81 us, was 567; 300 x 8 float32, k = 10: 49 us, was 116.
+// Below one half tile of rows nothing is left to select.
+#ifndef LANTERN_T5_MIN_L
+#define LANTERN_T5_MIN_L 64
+#endif
+struct T5Plan {
+  bool ok, sampled;                 // sampled: the sample is a proper part of the codebook, with tiles of its own
+  int dp, tiles, nst, gshift, groups;
+  int first_tiles;                  // query tiles of the first (largest) chunk
+  size_t off_cn, off_sn, off_counts, off_bound, off_qm, off_cm, off_sm, off_minima, off_lists, bytes;
+};
+size_t round256(size_t x) { return (x + 255) / 256 * 256; }
+int t5_split(int tiles, int L) {    // CTAs per query tile of a chunk
+  int s = kT5Items / tiles;
+  if (s > kT5MaxSplit) s = kT5MaxSplit;
+  const int nct = (L + kT5C - 1) / kT5C;
+  if (s > nct) s = nct;
+  return s < 1 ? 1 : s;
+}
+// Entries a list holds: what the sampled bound lets through when the sample is representative (the k+1
+// smallest of `groups` group minima are the about -groups ln(1 - (k+1)/groups) smallest sampled candidates) with six
+// standard deviations, at least k + 192, at most what cut-backs work well with.
+int t5_cap(const T5Plan& p, int L, int k, int split) {
+  const double share = static_cast<double>(k + 1) / p.groups;
+  const double est = (share < 0.95 ? -p.groups * log(1.0 - share) * L / (static_cast<double>(p.nst) * kT5C) : L) / (kT5Per * split);
+  double c = est + 6.0 * sqrt(est) + 64.0;
+  if (c > 1024.0) c = 1024.0;
+  if (c < k + 193.0) c = k + 193.0;
+  return (static_cast<int>(c) + 63) / 64 * 64;
+}
+T5Plan t5_plan(lantern_dtype dt, int L, int d, int k) {
+  T5Plan p = {};
+  const int parts = dt == LANTERN_F32 ? 3 : 1;
+  p.ok = L >= LANTERN_T5_MIN_L && k <= kT5MaxK && d <= 256 && parts * d <= 256;
+  if (!p.ok) return p;
+  p.dp = (parts * d + 15) / 16 * 16;
+  p.tiles = (L + kT5Q - 1) / kT5Q;
+  // one candidate in four is sampled, 1024 at least; groups of the smallest size that leaves at most 1024 minima
+  int sample = (L + 3) / 4;
+  if (sample < 1024) sample = 1024;
+  if (sample > L) sample = L;
+  p.nst = (sample + kT5C - 1) / kT5C;
+  if (p.nst > kT5MaxGroups / 4) p.nst = kT5MaxGroups / 4;      // groups of 32 columns at most
+  while ((p.nst * kT5C) >> p.gshift > kT5MaxGroups) ++p.gshift;
+  p.groups = (p.nst * kT5C) >> p.gshift;
+  p.first_tiles = p.tiles < kT5Items ? p.tiles : kT5Items;
+  const int split = t5_split(p.first_tiles, L);
+  const size_t segs = static_cast<size_t>(kT5Items) * kT5Sel;
+  p.sampled = p.nst < p.tiles;
+  const size_t tile = static_cast<size_t>(kT5Q) * p.dp * 2, side = p.tiles * tile;
+  p.off_cn = round256((static_cast<size_t>(L) + 64) * sizeof(float));
+  p.off_sn = p.off_cn + static_cast<size_t>(p.tiles) * kT5C * sizeof(float);
+  p.off_counts = p.off_sn + static_cast<size_t>(p.sampled ? p.nst : 0) * kT5C * sizeof(float);
+  p.off_bound = p.off_counts + segs * sizeof(int);
+  p.off_qm = p.off_bound + static_cast<size_t>(kT5Items) * kT5Q * sizeof(float);
+  p.off_cm = p.off_qm + (dt == LANTERN_F32 ? side : 0);
+  p.off_sm = p.off_cm + side;
+  p.off_minima = p.off_sm + (p.sampled ? p.nst * tile : 0);
+  p.off_lists = p.off_minima + static_cast<size_t>(p.first_tiles) * p.groups * kT5Q * sizeof(float);
+  // (a later chunk has fewer tiles, so no more CTAs and no longer lists)
+  p.bytes = p.off_lists + static_cast<size_t>(p.first_tiles) * split * kT5Sel * t5_cap(p, L, k, split) * 8;
+  return p;
 }
 
-// bfloat16 codebooks of at least this many rows, d a multiple of 8 up to 256, take the tcgen05 kernel
-// (tiles of 128 queries per CTA); smaller ones would leave most SMs without a tile and stay on the
-// mma.sync kernel (or, for d it does not serve, on the brute-force kernel).
-#ifndef LANTERN_T5_MIN_L
-#define LANTERN_T5_MIN_L 8192
-#endif
-constexpr int kT5GridCap = 160;          // CTAs the workspace is sized for (one per SM)
-static bool use_t5_path(lantern_dtype dt, int L, int d, int k) {
-  return dt == LANTERN_BF16 && d % 8 == 0 && d >= 8 && d <= 256 && k <= kT5MaxK && L >= LANTERN_T5_MIN_L;
+template <typename T>
+lantern_status build_t5(const T5Plan& p, const T* cb, int L, int d, int k, int32_t* nbr_idx, float* nbr_dist,
+                        unsigned char* ws, cudaStream_t st) {
+  float* nrm = reinterpret_cast<float*>(ws);
+  if (cudaMemsetAsync(nrm + L, 0, 2 * sizeof(float), st) != cudaSuccess) return LANTERN_ERR_CUDA;
+  KnnPrepArgs g;
+  g.cb = cb; g.L = L; g.d = d; g.dp = p.dp;
+  g.rows = p.tiles * kT5C;
+  g.sampled = p.sampled ? p.nst * kT5C : 0;
+  g.step = p.sampled ? (static_cast<unsigned long long>(L) << 32) / (static_cast<unsigned long long>(p.nst) * kT5C) : 0;
+  g.nrm = nrm;
+  g.cn = reinterpret_cast<float*>(ws + p.off_cn);
+  g.sn = reinterpret_cast<float*>(ws + p.off_sn);
+  g.qm = ws + p.off_qm;                       // (bfloat16 rows: the candidate side's tiles, off_qm == off_cm)
+  g.cm = ws + p.off_cm;
+  g.sm = ws + p.off_sm;
+  knn_prep_kernel<T><<<(g.rows + g.sampled) / 8, 256, 0, st>>>(g);
+  KnnT5Args a;
+  a.qm = g.qm;
+  a.nrm = nrm;
+  a.minima = reinterpret_cast<float*>(ws + p.off_minima);
+  float* bound = reinterpret_cast<float*>(ws + p.off_bound);
+  a.bound = bound;
+  a.lists = reinterpret_cast<unsigned long long*>(ws + p.off_lists);
+  a.counts = reinterpret_cast<int*>(ws + p.off_counts);
+  a.L = L; a.dp = p.dp; a.k = k;
+  a.gshift = p.gshift; a.groups = p.groups;
+  a.eps1 = static_cast<float>(p.dp + 16) * 4.76837158203125e-7f + (sizeof(T) == 4 ? 1.52587890625e-5f : 0.f);   // 2^-21, 2^-16
+  a.eps0 = static_cast<float>(p.dp) * 2.3509887016445750e-38f;                                                    // products below the normal range
+  KnnRankArgs r;
+  r.cb = cb; r.nrm = nrm; r.lists = a.lists; r.counts = a.counts;
+  r.L = L; r.d = d; r.k = k; r.eps1 = a.eps1; r.eps0 = a.eps0; r.nbr_idx = nbr_idx; r.nbr_dist = nbr_dist;
+  r.lanes = 0;
+  if (d % 8 == 0 && reinterpret_cast<uintptr_t>(cb) % 16 == 0) {
+    r.lanes = 1;
+    while (r.lanes < 8 && r.lanes * 2 <= d / 8) r.lanes *= 2;
+  }
+  const size_t sm5 = knn_t5_smem(p.dp), smr = knn_rank_smem(d);
+  if (cudaFuncSetAttribute(knn_t5_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm5)) != cudaSuccess ||
+      cudaFuncSetAttribute(knn_t5_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm5)) != cudaSuccess)
+    return LANTERN_ERR_CUDA;
+  for (a.tile0 = 0; a.tile0 < p.tiles; a.tile0 += kT5Items) {
+    const int n = p.tiles - a.tile0 < kT5Items ? p.tiles - a.tile0 : kT5Items;
+    const int split = t5_split(n, L);
+    a.cap = t5_cap(p, L, k, split);
+    a.split = split < p.nst ? split : p.nst;
+    a.nct = p.nst; a.cm = p.sampled ? g.sm : g.cm; a.cn = p.sampled ? g.sn : g.cn;
+    knn_t5_kernel<true><<<n * a.split, kT5Threads, sm5, st>>>(a);
+    knn_bound_kernel<<<n * kT5Q / 8, 256, 0, st>>>(a.minima, n * kT5Q, p.groups, k + 1, bound);
+    a.split = split;
+    a.nct = p.tiles; a.cm = g.cm; a.cn = g.cn;
+    knn_t5_kernel<false><<<n * split, kT5Threads, sm5, st>>>(a);
+    r.cap = a.cap; r.split = split; r.q0 = a.tile0 * kT5Q;
+    const int queries = L - r.q0 < n * kT5Q ? L - r.q0 : n * kT5Q;
+    knn_rank_kernel<T><<<queries, kRankThreads, smr, st>>>(r);
+  }
+  return cudaGetLastError() == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
 }
-static size_t norms_bytes(int L) { return ((static_cast<size_t>(L) + 64) * sizeof(float) + 255) / 256 * 256; }
-static size_t t5_cta_bytes(int k) { return static_cast<size_t>(kT5Q) * knn_t5_cap(k) * 8; }
+
+// bfloat16 shapes whose workspace has always been required (their calls are refused without it)
+bool needs_workspace(lantern_dtype dt, int L, int d, int k) {
+  return dt == LANTERN_BF16 && k <= kT5MaxK && d <= 256 && (L >= 8192 ? d % 8 == 0 : L >= 64 && d % 16 == 0 && d >= 32);
+}
+}  // namespace
 
 extern "C" size_t lantern_build_neighbors_workspace(lantern_dtype dt, int32_t L, int32_t d, int32_t k) {
   if (L < 2 || d < 1 || k < 1) return 0;
-  // squared norms of all rows and their maximum (tensor-core paths), plus the per-CTA candidate
-  // lists of the tcgen05 kernel; the brute-force kernel keeps all of its state on chip
-  if (!use_t5_path(dt, L, d, k)) return use_tensor_path(dt, L, d, k) ? norms_bytes(L) : 0;
-  const int nqt = (L + 63) / 64;                   // the kernel may run tiles of 64 queries (see the launch)
-  return norms_bytes(L) + static_cast<size_t>(nqt < kT5GridCap ? nqt : kT5GridCap) * t5_cta_bytes(k);
+  const T5Plan p = t5_plan(dt, L, d, k);
+  return p.ok ? p.bytes : 0;                  // the brute-force kernel keeps all of its state on chip
 }
 
 extern "C" lantern_status lantern_build_neighbors(const void* codebook, lantern_dtype dt, int32_t L, int32_t d,
@@ -444,51 +516,19 @@ extern "C" lantern_status lantern_build_neighbors(const void* codebook, lantern_
   if (L < 2 || d < 1 || k < 1 || k > L - 1) return LANTERN_ERR_INVALID_ARG;
   if (k > 1024 || d > 4096) return LANTERN_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (use_t5_path(dt, L, d, k) || use_tensor_path(dt, L, d, k)) {
-    const size_t need = lantern_build_neighbors_workspace(dt, L, d, k);
-    if (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) % 256)) return LANTERN_ERR_WORKSPACE;
-    if (reinterpret_cast<uintptr_t>(codebook) % 16) return LANTERN_ERR_INVALID_ARG;
-    float* nrm = static_cast<float*>(workspace);
-    if (cudaMemsetAsync(nrm + L, 0, sizeof(float), st) != cudaSuccess) return LANTERN_ERR_CUDA;
-    knn_norms_kernel<<<(L * 32 + 255) / 256, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(codebook), L, d, nrm);
-    if (cudaGetLastError() != cudaSuccess) return LANTERN_ERR_CUDA;
-    if (use_t5_path(dt, L, d, k)) {
-      KnnT5Args fa;
-      fa.cb = static_cast<const __nv_bfloat16*>(codebook); fa.nrm = nrm; fa.L = L; fa.d = d; fa.k = k;
-      fa.CAP = knn_t5_cap(k);
-      fa.lists = reinterpret_cast<unsigned long long*>(static_cast<unsigned char*>(workspace) + norms_bytes(L));
-      fa.nbr_idx = nbr_idx; fa.nbr_dist = nbr_dist;
-      int dev = 0, sms = 0;
-      if (cudaGetDevice(&dev) != cudaSuccess ||
-          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
-        return LANTERN_ERR_CUDA;
-      const long long afford = static_cast<long long>((workspace_bytes - norms_bytes(L)) / t5_cta_bytes(k));
-      // tiles of 128 queries, or of 64 (half of the tensor-memory lanes idle: the contraction is a small part
-      // of the kernel) when that is what it takes to give every SM a tile
-      fa.qtile = (L + kT5Q - 1) / kT5Q * 2 <= sms ? kT5Q / 2 : kT5Q;
-      int grid = (L + fa.qtile - 1) / fa.qtile;
-      if (grid > sms) grid = sms;
-      if (grid > afford) grid = static_cast<int>(afford);
-      if (grid < 1) return LANTERN_ERR_WORKSPACE;
-      const size_t fsm = knn_t5_smem(d, fa.CAP);
-      if (cudaFuncSetAttribute(knn_t5_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(fsm)) != cudaSuccess)
-        return LANTERN_ERR_CUDA;
-      knn_t5_kernel<<<grid, kT5Threads, fsm, st>>>(fa);
-      return cudaGetLastError() == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
+  const T5Plan p = t5_plan(dt, L, d, k);
+  if (p.ok) {
+    const bool have = workspace && workspace_bytes >= p.bytes && reinterpret_cast<uintptr_t>(workspace) % 256 == 0;
+    const bool aligned = reinterpret_cast<uintptr_t>(codebook) % 16 == 0;
+    if (needs_workspace(dt, L, d, k)) {
+      if (!have) return LANTERN_ERR_WORKSPACE;
+      if (!aligned) return LANTERN_ERR_INVALID_ARG;
     }
-    KnnTcArgs ta;
-    ta.cb = static_cast<const __nv_bfloat16*>(codebook); ta.nrm = nrm; ta.L = L; ta.d = d; ta.k = k;
-    ta.CAP = 256;
-    while (ta.CAP < k + 192) ta.CAP *= 2;
-    ta.nbr_idx = nbr_idx; ta.nbr_dist = nbr_dist;
-    const int ld = d + kTcPad;
-    const size_t tsm = static_cast<size_t>(kTcQT) * ta.CAP * 8 + static_cast<size_t>(kTcQT) * ld * 2 +
-                       static_cast<size_t>(2) * kTcCT * ld * 2 + 2 * kTcCT * 4 + 5 * kTcQT * 4 + 64 +
-                       260 * 4 + static_cast<size_t>(ta.CAP) * 8;
-    if (cudaFuncSetAttribute(knn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(tsm)) != cudaSuccess)
-      return LANTERN_ERR_CUDA;
-    knn_tc_kernel<<<(L + kTcQT - 1) / kTcQT, kKnnThreads, tsm, st>>>(ta);
-    return cudaGetLastError() == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
+    if (have) {
+      unsigned char* ws = static_cast<unsigned char*>(workspace);
+      return dt == LANTERN_F32 ? build_t5(p, static_cast<const float*>(codebook), L, d, k, nbr_idx, nbr_dist, ws, st)
+                               : build_t5(p, static_cast<const __nv_bfloat16*>(codebook), L, d, k, nbr_idx, nbr_dist, ws, st);
+    }
   }
   KnnArgs a;
   a.cb = codebook; a.L = L; a.d = d; a.k = k; a.nbr_idx = nbr_idx; a.nbr_dist = nbr_dist;

@@ -1,76 +1,98 @@
 // Blackwell tensor path of the latent-neighbour table (Sec. 2.2 / Sec. 4: B_k; App. A.1: the
-// codebook) for bfloat16 codebooks with d a multiple of 8 in [8, 256]: the distance contraction on
-// the fifth-generation tensor cores (tcgen05.mma, bf16 x bf16 -> float32 accumulators in tensor
-// memory), the selection fused behind it.  Rows are zero-padded in shared memory to a multiple of
-// 16 elements (the K extent of one MMA), which changes no inner product.
+// codebook): the distance contraction on the fifth-generation tensor cores (tcgen05.mma, bf16 x bf16
+// -> float32 accumulators in tensor memory) only selects candidates; the table is exact.
 //
-//   approximate distance  f(i,j) = |c_i|^2 + |c_j|^2 - 2 <c_i, c_j>   (float32),  |f - D| <= eps_i
-// as in knn_tc.cuh; a query keeps every candidate with f <= tau + 2 eps (tau: an upper bound of the
-// k-th smallest f at its last cut-back), so no true neighbour is ever dropped, and ranks the
-// survivors exactly (double precision, ties by index) at the end.  f is formed as
-// fl(g + |c_i|^2), g = fl(|c_j|^2 - 2 <c_i, c_j>): the same two roundings as in knn_tc.cuh.
+//   approximate distance  f(i,j) = |c_i|^2 + g(i,j),  g(i,j) = |c_j|^2 - 2 <c_i, c_j>   (float32)
+//   |f - D| <= eps_i for the exact squared distance D, eps_i = ((d+16) 2^-21 [+ 2^-16]) (|c_i|^2 + max_j |c_j|^2)
+// (accumulation of the products, the two norms, the final roundings, with a factor of slack).  Rows
+// are zero-padded to a multiple of 16 elements (the K extent of one MMA), which changes no inner
+// product.  Float32 rows enter as two bfloat16 halves h + l of every element: the query side is laid
+// out as [h l h], the candidate side as [h h l], so one contraction of length 3 d gives
+// hh + lh + hl; what is missing is below 3 * 2^-18 (1 + 2^-7) |x| |y| per product, which is the 2^-16 term above.
 //
-// One persistent CTA of 256 threads per SM; a CTA takes tiles of 128 queries (tensor-memory lane =
-// query) and streams all rows past them in tiles of 128 candidates (tensor-memory column =
-// candidate):
-//   warps 5-7  load operand tiles with 16-byte cp.async into the K-major core-matrix layout the
-//              tensor core reads without swizzling (a core matrix = 8 rows x 16 bytes, contiguous),
-//              two candidate stages in flight;
-//   warp 4     one thread issues d/16 tcgen05.mma per tile into one of two 128-column accumulators
-//              and commits to the mbarriers that free the stage and publish the accumulator;
-//   warps 0-3  thread t owns query t: it reads its lane of the accumulator with tcgen05.ld, forms f,
-//              and appends the few candidates under its threshold to its own list in global memory
-//              (no atomics); a list that fills up is cut back by its warp (radix select on a copy in
-//              shared memory), so the four warps never wait for one another.
-// After the last candidate tile the eight warps rank the 128 queries exactly, one query per warp at
-// a time.  Every wait on an mbarrier is bounded; a wait that runs out raises an abort flag that all
-// roles poll, the CTA frees its tensor memory and returns, and the rows it had not finished are
-// written as -1.
+// Four kernels per chunk of query tiles (a tile = 128 queries = tensor-memory lanes):
+//   knn_t5_kernel<true>    every sampled candidate (one in four, evenly spread): smallest g of every
+//                          group of G columns per query, one FMA and one minimum per distance.
+//   knn_bound_kernel, knn_t5_kernel<false>
+//                          the (k+1)-th smallest of a query's group minima bounds its (k+1)-th
+//                          smallest g (the query itself may be among them) whatever the data, so
+//                          everything with g <= that + 2 eps is a superset of the neighbours; those
+//                          entries are appended to the query's lists, about 4.4 k of them when the
+//                          sample is representative.  A list that would overflow all the same is cut
+//                          back by its warp.
+//   knn_rank_kernel        one CTA per query: cuts the lists down to the k-th smallest g + 2 eps and
+//                          ranks the survivors by (exact distance in double precision, index).
+// Measured on 65536 x 256, k = 200 (5.5 ms; one kernel that streamed from an open threshold, cut lists back
+// and ranked behind the contraction took 19.7): per chunk of 18944 queries 0.22 ms sample pass, 0.06 ms bounds,
+// 0.75 ms contraction, 0.64 ms ranking; the tensor rate alone would be 0.39 ms per chunk.  The contraction's
+// kernel is bound by the issue slots of its selection (nine instructions per distance, 61 % of the slots busy),
+// the ranking by issue slots too (widening, double-precision differences, sort).  8192 x 256: 0.42 ms, was 1.59.
+// Ranking wants many warps in flight (scattered row reads, long-latency double-precision chains), which is
+// why it is a kernel of its own.
+//
+// knn_t5_kernel: one CTA of 320 threads per (query tile, share of the candidates), candidates in
+// tiles of 128 (tensor-memory columns):
+//   warp 9     one thread copies operand tiles with cp.async.bulk, two candidate stages in flight: knn_prep_kernel has
+//              laid the codebook out once in the K-major core-matrix order the tensor core reads without
+//              swizzling (a core matrix = 8 rows x 16 bytes, contiguous), so a tile is one run of bytes;
+//   warp 8     one thread issues the MMAs of a tile into one of two 128-column accumulators and
+//              commits to the mbarriers that free the stage and publish the accumulator;
+//   warps 0-7  two threads per query, 64 columns each (four threads with 32 each: 5.79 ms instead of 5.54 on
+//              65536 x 256, k = 200), read their lane of the accumulator with
+//              tcgen05.ld and take minima, or append to a list of their own in global memory (no atomics).
+// Every wait on an mbarrier is bounded; a wait that runs out raises an abort flag that all roles poll,
+// the CTA frees its tensor memory and returns, and the rows of its queries are written as -1.
 #pragma once
 
-#include "knn_tc.cuh"
+#include <float.h>
+
+#include "common.cuh"
 
 namespace lantern {
 
-constexpr int kT5Q = 128;           // queries per CTA tile (tensor-memory lanes)
+constexpr int kT5Q = 128;           // queries per tile (tensor-memory lanes)
 constexpr int kT5C = 128;           // candidates per tile (tensor-memory columns per accumulator)
-constexpr int kT5Stages = 2;        // candidate tiles in flight in shared memory
-constexpr int kT5Threads = 256;
-constexpr int kT5Loaders = 96;      // warps 5-7
+constexpr int kT5Per = 2;           // threads per query in the selection
+constexpr int kT5Cols = kT5C / kT5Per;               // columns of a tile each of them looks at
+constexpr int kT5Sel = kT5Per * kT5Q;                // selection threads
+constexpr int kT5Mma = kT5Sel / 32;                  // the warp that issues the MMAs; the next one loads
+constexpr int kT5Threads = kT5Sel + 64;
 constexpr int kT5Sort = 512;        // exact ranking: candidates per query (power of two)
 constexpr int kT5MaxK = 320;
+constexpr int kT5Items = 148;       // CTAs per chunk (one per SM)
+constexpr int kT5MaxSplit = 8;      // shares of the candidates
+constexpr int kT5MaxGroups = 1024;  // group minima per query
+constexpr float kT5Huge = 1e37f;    // rows with a squared norm from here on never enter the contraction's bounds
 
 struct KnnT5Args {
-  const __nv_bfloat16* cb;
-  const float* nrm;                 // [L] squared norms, nrm[L] = their maximum
-  unsigned long long* lists;        // [gridDim.x][kT5Q][CAP] candidate lists (key << 32 | index)
-  int L, d, k, CAP;
-  int qtile;                        // queries a CTA tile really holds: 128, or 64 (the other lanes idle) when 128 would leave SMs without a tile
-  int32_t* nbr_idx;
-  float* nbr_dist;
+  // operand tiles of 128 rows in the layout the tensor core reads, [dpad/8 chunks][16 row groups][8 rows][16 bytes]:
+  const unsigned char *qm, *cm;     // query side, and candidate side (the sampled rows in the sample pass)
+  const float* cn;                  // squared norms of the candidate side's rows, +inf for rows that are none
+  const float* nrm;                 // [L] squared norms, nrm[L] = the largest below kT5Huge
+  float* minima;                    // [tiles][kT5Q][groups] (sample pass)
+  const float* bound;               // [tiles][kT5Q] knn_bound_kernel's result
+  unsigned long long* lists;        // [tiles][split][kT5Per][kT5Q][cap]: (bits of g) << 32 | index
+  int* counts;                      // [tiles][split][kT5Per][kT5Q] entries; -1: overflow, -9: a wait ran out
+  int L, dp, k, cap;                // dp: elements per operand row (a multiple of 16)
+  int tile0;                        // first query tile of the chunk
+  int split;                        // CTAs per query tile
+  int nct;                          // candidate tiles of this pass
+  int gshift;                       // log2 of the columns per group minimum (0 .. 5)
+  int groups;                       // group minima per query
+  float eps1;                       // eps_i = eps1 (|c_i|^2 + max) + eps0
+  float eps0;
 };
 
-// list capacity: room for one tile of appends above the cut-back level, which itself leaves the
-// larger of k and 192 entries of slack above k
-__host__ __device__ constexpr int knn_t5_dpad(int d) { return (d + 15) / 16 * 16; }     // K extent in shared memory
-__host__ __device__ constexpr int knn_t5_cap(int k) { return (k + kT5C + (k > 192 ? k : 192) + 63) / 64 * 64; }
-
-// bytes of one warp's slot in the final ranking: staged list, histogram, (distance, index) pairs,
-// the query row in double precision
-__host__ __device__ constexpr size_t knn_t5_slot(int cap, int d) {
-  return static_cast<size_t>(cap) * 8 + 256 * 4 + static_cast<size_t>(kT5Sort) * 12 + static_cast<size_t>(d) * 8;
-}
-// the candidate stages and the final ranking share one region
-__host__ __device__ constexpr size_t knn_t5_region(int d, int cap) {
-  const size_t stages = static_cast<size_t>(kT5Stages) * kT5C * knn_t5_dpad(d) * 2, rank = 8 * knn_t5_slot(cap, d);
-  return stages > rank ? stages : rank;
-}
-__host__ __device__ constexpr size_t knn_t5_smem(int d, int cap) {
-  return static_cast<size_t>(kT5Q) * knn_t5_dpad(d) * 2 + knn_t5_region(d, cap)   // query tile; stages / ranking
+__host__ __device__ constexpr size_t knn_t5_smem(int dp) {
+  return static_cast<size_t>(3) * kT5Q * dp * 2                       // query tile, two candidate stages
          + 4 * kT5C * 4                                               // candidate norms, 4 tiles deep
-         + kT5Q * 4 * 2                                               // 2 eps, list counts
-         + 4 * static_cast<size_t>(cap) * 8 + 4 * 256 * 4             // per-warp staging and histogram of a cut
-         + 16 * 8 + 8 * 8 + 24 * 4;                                   // mbarriers, arg-min scratch, misc
+         + kT5Mma * 256 * 4                                           // per-warp histogram of a cut
+         + 16 * 8 + 16;                                               // mbarriers, misc
+}
+
+// slack for the roundings between the thresholds and g: everything the bound has to cover, in g
+__device__ __forceinline__ float t5_margin(const KnnT5Args& a, float nq, float nmax) {
+  return 2.f * fmaf(a.eps1, nq + nmax, a.eps0);
 }
 
 __device__ __forceinline__ uint64_t t5_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
@@ -81,16 +103,14 @@ __device__ __forceinline__ uint64_t t5_desc(uint32_t saddr, uint32_t lbo_bytes, 
 }
 
 // bounded wait of one thread on an mbarrier phase that also gives up when another role has raised
-// `abort`: non-blocking polls (test_wait) with a short sleep between them, so the bound is about a
-// second and a waiting thread leaves the shared-memory pipe to the working warps
+// `abort`: the hardware suspends the thread for at most a microsecond per try, so the bound is about a second
 __device__ __forceinline__ bool t5_wait(uint32_t mbar, uint32_t parity, volatile int* abort) {
-  for (int it = 0; it < (1 << 24); ++it) {
+  for (int it = 0; it < (1 << 20); ++it) {
     uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(mbar), "r"(parity) : "memory");
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(mbar), "r"(parity), "r"(1000u) : "memory");
     if (ok) return true;
-    if (it >= 4) __nanosleep(40);
-    if ((it & 1023) == 1023 && *abort) return false;
+    if ((it & 255) == 255 && *abort) return false;
   }
   *abort = 1;
   return false;
@@ -105,73 +125,47 @@ __device__ __forceinline__ void t5_arrive(uint32_t mbar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
 }
 
-// One operand tile (rows [row0, row0 + 128) of the codebook, zero beyond L and beyond d) into the
-// core-matrix layout [dpad/8 chunks][16 row groups][8 rows][16 bytes].  A warp step covers 8 rows x 4 chunks: the
-// 8 rows of a chunk are one contiguous core matrix (conflict-free), each row reads 64 contiguous
-// bytes.  A warp walks along the rows of its row groups, so addresses advance by additions only.
-__device__ __forceinline__ void t5_load_tile(const __nv_bfloat16* __restrict__ cb, int L, int d, int row0,
-                                             unsigned char* dst, int ltid) {      // L: rows at or beyond it read as zero
-  const int lane = ltid & 31, lw = ltid >> 5;
-  const int r = lane & 7, c = lane >> 3;                          // row in the group, chunk in the quad
-  const int nch = d >> 3, pch = knn_t5_dpad(d) >> 3;               // 16-byte chunks per row: real, padded
-  for (int rg = lw; rg < 16; rg += kT5Loaders / 32) {
-    const int grow = row0 + rg * 8 + r;
-    const bool in = grow < L;
-    const __nv_bfloat16* src = cb + static_cast<long long>(in ? grow : 0) * d + c * 8;
-    uint32_t sdst = smem_u32(dst) + static_cast<uint32_t>((c * 16 + rg) * 128 + r * 16);
-    for (int kc = c; kc < pch; kc += 4) {
-      const bool real = in && kc < nch;
-      cp_async16(sdst, real ? src : cb, real ? 16u : 0u);
-      src += 32;
-      sdst += 4u * 16u * 128u;
-    }
+// `bytes` (a multiple of 16) from global to shared memory by bulk copies that complete on `mbar`, which must
+// already expect them; pieces of 8 KB, so that one tile is spread over several copy requests.
+__device__ __forceinline__ void t5_bulk(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
+  const unsigned char* g = static_cast<const unsigned char*>(src);
+  for (uint32_t o = 0; o < bytes; o += 8192u) {
+    const uint32_t n = min(8192u, bytes - o);
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst + o), "l"(g + o), "r"(n), "r"(mbar) : "memory");
   }
 }
+__device__ __forceinline__ void t5_expect(uint32_t mbar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+}
 
-// Cut-back of one list by one warp (the radix select of knn.cu on warp scale).  Lists in global
-// memory hold (float bits of f) << 32 | index.  The n entries of `src` are copied to `st` (shared
-// memory) with f turned into its monotone 32-bit key.  An upper bound of the k-th smallest key is
-// then found by histogram passes of up to 8 bits over key - min, starting at the highest bit in
-// which the keys differ (distances of one list share their leading bits: passes over those would
-// put every entry into one bin).  The passes stop when the bin that holds the k-th key has at most
-// SLACK entries (or bit 0 is reached); the bound is the upper edge of that bin, so at most SLACK
-// entries more than with the exact k-th key get through, which keeps the superset property.  The
-// entries whose key is at most limit_of(bound) are written to `dst` in their old order: back to
-// `src` as float bits (TO_RAW), or to `st` as keys.  Returns the number kept.  n >= k >= 1.
-template <bool TO_RAW, int SLACK, typename F>
-__device__ __forceinline__ int t5_warp_cut(const unsigned long long* src, int n, int k, unsigned long long* st,
-                                           uint32_t* hist, unsigned long long* dst, F&& limit_of, uint32_t* limit_out) {
+__device__ __forceinline__ void t5_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+               "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                 "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                 "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                 "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+               : "r"(taddr) : "memory");
+}
+
+// Digit passes shared by the cuts: narrows (k-th smallest key - kmin) from bit `hi` down by histograms of
+// up to 8 bits until its bin holds at most `slack` keys.  count(lo, mask, hi, prefix) fills hist[256]
+// (zeroed here); every warp of the caller evaluates the same histogram.  Returns an upper bound of the
+// k-th smallest key (the upper edge of its bin, at most kmax).
+template <typename SYNC, typename COUNT>
+__device__ __forceinline__ uint32_t t5_digit_select(uint32_t kmin, uint32_t kmax, int k, int slack, uint32_t* hist, int tid, int nt,
+                                                    SYNC&& sync, COUNT&& count) {
   const int lane = threadIdx.x & 31;
-  __syncwarp();                                               // the owner's appends are visible to the warp
-  uint32_t kmin = 0xffffffffu, kmax = 0u;
-#pragma unroll 8
-  for (int i = lane; i < n; i += 32) {
-    const unsigned long long e = src[i];
-    const uint32_t key = float_key(__uint_as_float(static_cast<uint32_t>(e >> 32)));
-    st[i] = (static_cast<unsigned long long>(key) << 32) | (e & 0xffffffffull);
-    kmin = min(kmin, key);
-    kmax = max(kmax, key);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    kmin = min(kmin, __shfl_xor_sync(0xffffffffu, kmin, o));
-    kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, o));
-  }
   int hi = 32 - __clz(kmax - kmin);                           // key - kmin < 2^hi
   uint32_t prefix = 0;                                        // (k-th key - kmin) >> hi, known so far
-  int rem = k;
+  uint32_t rem = static_cast<uint32_t>(k);
   while (hi > 0) {
     const int lo = hi > 8 ? hi - 8 : 0;
-    const uint32_t mask = (1u << (hi - lo)) - 1u;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) hist[lane + 32 * i] = 0;
-    __syncwarp();
-#pragma unroll 4
-    for (int i = lane; i < n; i += 32) {
-      const uint32_t rel = static_cast<uint32_t>(st[i] >> 32) - kmin;
-      if (hi == 32 || (rel >> hi) == prefix) atomicAdd(&hist[(rel >> lo) & mask], 1u);
-    }
-    __syncwarp();
+    for (int i = tid; i < 256; i += nt) hist[i] = 0;
+    sync();
+    count(lo, (1u << (hi - lo)) - 1u, hi, prefix);
+    sync();
     uint32_t c8[8], sum = 0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) { c8[i] = hist[lane * 8 + i]; sum += c8[i]; }
@@ -181,14 +175,14 @@ __device__ __forceinline__ int t5_warp_cut(const unsigned long long* src, int n,
       const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += t;
     }
-    const uint32_t before = incl - sum, want = static_cast<uint32_t>(rem);
-    const bool mine = before < want && want <= incl;          // exactly one lane
-    int bin = 0, nrem = 0, pop = 0;
+    const uint32_t before = incl - sum;
+    const bool mine = before < rem && rem <= incl;            // exactly one lane
+    uint32_t bin = 0, nrem = 0, pop = 0;
     if (mine) {
       uint32_t run = before;
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        if (run < want && want <= run + c8[i]) { bin = lane * 8 + i; nrem = static_cast<int>(want - run); pop = static_cast<int>(c8[i]); }
+        if (run < rem && rem <= run + c8[i]) { bin = lane * 8 + i; nrem = rem - run; pop = c8[i]; }
         run += c8[i];
       }
     }
@@ -196,24 +190,48 @@ __device__ __forceinline__ int t5_warp_cut(const unsigned long long* src, int n,
     bin = __shfl_sync(0xffffffffu, bin, owner);
     rem = __shfl_sync(0xffffffffu, nrem, owner);
     pop = __shfl_sync(0xffffffffu, pop, owner);
-    prefix = (prefix << (hi - lo)) | static_cast<uint32_t>(bin);
+    prefix = (prefix << (hi - lo)) | bin;
     hi = lo;
-    __syncwarp();
-    if (pop <= SLACK) break;
+    sync();
+    if (pop <= static_cast<uint32_t>(slack)) break;
   }
   // keys whose (key - kmin) >> hi equals prefix: the k-th smallest is among them
   const unsigned long long edge = static_cast<unsigned long long>(kmin) + ((static_cast<unsigned long long>(prefix) + 1ull) << hi) - 1ull;
-  const uint32_t limit = limit_of(edge < kmax ? static_cast<uint32_t>(edge) : kmax);
+  return edge < kmax ? static_cast<uint32_t>(edge) : kmax;
+}
+
+__device__ __forceinline__ uint32_t t5_entry_key(unsigned long long e) { return float_key(__uint_as_float(static_cast<uint32_t>(e >> 32))); }
+
+// Cut-back of one list of n > k entries by one warp, in place and in order: everything up to an upper
+// bound of the k-th smallest g plus `margin` stays.  Returns the number kept; *limit_out is the bound in g.
+__device__ __forceinline__ int t5_warp_cut(unsigned long long* lst, int n, int k, float margin, uint32_t* hist, float* limit_out) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();                                               // the owner's appends are visible to the warp
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll 4
+  for (int i = lane; i < n; i += 32) {
+    const uint32_t key = t5_entry_key(lst[i]);
+    kmin = min(kmin, key);
+    kmax = max(kmax, key);
+  }
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  const uint32_t kth = t5_digit_select(kmin, kmax, k, 32, hist, lane, 32, [] { __syncwarp(); },
+                                       [&](int lo, uint32_t mask, int hi, uint32_t prefix) {
+#pragma unroll 4
+    for (int i = lane; i < n; i += 32) {
+      const uint32_t rel = t5_entry_key(lst[i]) - kmin;
+      if (hi == 32 || (rel >> hi) == prefix) atomicAdd(&hist[(rel >> lo) & mask], 1u);
+    }
+  });
+  const float limit = __fadd_ru(key_float(kth), margin);
   int pos = 0;
   for (int i0 = 0; i0 < n; i0 += 32) {
     const int i = i0 + lane;
-    const unsigned long long e = i < n ? st[i] : ~0ull;
-    const bool keep = i < n && static_cast<uint32_t>(e >> 32) <= limit;
+    const unsigned long long e = i < n ? lst[i] : 0ull;
+    const bool keep = i < n && __uint_as_float(static_cast<uint32_t>(e >> 32)) <= limit;
     const uint32_t m = __ballot_sync(0xffffffffu, keep);      // every lane has read its entry before slots <= i are rewritten
-    if (keep)
-      dst[pos + __popc(m & ((1u << lane) - 1u))] =
-          TO_RAW ? (static_cast<unsigned long long>(__float_as_uint(key_float(static_cast<uint32_t>(e >> 32)))) << 32) | (e & 0xffffffffull)
-                 : e;
+    if (keep) lst[pos + __popc(m & ((1u << lane) - 1u))] = e;
     pos += __popc(m);
     __syncwarp();
   }
@@ -221,122 +239,73 @@ __device__ __forceinline__ int t5_warp_cut(const unsigned long long* src, int n,
   return pos;
 }
 
-// bfloat16 (low 16 bits of b16) to double without the conversion unit: for normal numbers the double's
-// high word is the sign, the exponent rebiased by 1023 - 127 and the 7 mantissa bits, all by integer
-// operations; zeros, subnormals, infinities and NaNs take the converting instruction.  Exact either way.
-__device__ __forceinline__ double t5_bf16_to_double(uint32_t b16) {
-  if (((b16 >> 7) & 0xffu) - 1u < 254u)
-    return __hiloint2double(static_cast<int>(((b16 & 0x8000u) << 16) | (((b16 & 0x7fffu) << 13) + (896u << 20))), 0);
-  return static_cast<double>(__uint_as_float(b16 << 16));
-}
-
-// Exact squared distances between the query row `qd` (doubles in shared memory) and the candidates
-// st[base + 32 u + lane], u < kT5Chains, each the sum of exact_dist_bf16x8 term by term in the same
-// order.  A double-precision FMA has a long latency and each sum is one dependent chain, so a lane
-// runs the chains of its candidates side by side.  Entries in [n, p2) are padded with +inf.
-constexpr int kT5Chains = 7;
-__device__ __forceinline__ void t5_exact_block(const double* qd, const __nv_bfloat16* __restrict__ cb, int d,
-                                               const unsigned long long* st, int n, int p2, int base, int nch,
-                                               unsigned long long* sortd, int* sorti) {
-  const int lane = threadIdx.x & 31;
-  // this call covers entries [base, base + 32 nch); nu of its chains hold at least one candidate
-  const int nu = min(nch, (min(n, p2) - base + 31) / 32);
-  const __nv_bfloat16* row[kT5Chains];
-  int idx[kT5Chains];
-  double acc[kT5Chains];
+// Upper bound (the edge of a bin of a few) of the (k+1)-th smallest group minimum of every query of the chunk,
+// one warp per query; FLT_MAX when fewer are finite.  A kernel of its own: inside the contraction's CTAs, two
+// warps per scheduler, the selection took as long as 60 candidate tiles.
+__global__ void __launch_bounds__(256) knn_bound_kernel(const float* __restrict__ minima, int queries, int groups, int want, float* __restrict__ bound) {
+  __shared__ uint32_t hist_s[8][256];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = blockIdx.x * 8 + warp;
+  if (q >= queries) return;
+  const float* src = minima + static_cast<size_t>(q) * groups;
+  uint32_t* hist = hist_s[warp];
+  uint32_t key[kT5MaxGroups / 32];
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+  const uint32_t top = float_key(FLT_MAX);
+  int finite = 0;
 #pragma unroll
-  for (int u = 0; u < kT5Chains; ++u) {
-    const int i = base + 32 * u + lane;
-    idx[u] = (u < nch && i < n) ? static_cast<int>(st[i] & 0xffffffffu) : -1;
-    row[u] = cb + static_cast<long long>(idx[u] < 0 ? 0 : idx[u]) * d;
-    acc[u] = 0.0;
+  for (int i = 0; i < kT5MaxGroups / 32; ++i) {
+    const int m = i * 32 + lane;
+    key[i] = m < groups ? float_key(__ldg(src + m)) : 0xffffffffu;
+    kmin = min(kmin, key[i]);
+    if (key[i] <= top) { kmax = max(kmax, key[i]); ++finite; }
   }
-  for (int t = 0; t < d; t += 8) {
-    uint4 bv[kT5Chains];
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  finite = __reduce_add_sync(0xffffffffu, finite);
+  float v = FLT_MAX;
+  if (finite >= want) {
+    const uint32_t kth = t5_digit_select(kmin, kmax, want, 8, hist, lane, 32, [] { __syncwarp(); },
+                                         [&](int lo, uint32_t mask, int hi, uint32_t prefix) {
 #pragma unroll
-    for (int u = 0; u < kT5Chains; ++u)
-      if (u < nu) bv[u] = __ldg(reinterpret_cast<const uint4*>(row[u] + t));
-    double q[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) q[i] = qd[t + i];
-#pragma unroll
-    for (int u = 0; u < kT5Chains; ++u) {
-      if (u < nu) {
-        const uint32_t bw[4] = {bv[u].x, bv[u].y, bv[u].z, bv[u].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const double d0 = q[2 * i] - t5_bf16_to_double(bw[i] & 0xffffu);
-          acc[u] = fma(d0, d0, acc[u]);
-          const double d1 = q[2 * i + 1] - t5_bf16_to_double(bw[i] >> 16);
-          acc[u] = fma(d1, d1, acc[u]);
-        }
+      for (int i = 0; i < kT5MaxGroups / 32; ++i) {
+        const uint32_t rel = key[i] - kmin;
+        if (key[i] <= top && (hi == 32 || (rel >> hi) == prefix)) atomicAdd(&hist[(rel >> lo) & mask], 1u);
       }
-    }
+    });
+    v = key_float(kth);
   }
-#pragma unroll
-  for (int u = 0; u < kT5Chains; ++u) {
-    const int i = base + 32 * u + lane;
-    if (u < nch && i < p2) {
-      sorti[i] = idx[u] < 0 ? 0x7fffffff : idx[u];
-      sortd[i] = idx[u] < 0 ? 0x7ff0000000000000ull : static_cast<unsigned long long>(__double_as_longlong(acc[u]));
-    }
-  }
+  if (lane == 0) bound[q] = v;
 }
 
-// ascending bitonic sort of n (power of two) (distance, index) pairs by one warp.  Distances are
-// non-negative doubles (or +inf padding), whose bit patterns order like their values: the compares
-// run on the integer pipe.
-__device__ __forceinline__ void t5_warp_sort(unsigned long long* dv, int* iv, int n) {
-  const int lane = threadIdx.x & 31;
-  for (int size = 2; size <= n; size <<= 1) {
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-#pragma unroll 4
-      for (int i = lane; i < (n >> 1); i += 32) {
-        const int lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
-        const bool up = (lo & size) == 0;
-        const unsigned long long dx = dv[lo], dy = dv[hi];
-        const int ix = iv[lo], iy = iv[hi];
-        const bool gt = dx > dy || (dx == dy && ix > iy);
-        if (gt == up) { dv[lo] = dy; dv[hi] = dx; iv[lo] = iy; iv[hi] = ix; }
-      }
-      __syncwarp();
-    }
-  }
-}
-
+template <bool SAMPLE>
 __global__ void __launch_bounds__(kT5Threads, 1) knn_t5_kernel(const KnnT5Args a) {
   extern __shared__ __align__(128) unsigned char t5_smem[];
-  const int d = a.d, L = a.L, k = a.k, CAP = a.CAP, dp = knn_t5_dpad(a.d);
-  const __nv_bfloat16* cb = a.cb;
+  const int L = a.L, dp = a.dp;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  unsigned char* As = t5_smem;                                        // [d/8][16][8][16 B]
-  unsigned char* Bs = As + static_cast<size_t>(kT5Q) * dp * 2;         // [stages][d/8][16][8][16 B] | ranking slots
   const size_t tile_bytes = static_cast<size_t>(kT5C) * dp * 2;
-  float* ncs = reinterpret_cast<float*>(Bs + knn_t5_region(d, CAP));  // [4][kT5C] candidate norms
-  float* eps2s = ncs + 4 * kT5C;                                      // [kT5Q]
-  int* cnts = reinterpret_cast<int*>(eps2s + kT5Q);                   // [kT5Q] list lengths (-1: overflow, -2: exact fallback)
-  unsigned long long* cut_st = reinterpret_cast<unsigned long long*>(cnts + kT5Q);     // [4][CAP]
-  uint32_t* cut_hist = reinterpret_cast<uint32_t*>(cut_st + 4 * static_cast<size_t>(CAP));   // [4][256]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(cut_hist + 4 * 256);   // full[2] empty[2] tfull[2] tempty[2] afull aempty | redd[8]
-  int* misc = reinterpret_cast<int*>(bars + 24);                      // [0] tensor-memory base, [1] abort, [16..23] redi
+  unsigned char* As = t5_smem;                                        // [dp/8][16][8][16 B]
+  unsigned char* Bs = As + tile_bytes;                                // [2 stages][dp/8][16][8][16 B]
+  float* ncs = reinterpret_cast<float*>(Bs + 2 * tile_bytes);         // [4][kT5C] candidate norms
+  uint32_t* cut_hist = reinterpret_cast<uint32_t*>(ncs + 4 * kT5C);   // [kT5Mma][256]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(cut_hist + kT5Mma * 256);   // full[2] empty[2] tfull[2] tempty[2] afull
+  int* misc = reinterpret_cast<int*>(bars + 16);                      // [0] tensor-memory base, [1] abort, [3] the loading thread's last waits
 
   const uint32_t bar0 = smem_u32(bars);
   auto full = [&](uint32_t s2) { return bar0 + 8u * s2; };
   auto empty = [&](uint32_t s2) { return bar0 + 8u * (2 + s2); };
   auto tfull = [&](uint32_t b) { return bar0 + 8u * (4 + b); };
   auto tempty = [&](uint32_t b) { return bar0 + 8u * (6 + b); };
-  const uint32_t afull = bar0 + 8u * 8, aempty = bar0 + 8u * 9;
+  const uint32_t afull = bar0 + 8u * 8;
   volatile int* abort = misc + 1;
-
   if (tid == 0) {
     auto init = [&](uint32_t b, int count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(b), "r"(count) : "memory"); };
-    for (uint32_t s2 = 0; s2 < 2; ++s2) { init(full(s2), kT5Loaders); init(empty(s2), 1); init(tfull(s2), 1); init(tempty(s2), kT5Q); }
-    init(afull, kT5Loaders);
-    init(aempty, 1);
+    for (uint32_t s2 = 0; s2 < 2; ++s2) { init(full(s2), 1); init(empty(s2), 1); init(tfull(s2), 1); init(tempty(s2), kT5Sel); }
+    init(afull, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     misc[1] = 0;
+    misc[3] = 0;
   }
-  if (warp == 4) {
+  if (warp == kT5Mma) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(misc)), "r"(2 * kT5C) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -345,254 +314,439 @@ __global__ void __launch_bounds__(kT5Threads, 1) knn_t5_kernel(const KnnT5Args a
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tbase = static_cast<uint32_t>(misc[0]);
 
-  const int QT = a.qtile;
-  const int nqt = (L + QT - 1) / QT;                // query tiles
-  const int nct = (L + kT5C - 1) / kT5C;            // candidate tiles per query tile
+  // this CTA's query tile (within the chunk) and its share [t0, t1) of the candidate tiles
+  const int tile = blockIdx.x / a.split, part = blockIdx.x - tile * a.split;
+  const int q0 = (a.tile0 + tile) * kT5Q;
+  const int nct = a.nct;
+  const int t0 = static_cast<int>(static_cast<long long>(nct) * part / a.split);
+  const int t1 = static_cast<int>(static_cast<long long>(nct) * (part + 1) / a.split);
   const float nmax = a.nrm[L];
-  unsigned long long* my_lists = a.lists + static_cast<size_t>(blockIdx.x) * kT5Q * CAP;
-  bool dead = false;                                // a wait ran out (here or in another role): work is skipped, barriers are kept
-  uint32_t tiles_done = 0, qtiles_done = 0;         // per role: candidate tiles / query tiles handled so far
+  bool dead = false;                                // a wait ran out (here or in another role): work is skipped
 
-  for (int qt = blockIdx.x; qt < nqt; qt += gridDim.x) {
-    const int q0 = qt * QT;
-    if (warp >= 5) {
-      // ---------------------------------------------------------------- loaders (warps 5-7)
-      const int ltid = tid - 160;
-      uint32_t pending;                              // barrier of the copy group committed last
-      if (!dead) dead = !t5_wait_warp(aempty, (qtiles_done & 1u) ^ 1u, abort);
-      if (!dead) t5_load_tile(cb, min(L, q0 + QT), d, q0, As, ltid);
-      cp_async_commit();
-      pending = afull;
-      for (int t = 0; t < nct; ++t) {
-        const uint32_t s2 = tiles_done & 1u;
-        if (!dead) dead = !t5_wait_warp(empty(s2), ((tiles_done >> 1) & 1u) ^ 1u, abort);
-        if (!dead) {
-          t5_load_tile(cb, L, d, t * kT5C, Bs + s2 * tile_bytes, ltid);
-          for (int i = ltid; i < kT5C; i += kT5Loaders) {
-            const int j = t * kT5C + i;
-            const bool in = j < L;
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(ncs + (tiles_done & 3u) * kT5C + i)),
-                         "l"(a.nrm + (in ? j : 0)), "r"(in ? 4u : 0u) : "memory");
-          }
-        }
-        cp_async_commit();
-        cp_async_wait<1>();                          // the group committed before this one has landed: publish it
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        t5_arrive(pending);
-        pending = full(s2);
-        ++tiles_done;
+  if (warp == kT5Mma + 1) {
+    // ---------------------------------------------------------------- loads (one thread)
+    if (lane == 0) {
+      const uint32_t tb = static_cast<uint32_t>(tile_bytes);
+      t5_expect(afull, tb);
+      t5_bulk(smem_u32(As), a.qm + static_cast<size_t>(a.tile0 + tile) * tile_bytes, tb, afull);
+      uint32_t n = 0;
+      for (int t = t0; t < t1; ++t, ++n) {
+        const uint32_t s2 = n & 1u;
+        if (!t5_wait(empty(s2), ((n >> 1) & 1u) ^ 1u, abort)) break;
+        t5_expect(full(s2), tb + kT5C * 4u);
+        t5_bulk(smem_u32(Bs + s2 * tile_bytes), a.cm + static_cast<size_t>(t) * tile_bytes, tb, full(s2));
+        t5_bulk(smem_u32(ncs + (n & 3u) * kT5C), a.cn + static_cast<size_t>(t) * kT5C, kT5C * 4u, full(s2));
       }
-      cp_async_wait<0>();
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      t5_arrive(pending);
-      ++qtiles_done;
-    } else if (warp == 4) {
-      // ---------------------------------------------------------------- tensor-core issue (one thread)
-      if (lane == 0) {
-        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(kT5C >> 3) << 17) |
-                               (static_cast<uint32_t>(kT5Q >> 4) << 24);     // f32 += bf16 x bf16, K-major, N, M
-        const uint32_t lbo = 16u * 128u, sbo = 128u;
-        if (!dead) dead = !t5_wait(afull, qtiles_done & 1u, abort);
-        for (int t = 0; t < nct; ++t) {
-          const uint32_t s2 = tiles_done & 1u, par = (tiles_done >> 1) & 1u;
-          if (!dead) dead = !t5_wait(full(s2), par, abort);
-          if (!dead) dead = !t5_wait(tempty(s2), par ^ 1u, abort);
-          if (!dead) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs + s2 * tile_bytes);
-            for (int kk = 0; kk < dp / 16; ++kk) {
-              const uint64_t da = t5_desc(a0 + kk * 2u * lbo, lbo, sbo);
-              const uint64_t db = t5_desc(b0 + kk * 2u * lbo, lbo, sbo);
-              const uint32_t acc = kk > 0 ? 1u : 0u;
-              asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
-                           "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                           ::"r"(tbase + s2 * kT5C), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
-            }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty(s2)) : "memory");
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tfull(s2)) : "memory");
-          }
-          ++tiles_done;
-        }
-        if (!dead)
-          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(aempty) : "memory");
-        ++qtiles_done;
-      }
-    } else {
-      // ---------------------------------------------------------------- selection (warps 0-3): thread = query
-      const int qi = q0 + tid;
-      const bool active = qi < L && tid < QT;
-      const float nq = active ? a.nrm[qi] : 0.f;
-      const float e2 = 2.f * static_cast<float>(d + 8) * 4.76837158203125e-7f * (nq + nmax);     // 2 eps, 2^-21
-      eps2s[tid] = e2;
-      unsigned long long* lst = my_lists + static_cast<size_t>(tid) * CAP;
-      unsigned long long* st_w = cut_st + static_cast<size_t>(warp) * CAP;
-      uint32_t* hist_w = cut_hist + warp * 256;
-      // the filter compares g with thr_g >= thr - |q|^2, the slack covering the roundings of f = fl(g + |q|^2)
-      // and of the subtraction, so it passes a superset of {f <= thr}
-      float thr_g = INFINITY;
-      uint32_t woff = 0;                             // byte offset of the next free entry of the own list
-      int cnt = 0;
-      bool ovf = false;
-      for (int t = 0; t < nct; ++t) {
-        const uint32_t b = tiles_done & 1u;
-        const bool special = t == nct - 1 || t == q0 / kT5C;
-        if (!dead) dead = !t5_wait_warp(tfull(b), (tiles_done >> 1) & 1u, abort);   // warp-uniform
+      // the CTA may not leave while a copy is on its way into its shared memory
+      t5_wait(afull, 0u, abort + 2);
+      for (uint32_t back = 1; back <= 2 && back <= n; ++back) t5_wait(full((n - back) & 1u), ((n - back) >> 1) & 1u, abort + 2);
+    }
+  } else if (warp == kT5Mma) {
+    // ---------------------------------------------------------------- tensor-core issue (one thread)
+    if (lane == 0) {
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(kT5C >> 3) << 17) |
+                             (static_cast<uint32_t>(kT5Q >> 4) << 24);     // f32 += bf16 x bf16, K-major, N, M
+      const uint32_t lbo = 16u * 128u, sbo = 128u;
+      dead = !t5_wait(afull, 0u, abort);
+      for (int t = t0; t < t1; ++t) {
+        const uint32_t n = static_cast<uint32_t>(t - t0), s2 = n & 1u, par = (n >> 1) & 1u;
+        if (!dead) dead = !t5_wait(full(s2), par, abort);
+        if (!dead) dead = !t5_wait(tempty(s2), par ^ 1u, abort);
         if (!dead) {
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const float* nc = ncs + (tiles_done & 3u) * kT5C;
+          const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs + s2 * tile_bytes);
+          for (int kk = 0; kk < dp / 16; ++kk) {
+            const uint64_t da = t5_desc(a0 + kk * 2u * lbo, lbo, sbo);
+            const uint64_t db = t5_desc(b0 + kk * 2u * lbo, lbo, sbo);
+            const uint32_t acc = kk > 0 ? 1u : 0u;
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                         ::"r"(tbase + s2 * kT5C), "l"(da), "l"(db), "r"(idesc), "r"(acc) : "memory");
+          }
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(empty(s2)) : "memory");
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(tfull(s2)) : "memory");
+        }
+      }
+    }
+  } else {
+    // ---------------------------------------------------------------- selection (warps 0-7): two threads per query
+    const int q = (warp & 3) * 32 + lane, half = warp >> 2;
+    const int qi = q0 + q;
+    const float nq = qi < L ? a.nrm[qi] : 0.f;
+    const bool active = qi < L && nq < kT5Huge;      // (other rows are ranked without the contraction)
+    const float margin = t5_margin(a, nq, nmax);
+    float thr = __int_as_float(0x7fffffff);          // NaN: nothing passes (rows without a query)
+    if (!SAMPLE && active) thr = fminf(__fadd_ru(a.bound[tile * kT5Q + q], margin), FLT_MAX);
+    const size_t seg = static_cast<size_t>((tile * a.split + part) * kT5Per + half) * kT5Q + q;
+    float* mins = a.minima + (static_cast<size_t>(tile) * kT5Q + q) * a.groups;
+    uint32_t* hist_w = cut_hist + warp * 256;
+    const uint32_t base = static_cast<uint32_t>(seg * a.cap * 8);   // (the lists of a chunk take less than 4 GB)
+    uint32_t woff = base;                            // byte offset of the next free entry of the own list
+    bool ovf = false;
+    for (int t = t0; t < t1; ++t) {
+      const uint32_t n = static_cast<uint32_t>(t - t0), b = n & 1u;
+      if (!dead) dead = !t5_wait_warp(tfull(b), (n >> 1) & 1u, abort);   // warp-uniform
+      if (!dead) asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const float* nc = ncs + (n & 3u) * kT5C + half * kT5Cols;
 #pragma unroll 1
-          for (int c0 = 0; c0 < kT5C; c0 += 32) {
-            uint32_t r[32];
-            const uint32_t taddr = tbase + (static_cast<uint32_t>(warp * 32) << 16) + b * kT5C + c0;
-            asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                           "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                         : "r"(taddr) : "memory");
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (active && !ovf) {
-              const int cbase = t * kT5C + c0;
-              if (!special) {
-                // per candidate: one FMA, one compare, and a store and pointer step that are predicated
-                // in the instruction stream (a branch here would diverge on nearly every candidate
-                // while the thresholds are still loose)
+      for (int c0 = 0; c0 < kT5Cols; c0 += 32) {
+        uint32_t r[32];
+        if (!dead) {
+          t5_ld32(tbase + (static_cast<uint32_t>((warp & 3) * 32) << 16) + b * kT5C + half * kT5Cols + c0, r);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        }
+        if (SAMPLE) {
+          float v[32];
 #pragma unroll
-                for (int j4 = 0; j4 < 32; j4 += 4) {
-                  const float4 n4 = *reinterpret_cast<const float4*>(nc + c0 + j4);
-                  const float nn[4] = {n4.x, n4.y, n4.z, n4.w};
+          for (int j = 0; j < 32; ++j) v[j] = dead ? INFINITY : fmaf(-2.f, __uint_as_float(r[j]), nc[c0 + j]);
+          const int gs = a.gshift, G = 1 << gs;
 #pragma unroll
-                  for (int jj = 0; jj < 4; ++jj) {
-                    const float g = fmaf(-2.f, __uint_as_float(r[j4 + jj]), nn[jj]);
-                    asm volatile("{\n\t.reg .pred p;\n\t.reg .u64 a;\n\t.reg .f32 f;\n\tsetp.le.f32 p, %1, %2;\n\t"
-                                 "cvt.u64.u32 a, %0;\n\tadd.u64 a, a, %5;\n\t"
-                                 "@p add.rn.f32 f, %1, %4;\n\t"
-                                 "@p st.global.v2.b32 [a], {%3, f};\n\t"
-                                 "@p add.u32 %0, %0, 8;\n\t}"
-                                 : "+r"(woff) : "f"(g), "f"(thr_g), "r"(cbase + j4 + jj), "f"(nq), "l"(lst) : "memory");
-                  }
-                }
-              } else {
-                // the ragged last candidate tile and the tile that holds the queries themselves
+          for (int w = 1; w < 32; w *= 2) {
+            if (G > w) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                  const float g = fmaf(-2.f, __uint_as_float(r[j]), nc[c0 + j]);
-                  const int cand = cbase + j;
-                  if (g <= thr_g && cand < L && cand != qi) {
-                    lst[woff >> 3] = (static_cast<unsigned long long>(__float_as_uint(g + nq)) << 32) | static_cast<unsigned>(cand);
-                    woff += 8;
-                  }
-                }
+              for (int j = 0; j < 32; ++j)
+                if (j % (2 * w) == 0) v[j] = fminf(v[j], v[j + w]);
+            }
+          }
+          float* to = mins + ((t * kT5C + half * kT5Cols + c0) >> gs);
+          if (G >= 16) {
+            to[0] = v[0];
+            if (G == 16) to[1] = v[16];
+          } else {                                   // four minima and more per 32 columns: 16-byte stores
+#pragma unroll
+            for (int w = 1; w < 16; w *= 2) {
+              if (G == w) {
+#pragma unroll
+                for (int j = 0; j < 32 / w; j += 4)
+                  *reinterpret_cast<float4*>(to + j) = make_float4(v[j * w], v[(j + 1) * w], v[(j + 2) * w], v[(j + 3) * w]);
               }
             }
           }
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          t5_arrive(tempty(b));
+        } else if (!dead && !ovf) {
+          const int cbase = t * kT5C + half * kT5Cols + c0;
+          // per candidate: one FMA, one compare, and a store and pointer step that are predicated in the
+          // instruction stream (a branch here would diverge on a fifth of the candidates)
+#pragma unroll
+          for (int j4 = 0; j4 < 32; j4 += 4) {
+            const float4 n4 = *reinterpret_cast<const float4*>(nc + c0 + j4);
+            const float nn[4] = {n4.x, n4.y, n4.z, n4.w};
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+              const float g = fmaf(-2.f, __uint_as_float(r[j4 + jj]), nn[jj]);
+              asm volatile("{\n\t.reg .pred p;\n\tsetp.le.f32 p, %1, %2;\n\t"
+                           ".reg .u64 a;\n\tcvt.u64.u32 a, %0;\n\tadd.u64 a, %4, a;\n\t"
+                           "@p st.global.v2.b32 [a], {%3, %1};\n\t"
+                           "@p add.u32 %0, %0, 8;\n\t}"
+                           : "+r"(woff) : "f"(g), "f"(thr), "r"(cbase + j4 + jj), "l"(a.lists) : "memory");
+            }
+          }
         }
-        ++tiles_done;
-        cnt = static_cast<int>(woff >> 3);
+      }
+      if (!dead) {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        t5_arrive(tempty(b));
+      }
+      if (!SAMPLE) {
         // a list that could overflow during the next tile is cut back by its warp
-        uint32_t m = __ballot_sync(0xffffffffu, active && !ovf && !dead && cnt > CAP - kT5C);
+        uint32_t m = __ballot_sync(0xffffffffu, !ovf && !dead && static_cast<int>((woff - base) >> 3) > a.cap - kT5Cols);
         while (m) {
           const int src = __ffs(m) - 1;
           m &= m - 1;
-          const int nq_l = __shfl_sync(0xffffffffu, cnt, src);
-          const float eq = __shfl_sync(0xffffffffu, e2, src);
-          unsigned long long* lq = my_lists + static_cast<size_t>(warp * 32 + src) * CAP;
-          uint32_t limit;
-          const int kept = t5_warp_cut<true, 32>(lq, nq_l, k, st_w, hist_w, lq,
-                                       [&](uint32_t kth) { return float_key(key_float(kth) + eq); }, &limit);
+          const int cnt = __shfl_sync(0xffffffffu, static_cast<int>((woff - base) >> 3), src);
+          const float mg = __shfl_sync(0xffffffffu, margin, src);
+          unsigned long long* lq = a.lists + (static_cast<size_t>((tile * a.split + part) * kT5Per + half) * kT5Q + (warp & 3) * 32 + src) * a.cap;
+          float limit;
+          const int kept = t5_warp_cut(lq, cnt, a.k + 1, mg, hist_w, &limit);
           if (lane == src) {
-            cnt = kept;
-            woff = static_cast<uint32_t>(kept) * 8u;
-            const float thr = key_float(limit);
-            thr_g = (thr - nq) + 4.76837158203125e-7f * (fabsf(thr) + nq);
-            if (kept > CAP - kT5C) ovf = true;                  // too many rows within the error margin
+            woff = base + static_cast<uint32_t>(kept) * 8u;
+            thr = fminf(thr, limit);
+            if (kept > a.cap - kT5Cols) ovf = true;              // too many rows within the error margin
           }
         }
       }
-      cnts[tid] = ovf ? -1 : cnt;
     }
-    __syncthreads();                                 // every role is through this query tile; the stages are free
-    dead = dead || *abort != 0;
-    // ---------------------------------------------------------------- exact ranking: one query per warp at a time
-    {
-      unsigned char* slot = Bs + static_cast<size_t>(warp) * knn_t5_slot(CAP, d);
-      unsigned long long* st = reinterpret_cast<unsigned long long*>(slot);
-      uint32_t* hist = reinterpret_cast<uint32_t*>(st + CAP);
-      unsigned long long* sortd = reinterpret_cast<unsigned long long*>(hist + 256);   // bit patterns of doubles >= 0
-      int* sorti = reinterpret_cast<int*>(sortd + kT5Sort);
-      double* qd = reinterpret_cast<double*>(sorti + kT5Sort);
-      for (int q = warp; q < QT; q += kT5Threads / 32) {
-        const int qi = q0 + q;
-        if (qi >= L) break;
-        int32_t* out_i = a.nbr_idx + static_cast<long long>(qi) * k;
-        float* out_d = a.nbr_dist ? a.nbr_dist + static_cast<long long>(qi) * k : nullptr;
-        if (dead) {
-          for (int r = lane; r < k; r += 32) { out_i[r] = -1; if (out_d) out_d[r] = 0.f; }
-          continue;
-        }
-        const unsigned long long* lq = my_lists + static_cast<size_t>(q) * CAP;
-        int n = cnts[q];
-        bool fallback = n < 0;
-        if (!fallback) {
-          if (n > k) {
-            const float eq = eps2s[q];
-            uint32_t limit;
-            n = t5_warp_cut<false, 2>(lq, n, k, st, hist, st, [&](uint32_t kth) { return float_key(key_float(kth) + eq); }, &limit);
-          } else {
-            for (int i = lane; i < n; i += 32) st[i] = lq[i];
-            __syncwarp();
-          }
-          fallback = n > kT5Sort;
-        }
-        if (fallback) {
-          if (lane == 0) cnts[q] = -2;
-          continue;
-        }
-        int p2 = 32;
-        while (p2 < n) p2 *= 2;
-        const __nv_bfloat16* q_row = cb + static_cast<long long>(qi) * d;
-        for (int t = lane; t < d; t += 32) qd[t] = t5_bf16_to_double(__bfloat16_as_ushort(q_row[t]));
-        __syncwarp();
-        {
-          // groups of 32 candidates, spread evenly over as few calls as the chains per lane allow
-          const int groups = max((n + 31) / 32, 1), calls = (groups + kT5Chains - 1) / kT5Chains;
-          const int nch = (groups + calls - 1) / calls;
-          for (int c2 = 0; c2 < calls; ++c2) t5_exact_block(qd, cb, d, st, n, p2, c2 * 32 * nch, nch, sortd, sorti);
-          for (int i = calls * 32 * nch + lane; i < p2; i += 32) {       // padding of the sort beyond the calls' range
-            sorti[i] = 0x7fffffff;
-            sortd[i] = 0x7ff0000000000000ull;
-          }
-        }
-        __syncwarp();
-        t5_warp_sort(sortd, sorti, p2);
-        for (int r = lane; r < k; r += 32) {
-          out_i[r] = sorti[r];
-          if (out_d) out_d[r] = static_cast<float>(__longlong_as_double(static_cast<long long>(sortd[r])));
-        }
-        __syncwarp();
-      }
-    }
-    __syncthreads();
-    // queries with too many rows inside the error margin (duplicated rows): exact arg-min rounds by the whole CTA
-    if (!dead) {
-      double* redd = reinterpret_cast<double*>(bars + 16);
-      int* redi = misc + 16;
-      for (int q = 0; q < QT && q0 + q < L; ++q) {
-        if (cnts[q] != -2) continue;                 // shared value: the same decision in every thread
-        const int qi = q0 + q;
-        rank_query<__nv_bfloat16>(cb, L, d, k, qi, nullptr, 0, true, 0, nullptr, nullptr, redd, redi,
-                                  a.nbr_idx + static_cast<long long>(qi) * k,
-                                  a.nbr_dist ? a.nbr_dist + static_cast<long long>(qi) * k : nullptr);
-      }
-    }
-    __syncthreads();                                 // the stages go back to the loaders
+    if (!SAMPLE) a.counts[seg] = dead ? -9 : (ovf || !active ? -1 : static_cast<int>((woff - base) >> 3));
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 4) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(2 * kT5C) : "memory");
+  if (warp == kT5Mma) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(2 * kT5C) : "memory");
+}
+
+// Squared norms (float32) and the largest of those below kT5Huge, and the operand tiles (the layout is at KnnT5Args):
+// [h l h] and [h h l] of float32 elements (each part d elements) on the query and the candidate side, bfloat16
+// rows as they are on both, zero beyond.  One warp per row of a tile; rows from `tiles` * 128 on are those of the
+// sample, row i of it being codebook row (i * step) >> 32.  The eight warps of a CTA write one row group, 128
+// contiguous bytes per chunk.
+struct KnnPrepArgs {
+  const void* cb;
+  int L, d, dp, rows, sampled;      // tile rows of the candidate side, of the sample (multiples of 128; 0: no sample tiles)
+  unsigned long long step;
+  float *nrm, *cn, *sn;             // nrm[L + 1]: non-zero when an element is not +0 and not of ordinary size (bfloat16 rows)
+  unsigned char *qm, *cm, *sm;      // cm == qm for bfloat16 rows
+};
+template <typename T>
+__global__ void __launch_bounds__(256) knn_prep_kernel(const KnnPrepArgs a) {
+  const int out = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  const bool sample = out >= a.rows;
+  const int tr = sample ? out - a.rows : out;                  // row among the tiles of its side
+  const int row = sample ? static_cast<int>((static_cast<unsigned long long>(tr) * a.step) >> 32) : tr;
+  const bool in = row < a.L;
+  const int d = a.d, dp = a.dp;
+  const T* src = static_cast<const T*>(a.cb) + static_cast<long long>(in ? row : 0) * d;
+  float s = 0.f;
+  bool odd = false;                                            // -0, below 2^-60, infinite or NaN
+  for (int t = lane; t < d; t += 32) {
+    const float v = static_cast<float>(src[t]);
+    s = fmaf(v, v, s);
+    odd |= !(fabsf(v) >= 8.673617379884035e-19f && fabsf(v) <= FLT_MAX) && __float_as_uint(v) != 0u;
+  }
+  s = warp_sum(s);
+  odd = __any_sync(0xffffffffu, odd);
+  if (lane == 0) {
+    if (odd && !sample && in) a.nrm[a.L + 1] = 1.f;
+    (sample ? a.sn : a.cn)[tr] = in ? s : INFINITY;
+    if (!sample && in) {
+      a.nrm[row] = s;
+      unsigned int* top = reinterpret_cast<unsigned int*>(a.nrm + a.L);      // s >= 0: bit order = value order
+      if (s < kT5Huge && __float_as_uint(s) > __ldcg(top)) atomicMax(top, __float_as_uint(s));
+    }
+  }
+  const size_t base = static_cast<size_t>(tr >> 7) * (static_cast<size_t>(dp) * 256) + static_cast<size_t>((tr & 127) >> 3) * 128 + (tr & 7) * 16;
+  for (int c = lane; c < dp / 8; c += 32) {
+    union { __nv_bfloat16 h[8]; uint4 v; } x, y;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int t = c * 8 + e;
+      x.h[e] = y.h[e] = __float2bfloat16_rn(0.f);
+      if (sizeof(T) == 2) {
+        if (in && t < d) x.h[e] = __float2bfloat16_rn(static_cast<float>(src[t]));
+      } else if (in && t < 3 * d) {
+        const int part = t / d;
+        const float v = static_cast<float>(src[t - part * d]);
+        const __nv_bfloat16 h = __float2bfloat16_rn(v), l = __float2bfloat16_rn(v - __bfloat162float(h));
+        x.h[e] = part == 1 ? l : h;
+        y.h[e] = part == 2 ? l : h;
+      }
+    }
+    const size_t at = base + static_cast<size_t>(c) * 2048;
+    if (sizeof(T) == 2) {
+      *reinterpret_cast<uint4*>((sample ? a.sm : a.qm) + at) = x.v;
+    } else {
+      if (!sample) *reinterpret_cast<uint4*>(a.qm + at) = x.v;
+      *reinterpret_cast<uint4*>((sample ? a.sm : a.cm) + at) = y.v;
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------ exact ranking
+struct KnnRankArgs {
+  const void* cb;
+  const float* nrm;
+  const unsigned long long* lists;
+  const int* counts;
+  int L, d, k, cap, split;
+  int q0;                           // first query of the chunk
+  int lanes;                        // lanes that share one candidate's distance (power of two); 0: rows read element by element
+  float eps1, eps0;
+  int32_t* nbr_idx;
+  float* nbr_dist;
+};
+constexpr int kRankThreads = 128;
+__host__ __device__ constexpr size_t knn_rank_smem(int d) {
+  return kT5Sort * (8 + 8 + 4) + 256 * 4 + static_cast<size_t>((d + 7) / 8 * 8) * 8 + 16 * 8 + 64;
+}
+
+// Eight elements to double.  For normal bfloat16 numbers the double's high word is the sign, the exponent rebiased by
+// 1023 - 127 and the 7 mantissa bits: integer operations instead of the converting instruction's quarter rate.
+// The same operations turn +0 into 2^-127, which changes no difference with a number of at least 2^-60 in
+// magnitude and none between zeros; codebooks with anything else (knn_prep_kernel looks) take the instruction (PLAIN).
+__device__ __forceinline__ double bf16_high_to_double(uint32_t w) {          // the upper 16 bits
+  return __hiloint2double((static_cast<int>(w) >> 3 & static_cast<int>(0x8fffe000u)) + (896 << 20), 0);
+}
+template <bool PLAIN>
+__device__ __forceinline__ void widen8(const __nv_bfloat16* p, double (&x)[8]) {
+  const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    x[2 * i] = PLAIN ? static_cast<double>(__uint_as_float(w[i] << 16)) : bf16_high_to_double(w[i] << 16);
+    x[2 * i + 1] = PLAIN ? static_cast<double>(__uint_as_float(w[i] & 0xffff0000u)) : bf16_high_to_double(w[i]);
+  }
+}
+template <bool PLAIN>
+__device__ __forceinline__ void widen8(const float* p, double (&x)[8]) {
+  const float4 v = __ldg(reinterpret_cast<const float4*>(p)), w = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; x[4] = w.x; x[5] = w.y; x[6] = w.z; x[7] = w.w;
+}
+
+// Exact squared distances between the query row `qd` (pair e of chunk c at pair e * (d / 8) + c) and the n candidates of
+// `st`: G lanes per candidate, lane g of them sums the elements [8 c, 8 c + 8), c = g (mod G).
+template <typename T, bool PLAIN>
+__device__ __forceinline__ void exact_block(const T* __restrict__ cb, int d, int G, const double* qd, const unsigned long long* st, int n,
+                                            unsigned long long* sortd, int* sorti) {
+  const int tid = threadIdx.x, g = tid & (G - 1), per = kRankThreads / G, nch = d >> 3;
+  for (int i0 = 0; i0 < n; i0 += per) {
+    const int i = i0 + tid / G;
+    const int j = i < n ? static_cast<int>(st[i] & 0xffffffffu) : 0;
+    const T* row = cb + static_cast<long long>(j) * d;
+    double s = 0.0;
+#pragma unroll 4
+    for (int c = g; c < nch; c += G) {
+      double x[8];
+      widen8<PLAIN>(row + c * 8, x);
+      const double2* qp = reinterpret_cast<const double2*>(qd) + c;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const double2 qv = qp[e * nch];
+        const double d0 = qv.x - x[2 * e], d1 = qv.y - x[2 * e + 1];
+        s = fma(d0, d0, s);
+        s = fma(d1, d1, s);
+      }
+    }
+    for (int o = 1; o < G; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (g == 0 && i < n) { sorti[i] = j; sortd[i] = static_cast<unsigned long long>(__double_as_longlong(s)); }
+  }
+}
+
+// One CTA of 128 threads per query, up to 16 of them per SM: every step is short, and what bounds it is
+// the latency of scattered row reads (L2) and of the double-precision chains, so warps in flight count.
+// A candidate's distance is shared by up to 8 lanes, 8 consecutive elements (one or two 16-byte loads) each, so
+// that a warp reads whole 128-byte lines.
+template <typename T>
+__global__ void __launch_bounds__(kRankThreads) knn_rank_kernel(const KnnRankArgs a) {
+  extern __shared__ __align__(16) unsigned char rank_smem[];
+  unsigned long long* st = reinterpret_cast<unsigned long long*>(rank_smem);     // [kT5Sort] survivors
+  unsigned long long* sortd = st + kT5Sort;                                      // [kT5Sort] bits of doubles >= 0
+  double* qd = reinterpret_cast<double*>(sortd + kT5Sort);                       // [d] the query row
+  double* redd = qd + (a.d + 7) / 8 * 8;                                         // [4]
+  int* sorti = reinterpret_cast<int*>(redd + 16);                                // [kT5Sort]
+  uint32_t* hist = reinterpret_cast<uint32_t*>(sorti + kT5Sort);                 // [256]
+  int* misc = reinterpret_cast<int*>(hist + 256);                                // [0] survivors, [1..4] minima, [5..8] maxima, [9..12] counts, [12..15] redi
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const T* cb = static_cast<const T*>(a.cb);
+  const int ql = blockIdx.x, qi = a.q0 + ql, k = a.k, d = a.d;
+  const int nseg = a.split * kT5Per;
+  int32_t* out_i = a.nbr_idx + static_cast<long long>(qi) * k;
+  float* out_d = a.nbr_dist ? a.nbr_dist + static_cast<long long>(qi) * k : nullptr;
+  const size_t seg0 = static_cast<size_t>(ql / kT5Q) * nseg * kT5Q + ql % kT5Q;      // segment s: + s * kT5Q
+  const float nq = a.nrm[qi], nmax = a.nrm[a.L];
+  const bool nrm_odd = a.nrm[a.L + 1] != 0.f;
+  bool lost = false, whole = nq < kT5Huge && nmax < 1e35f;
+  for (int s = 0; s < nseg; ++s) {
+    const int c = a.counts[seg0 + static_cast<size_t>(s) * kT5Q];
+    lost |= c == -9;
+    whole &= c >= 0;
+  }
+  if (lost) {                                        // a wait of the contraction ran out
+    for (int r = tid; r < k; r += kRankThreads) { out_i[r] = -1; if (out_d) out_d[r] = 0.f; }
+    return;
+  }
+  // the query row in double precision; pair e of chunk c (elements 8 c + 2 e, + 1) at pair e * (d / 8) + c, so that the
+  // lanes of one candidate read consecutive 16-byte words
+  if (a.lanes > 0)
+    for (int t = tid; t < d; t += kRankThreads)
+      qd[(((t & 7) >> 1) * (d >> 3) + (t >> 3)) * 2 + (t & 1)] =
+          (sizeof(T) == 4 || nrm_odd) ? static_cast<double>(static_cast<float>(cb[static_cast<long long>(qi) * d + t]))
+                                      : bf16_high_to_double(__float_as_uint(static_cast<float>(cb[static_cast<long long>(qi) * d + t])));
+  if (tid == 0) misc[0] = 0;
+  // fn(entry, whether there is one) for every list entry but the query itself, by whole warps
+  auto for_each = [&](auto&& fn) {
+    for (int s = 0; s < nseg; ++s) {
+      const size_t seg = seg0 + static_cast<size_t>(s) * kT5Q;
+      const unsigned long long* lst = a.lists + seg * a.cap;
+      const int n = a.counts[seg];
+      for (int i0 = warp * 32; i0 < n; i0 += kRankThreads) {
+        const int i = i0 + lane;
+        const unsigned long long e = i < n ? lst[i] : 0ull;
+        fn(e, i < n && static_cast<int>(e & 0xffffffffu) != qi);
+      }
+    }
+  };
+  int n = 0;
+  if (whole) {
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+    int cnt = 0;
+    for_each([&](unsigned long long e, bool in) {
+      const uint32_t key = t5_entry_key(e);
+      if (in) {
+        kmin = min(kmin, key);
+        kmax = max(kmax, key);
+        ++cnt;
+      }
+    });
+    kmin = __reduce_min_sync(0xffffffffu, kmin);
+    kmax = __reduce_max_sync(0xffffffffu, kmax);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) { hist[warp] = kmin; hist[4 + warp] = kmax; hist[8 + warp] = static_cast<uint32_t>(cnt); }
+    __syncthreads();
+    kmin = min(min(hist[0], hist[1]), min(hist[2], hist[3]));
+    kmax = max(max(hist[4], hist[5]), max(hist[6], hist[7]));
+    cnt = static_cast<int>(hist[8] + hist[9] + hist[10] + hist[11]);
+    __syncthreads();
+    whole = cnt >= k;
+    if (whole) {
+      uint32_t kth = kmax;
+      if (cnt > k)
+        kth = t5_digit_select(kmin, kmax, k, 2, hist, tid, kRankThreads, [] { __syncthreads(); },
+                              [&](int lo, uint32_t mask, int hi, uint32_t prefix) {
+          for_each([&](unsigned long long e, bool in) {
+            const uint32_t rel = t5_entry_key(e) - kmin;
+            if (in && (hi == 32 || (rel >> hi) == prefix)) atomicAdd(&hist[(rel >> lo) & mask], 1u);
+          });
+        });
+      const float limit = __fadd_ru(key_float(kth), 2.f * fmaf(a.eps1, nq + nmax, a.eps0));
+      for_each([&](unsigned long long e, bool in) {
+        const bool keep = in && __uint_as_float(static_cast<uint32_t>(e >> 32)) <= limit;
+        const uint32_t m = __ballot_sync(0xffffffffu, keep);
+        if (m == 0u) return;
+        int pos = 0;
+        if (lane == 0) pos = atomicAdd(&misc[0], __popc(m));
+        pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(m & ((1u << lane) - 1u));
+        if (keep && pos < kT5Sort) st[pos] = e;
+      });
+      __syncthreads();
+      n = misc[0];
+      whole = n <= kT5Sort;
+    }
+  } else {
+    __syncthreads();
+  }
+  if (!whole) {                                      // too few or too many rows under the bound: duplicated rows, huge norms
+    argmin_rounds<T, kRankThreads>(cb, a.L, d, k, qi, redd, misc + 12, out_i, out_d);
+    return;
+  }
+  int p2 = 32;
+  while (p2 < n) p2 *= 2;
+  if (a.lanes > 0) {
+    if (sizeof(T) == 4 || nrm_odd) exact_block<T, true>(cb, d, a.lanes, qd, st, n, sortd, sorti);
+    else exact_block<T, false>(cb, d, a.lanes, qd, st, n, sortd, sorti);
+  } else {
+    for (int i = tid; i < n; i += kRankThreads) {
+      const int j = static_cast<int>(st[i] & 0xffffffffu);
+      sorti[i] = j;
+      sortd[i] = static_cast<unsigned long long>(__double_as_longlong(exact_dist<T>(cb, d, qi, j)));
+    }
+  }
+  for (int i = n + tid; i < p2; i += kRankThreads) { sorti[i] = 0x7fffffff; sortd[i] = 0x7ff0000000000000ull; }
+  __syncthreads();
+  // ascending bitonic sort of (distance, index): non-negative doubles order like their bit patterns
+  for (int size = 2; size <= p2; size <<= 1) {
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      for (int i = tid; i < (p2 >> 1); i += kRankThreads) {
+        const int lo = 2 * i - (i & (stride - 1)), hi = lo + stride;
+        const bool up = (lo & size) == 0;
+        const unsigned long long dx = sortd[lo], dy = sortd[hi];
+        const int ix = sorti[lo], iy = sorti[hi];
+        const bool gt = dx > dy || (dx == dy && ix > iy);
+        if (gt == up) { sortd[lo] = dy; sortd[hi] = dx; sorti[lo] = iy; sorti[hi] = ix; }
+      }
+      __syncthreads();
+    }
+  }
+  for (int r = tid; r < k; r += kRankThreads) {
+    out_i[r] = sorti[r];
+    if (out_d) out_d[r] = static_cast<float>(__longlong_as_double(static_cast<long long>(sortd[r])));
+  }
 }
 
 }  // namespace lantern

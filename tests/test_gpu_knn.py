@@ -173,3 +173,72 @@ def test_tcgen05_kernel_on_clustered_rows_with_many_near_ties(L):
     assert idx.min() >= 0 and idx.max() < n
     # the first 129 neighbours of a row lie in its own cluster (same index modulo 64)
     assert np.all(idx[:, :100] % 64 == (np.arange(n) % 64)[:, None])
+
+
+@pytest.mark.parametrize("n,d,k,dt", [(64, 5, 40, "f32"), (127, 1, 20, "f32"), (129, 85, 100, "f32"), (700, 86, 30, "f32"),
+                                      (1025, 8, 320, "f32"), (4097, 33, 64, "f32"), (300, 12, 50, "bf16"), (2050, 100, 200, "bf16"),
+                                      (1151, 256, 1, "bf16"), (18945, 16, 30, "bf16"), (19100, 4, 9, "f32"), (65600, 8, 3, "f32")])
+def test_tcgen05_kernels_at_the_edges_of_their_tiles(L, n, d, k, dt):
+    """Ragged and single tiles, one and several shares of the candidates per query tile, a second chunk of query
+    tiles (more than 148 * 128 rows), float32 rows of one to 85 elements and one too wide, bfloat16 rows whose
+    length no vector load divides, the smallest and the largest k; duplicate rows throughout."""
+    cb = W.make_codebook(n, d, dt, seed=n + d + k, dup_frac=0.05)
+    rng = np.random.default_rng(4)
+    last = ((n - 1) // 128) * 128
+    rows = None if n <= 300 else [0, 127, 128, n - 1, last, max(0, last - 1)] + [int(x) for x in rng.integers(0, n, 8)]
+    idx, _ = _check(L, cb, k, rows=rows)
+    assert idx.min() >= 0 and idx.max() < n and not np.any(idx == np.arange(n)[:, None])
+    s = np.sort(idx, axis=1)
+    assert np.all(s[:, 1:] != s[:, :-1])
+
+
+def _extreme(kind, n, d, g):
+    cb = torch.randn((n, d), generator=g)
+    if kind == "zeros":                  # half of all elements zero, some of them -0
+        m = torch.rand((n, d), generator=g)
+        cb[m < 0.5] = 0.0
+        cb[m < 0.05] = -0.0
+    elif kind == "tiny":                 # squares far below the normal range of float32
+        cb *= 1e-22
+    elif kind == "huge":                 # a few rows whose squared norm no float32 holds
+        cb[5::97] *= 1e22
+    elif kind == "far":                  # a common offset: the inner products cancel almost entirely
+        cb += 300.0
+    elif kind == "sorted":               # rows in the order of their first element: neighbours sit in a few tiles
+        cb = cb * 0.05
+        cb[:, 0] = torch.linspace(-50.0, 50.0, n)
+    return cb
+
+
+@pytest.mark.parametrize("kind", ["zeros", "tiny", "huge", "far", "sorted"])
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+def test_tcgen05_kernels_on_extreme_rows(L, kind, dt):
+    n, d, k = 1400, 16, 24
+    cb = _extreme(kind, n, d, torch.Generator().manual_seed(8)).to(torch.float32 if dt == "f32" else torch.bfloat16)
+    idx, dist = L.build_neighbors(cb.cuda(), k, return_dist=True)
+    idx, dist = idx.cpu().numpy(), dist.cpu().numpy()
+    x = cb.to(torch.float64).numpy()
+    for i in [0, 5, 6, 102, 700, n - 1]:
+        D = ((x - x[i]) ** 2).sum(axis=1)
+        D[i] = np.inf
+        want = np.lexsort((np.arange(n), D))[:k]
+        # (the double sums differ in their last bits between the two sides: only distances closer than that may swap)
+        assert np.all((idx[i] == want) | (np.abs(D[idx[i]] - D[want]) <= 1e-13 * D[want]))
+        with np.errstate(over="ignore"):
+            assert np.allclose(dist[i], D[idx[i]].astype(np.float32), rtol=1e-6, atol=0)
+
+
+def test_float32_codebook_without_a_workspace_takes_the_brute_force_kernel(L):
+    import ctypes
+    from paper_2502_06352_b200.binding import lib
+    n, d, k = 900, 10, 12
+    cb = W.make_codebook(n, d, "f32", seed=2, dup_frac=0.05).cuda()
+    want, wd = L.build_neighbors(cb, k, return_dist=True)
+    idx, dist = torch.empty_like(want), torch.empty_like(wd)
+    p = lambda t: ctypes.c_void_p(t.data_ptr())
+    assert lib.lantern_build_neighbors(p(cb), 0, n, d, k, p(idx), p(dist), None, 0, None) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(idx, want) and torch.equal(dist, wd)
+    # a bfloat16 shape that has always needed its workspace is still refused
+    b = W.make_codebook(600, 32, "bf16", seed=2).cuda()
+    assert lib.lantern_build_neighbors(p(b), 1, 600, 32, k, p(idx), p(dist), None, 0, None) == 3
