@@ -15,6 +15,8 @@
 namespace lantern {
 using namespace v1024;
 
+constexpr int kInlineParents = 128;   // parents per sequence that travel in the kernel arguments
+
 struct SampleArgs {
   const void *dc, *du;
   long long row_stride, seq_stride;
@@ -31,6 +33,9 @@ struct SampleArgs {
   int n_parents;       // parents per sequence in this launch
   int repair;          // non-zero: draw only the parents whose first child's token is the redo marker
   uint32_t rk0[10], rk1[10];   // Philox round keys of `seed`
+  int inlined;         // non-zero: the parents of this launch, their first children and numbers of children are below
+  uint16_t p_node[kInlineParents], p_child[kInlineParents];
+  uint8_t p_count[kInlineParents];
 };
 
 }  // namespace lantern
@@ -429,18 +434,17 @@ bool sampler_uses_lists(const lantern_params* p) {
 }
 }  // namespace
 
-// Rows that no top-k truncates can take the streaming kernel; it does when the call expands at
-// least kStreamMinParents parents or kStreamMinLogits / V of them (fewer fit the dense kernel's one
-// wave of CTAs, or of CTA clusters for wide rows, whose shared-memory row shortens the chain of
-// dependent steps: the measured cross-over lies between 2.6 M and 5.2 M parents x V for V = 16384
-// and 65536, whatever the allowed range), when the dense kernel cannot hold the row, or when asked to.
+// Rows that no top-k truncates take the streaming kernel, but for a few narrow rows (below kStreamMinV
+// tokens one CTA of the dense kernel holds a float32 row in one load per thread, with no cluster), unless
+// the parameters say otherwise.  One row of 16384 logits: 8 us, dense 13; four to twenty rows of 65536 of which 8192
+// tokens are allowed: 8 us, dense 18 to 35.
 constexpr int kStreamMinParents = 256;
-constexpr long long kStreamMinLogits = 4ll << 20;
+constexpr int kStreamMinV = 4096;
 static bool sampler_uses_stream(const lantern_params* p, long long parents, bool fits_dense) {
   if ((p->top_k_draft > 0 && p->top_k_draft < p->vocab) || p->vocab > stream::kMaxV) return false;
   if (p->kernels == 2) return !fits_dense;
   if (p->kernels == 1) return true;
-  return parents >= kStreamMinParents || parents * p->vocab >= kStreamMinLogits || !fits_dense;
+  return parents >= kStreamMinParents || p->vocab >= kStreamMinV || !fits_dense;
 }
 
 extern "C" int32_t lantern_sample_draft_tree_path(const lantern_params* p, const lantern_tree* tree, int32_t batch) {
@@ -491,6 +495,16 @@ extern "C" lantern_status lantern_sample_draft_tree(
   a.tokens = tokens; a.draft_prob = draft_prob; a.status = device_status;
   a.n_parents = i1 - i0;
   a.repair = 0;
+  a.inlined = (i1 - i0 <= kInlineParents && t->n_nodes <= 65536) ? 1 : 0;
+  if (a.inlined) {
+    int w = 0;
+    for (int n = parent_begin; n < parent_end; ++n) {
+      if (t->h_n_child[n] == 0) continue;
+      a.p_node[w] = static_cast<uint16_t>(n);
+      a.p_child[w] = static_cast<uint16_t>(t->h_first_child[n]);
+      a.p_count[w++] = static_cast<uint8_t>(t->h_n_child[n]);
+    }
+  }
   for (int r = 0; r < 10; ++r) {
     a.rk0[r] = static_cast<uint32_t>(p->seed) + static_cast<uint32_t>(r) * 0x9E3779B9u;
     a.rk1[r] = static_cast<uint32_t>(p->seed >> 32) + static_cast<uint32_t>(r) * 0xBB67AE85u;
@@ -503,8 +517,10 @@ extern "C" lantern_status lantern_sample_draft_tree(
   const bool fits_dense = sampler_shape(V, batch * (i1 - i0), dt == LANTERN_F32 ? 4 : 8, ov, &cs_d, &e_d, &smem_d);
   if (p->kernels < 0 || p->kernels > 2) return LANTERN_ERR_INVALID_ARG;
   if (sampler_uses_stream(p, static_cast<long long>(batch) * (i1 - i0), fits_dense)) {
-    // CTAs per parent: the smallest power of two that gives every SM a CTA (measured on rows of 65536 logits:
-    // 80 and 100 parents run fastest split in two, 200 unsplit; wider clusters pay for their merge)
+    // CTAs per parent: the smallest power of two that gives every SM a CTA while every warp keeps at least one
+    // full step of the row.  Wider clusters repeat the chain of a CTA's first chunk and merge more lists: 144 rows
+    // of 65536 logits take 39 / 28 / 34 / 40 us on 1 / 2 / 4 / 8 CTAs, one row of 16384 takes 12 / 10 / 8 / 10 us on
+    // 1 / 4 / 8 / 16.
     int cs = ov;
     if (cs <= 0) {
       int dev = 0, sms = 0;
@@ -513,7 +529,7 @@ extern "C" lantern_status lantern_sample_draft_tree(
         sms = 148;
       const int nvec = (allow_hi - allow_lo) / (dt == LANTERN_F32 ? 4 : 8);
       cs = 1;
-      while (cs < 16 && static_cast<long long>(batch) * (i1 - i0) * cs < sms && nvec / (2 * cs * stream::SW) >= 32) cs *= 2;
+      while (cs < 8 && static_cast<long long>(batch) * (i1 - i0) * cs < sms && nvec / (2 * cs * stream::SW) >= 32) cs *= 2;
     }
     return launch_sample_stream(a, cs, dt == LANTERN_F32, cfg, st) == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
   }

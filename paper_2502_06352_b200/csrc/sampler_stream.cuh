@@ -2,15 +2,22 @@
 //
 // The s children of a parent are the s largest keys z_j + G_j, G_j = -log(-log U_j) (Gumbel-top-s,
 // sampling without replacement from p).  The drafter row is streamed from HBM once and never held
-// on chip: every element gets a float32 key from fast logarithms (absolute error below kKeyEps),
-// and only the elements whose key exceeds a running threshold T are appended to a short candidate
-// list in shared memory.  T is a lower bound of the (s+4)-th largest key seen so far: when the
-// list would overflow it is cut back to its s+4 best entries and T rises to the last of them, so
-// every element left out has key <= T.  At the end the few candidates are ranked by keys
-// recomputed in double precision (ties: lower token id); the result is the exact ranking as
-// long as the s-th exact key clears T by kKeyEps, which is checked (LANTERN_DEV_KEY_TIES
-// otherwise: more than s+4 keys within 2.5e-4 of each other at the top).  The softmax
-// denominator for draft_prob comes from the same pass.
+// on chip.  The first chunk's elements get float32 keys from fast logarithms (absolute error below
+// kKeyEps); the (s+4)-th best of a few of them is a threshold T.  Every later element only has to
+// show whether it could beat T: z + G > T means -log U < e^(z-T), and -log U >= 1 - U, so an element
+// with 1 - U >= e^(z-T) is out.  That test costs one exponential and no logarithm, and the few
+// elements that pass it go to a candidate list in shared memory, whose keys are formed when the list
+// is cut back to its s+4 best entries and T rises to the last of them.  Every element left out has
+// key <= T.  At the end the few candidates are ranked by their float32 keys, or, when two of them (or
+// one and T) are closer than the keys' errors, by keys recomputed in double precision (ties: lower
+// token id); the result is the exact ranking as long as the s-th exact key clears T by kKeyEps, which
+// is checked (LANTERN_DEV_KEY_TIES otherwise: more than s+4 keys within 2.5e-4 of each other at the
+// top).  The softmax denominator for draft_prob comes from the same pass.
+//
+// Bound: instruction issue; the generator alone is 10 to 12 of about 20 instructions per element.  3200 rows of
+// 65536 bfloat16 logits: 244 us (two logarithms per element and branches between the vectors: 320); 144 rows of
+// 65536 float32 logits with guidance: 28 us, was 40; a row whose elements are one chunk per CTA is a chain of
+// barriers, 8 us on 8 CTAs.
 #pragma once
 #include "verify_stream.cuh"
 
@@ -19,12 +26,14 @@ namespace stream {
 
 constexpr int kIterElems = 4096;                 // row elements one CTA handles between two barriers
 constexpr int kListCap = kIterElems + 256;       // candidate entries
-constexpr int kFinal = 256;                      // candidates ranked exactly at the end
 constexpr int kExtra = 4;                        // the list is cut back to s + kExtra entries
-constexpr float kKeyEps = 2.5e-4f;               // bound on |fast key - exact key|
+constexpr int kMaxR = LANTERN_MAX_CHILDREN + kExtra;
+constexpr int kFinal = kMaxCluster * kMaxR;      // candidates of all CTAs of a row
+constexpr float kKeyEps = 2.5e-4f;               // bound on |fast key - exact key| (up to the constant below)
+constexpr float kKeyShift = -0.36651292f;        // ln(ln 2): fast keys are z + G + ln(ln 2)
 
 __host__ __device__ constexpr size_t sampler_stream_smem() {
-  return kSmallBytes + kListCap * 8 + kFinal * 12 + 2 * 2 * SW * 8 + 16 * 8;
+  return kSmallBytes + kListCap * 8 + kFinal * 16 + 2 * 2 * SW * 8 + 16 * 8 + kMaxCluster * 8;
 }
 
 __device__ __forceinline__ float lg2_approx(float x) {
@@ -55,12 +64,13 @@ __device__ __forceinline__ void warp_key_first(float& k, int& i) {
 }
 
 struct SampSmem {
-  uint2* list;      // [kListCap] (key bits, token)
+  uint2* list;      // [kListCap] (key bits, token); entries that only passed the test of the pass hold z bits instead
   int* cnt;         // entries in the list
-  double* fkey;     // [kFinal] exact keys
-  int* ftok;        // [kFinal]
+  uint2* fin;       // [kFinal] candidates of all CTAs of the row (key bits, token), in CTA 0
+  double* fkey;     // [kFinal] their exact keys
   uint2* pk;        // [2][SW] warps' best entries of a selection round
   uint2* top;       // [16] winners of the rounds of a cut
+  uint2* rinfo;     // [kMaxCluster] per CTA of the row: number of candidates, T (in CTA 0)
 };
 
 // Cut the list back to its R best entries (key descending, token ascending).  Returns the new
@@ -101,41 +111,36 @@ __device__ __forceinline__ float cut_list(const SampSmem& s, int R, float T) {
   return got == R ? pk : T;
 }
 
-// The same cut for a short list, by warp 0 alone (no barriers inside the rounds); every thread
-// calls it between two barriers' worth of quiet: nobody appends while it runs.  R <= 15.
-__device__ __forceinline__ float cut_small(const SampSmem& s, int R, float T) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int n = min(*s.cnt, kListCap);
-  __syncthreads();                               // every thread has read the count
-  if (tid < 32) {
-    float pk = INFINITY;
-    int pt = -1;
-    int got = 0;
-    for (int round = 0; round < R; ++round) {
-      float bk = -INFINITY;
-      int bt = 0x7fffffff;
-      for (int i = lane; i < n; i += 32) {
-        const uint2 en = s.list[i];
-        const float k = __uint_as_float(en.x);
-        const int t = static_cast<int>(en.y);
-        if (key_before(pk, pt, k, t) && key_before(k, t, bk, bt)) { bk = k; bt = t; }
-      }
-      warp_key_first(bk, bt);
-      if (bt == 0x7fffffff) break;               // fewer than R entries (the same in every lane)
-      if (lane == 0) s.top[round] = make_uint2(__float_as_uint(bk), static_cast<uint32_t>(bt));
-      pk = bk;
-      pt = bt;
-      ++got;
-    }
-    __syncwarp();
-    if (lane < got) s.list[lane] = s.top[lane];
-    if (lane == 0) {
-      *s.cnt = got;
-      s.top[15].x = __float_as_uint(got == R ? pk : T);
+// The same cut for a list of at most ST entries: every thread counts how many entries rank before its
+// own, so there is no chain of selection rounds.
+__device__ __forceinline__ float cut_ranked(const SampSmem& s, int R, float T) {
+  const int tid = threadIdx.x, n = *s.cnt;
+  float k = -INFINITY;
+  int t = 0x7fffffff, rank = 0;
+  if (tid < n) {
+    const uint2 en = s.list[tid];
+    k = __uint_as_float(en.x);
+    t = static_cast<int>(en.y);
+#pragma unroll 8
+    for (int i = 0; i < n; ++i) {
+      const uint2 o = s.list[i];
+      rank += key_before(__uint_as_float(o.x), static_cast<int>(o.y), k, t) ? 1 : 0;
     }
   }
+  __syncthreads();                               // every thread has read the list and its length
+  if (tid < n && rank < R) {
+    s.list[rank] = make_uint2(__float_as_uint(k), static_cast<uint32_t>(t));
+    if (rank == R - 1) s.top[15].x = __float_as_uint(k);
+  }
+  if (tid == 0) *s.cnt = min(n, R);
   __syncthreads();
-  return __uint_as_float(s.top[15].x);
+  return n >= R ? __uint_as_float(s.top[15].x) : T;
+}
+
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void dsmem_st_u64(uint32_t addr, uint2 v) {
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(v.x), "r"(v.y) : "memory");
 }
 
 template <typename T, bool CFG, bool TAU1>
@@ -154,20 +159,23 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
   int* misc = reinterpret_cast<int*>(c.gath + kMaxCluster * 4);     // [32]
   SampSmem s;
   s.list = reinterpret_cast<uint2*>(samp_smem + kSmallBytes);
-  s.fkey = reinterpret_cast<double*>(s.list + kListCap);
-  s.ftok = reinterpret_cast<int*>(s.fkey + kFinal);
-  s.pk = reinterpret_cast<uint2*>(s.ftok + kFinal);
-  s.top = s.pk + 2 * SW;
+  s.fin = s.list + kListCap;
+  s.fkey = reinterpret_cast<double*>(s.fin + kFinal);
+  s.pk = reinterpret_cast<uint2*>(s.fkey + kFinal);
+  s.top = s.pk + 2 * 2 * SW;
+  s.rinfo = s.top + 16;
   s.cnt = misc;
   c.rank = cluster_ctarank();
   c.nrank = cluster_nctarank();
   c.parity = 0;
+  if (c.nrank > 1) cluster_arrive_relaxed();          // waited for before the first access to a peer's shared memory
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int idx = blockIdx.x / c.nrank;
-  const int b = idx % a.B;
-  const int n = a.order[a.order_begin + idx / a.B];
-  const int fc = a.first_child[n], nc = a.n_child[n];
+  const int b = idx % a.B, slot = idx / a.B;
+  // few parents travel with the launch: no chain of reads in front of the row's first load
+  const int n = a.inlined ? a.p_node[slot] : a.order[a.order_begin + slot];
+  const int fc = a.inlined ? a.p_child[slot] : a.first_child[n], nc = a.inlined ? a.p_count[slot] : a.n_child[n];
   const long long row_off = static_cast<long long>(b) * a.seq_stride + static_cast<long long>(n) * a.row_stride;
   const long long out_b = static_cast<long long>(b) * a.N;
   const uint32_t row_id = static_cast<uint32_t>(out_b + n);
@@ -195,17 +203,13 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
   if (tid == 0) *s.cnt = 0;
   __syncthreads();
 
-  // Uniforms of tokens j .. j+VN-1 (j a multiple of VN); returns whether one of them exceeds 0.999.
-  // Philox words become floats without an integer conversion: the 23 mantissa bits under the
-  // exponent of 1.0 give 1 + i 2^-23, and subtracting 1 - 2^-24 leaves (i + 1/2) 2^-23 exactly.
-  auto uniforms = [&](int j, float (&U)[VN]) -> bool {
-    bool near_one = false;
+  // 1 + U of tokens j .. j+VN-1 (j a multiple of VN).  Philox words become floats without an integer
+  // conversion: the 23 mantissa bits under the exponent of 1.0 give F = 1 + i 2^-23, and subtracting
+  // 1 - 2^-24 leaves U = (i + 1/2) 2^-23 exactly.
+  auto words = [&](int j, float (&F)[VN]) {
     if (gum) {
 #pragma unroll
-      for (int e = 0; e < VN; ++e) {
-        U[e] = (j + e < a.V) ? __ldcs(gum + j + e) : 0.5f;
-        near_one |= U[e] > 0.999f;
-      }
+      for (int e = 0; e < VN; ++e) F[e] = 1.f + ((j + e < a.V) ? __ldcs(gum + j + e) : 0.5f);
     } else {
 #pragma unroll
       for (int q = 0; q < VN / 4; ++q) {
@@ -213,12 +217,26 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
                                              (static_cast<uint32_t>(a.step >> 32) << 2) | kStreamGumbel, a.rk0, a.rk1);
         const uint32_t w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          U[4 * q + e] = __uint_as_float(0x3f800000u | (w[e] >> 9)) - 0.99999994f;
-        near_one |= (max(max(r.x, r.y), max(r.z, r.w)) >> 9) > 8380219u;       // 0.999 * 2^23
+        for (int e = 0; e < 4; ++e) F[4 * q + e] = __uint_as_float(__funnelshift_r(w[e], 0x7fu, 9));
       }
     }
-    return near_one;
+  };
+  auto uniform_at = [&](int t) -> float {
+    if (gum) return __ldcs(gum + t);
+    const Philox4 r = philox4x32_10_keys(static_cast<uint32_t>(t >> 2), row_id, static_cast<uint32_t>(a.step),
+                                         (static_cast<uint32_t>(a.step >> 32) << 2) | kStreamGumbel, a.rk0, a.rk1);
+    return uniform_open((t & 3) == 0 ? r.x : ((t & 3) == 1 ? r.y : ((t & 3) == 2 ? r.z : r.w)));
+  };
+  // Cut of the list to its R best entries; entries from `raw` on still hold z in the place of their key.
+  auto cut = [&](int raw, float T) -> float {
+    const int n = min(*s.cnt, kListCap);
+    for (int i = raw + tid; i < n; i += ST) {
+      const uint2 en = s.list[i];
+      const float U = uniform_at(static_cast<int>(en.y)), z = __uint_as_float(en.x);
+      s.list[i].x = __float_as_uint(U > 0.999f ? careful_key(z, U) : fast_key(z, U));
+    }
+    __syncthreads();
+    return n <= ST ? cut_ranked(s, R, T) : cut_list(s, R, T);
   };
 
   // One entry for the list (appends are rare after the first cut: a shared-memory atomic each)
@@ -234,18 +252,20 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
   // row is redone with a check after every chunk.
   float Tk = -INFINITY;                               // every element left out has key <= Tk
   float mx = -INFINITY, sx = 0.f;
+  int raw = kListCap;                                 // list entries from here on have no key yet
   const int iters = (ge.vw + 32 * UV - 1) / (32 * UV);
   const int cut_it = max(1, iters / 3);                // the one scheduled cut of the optimistic pass
   for (int mode = 0; mode < 2; ++mode) {
     Tk = -INFINITY;
     mx = -INFINITY;
     sx = 0.f;
-    for (int it = 0; it < iters; ++it) {
-      const int base = vbeg + it * 32 * UV;
+    raw = kListCap;
+    // ---- first chunk
+    {
       uint4 rc[UV], ru[UV];
 #pragma unroll
       for (int u = 0; u < UV; ++u) {
-        const int vv = base + 32 * u + lane;
+        const int vv = vbeg + 32 * u + lane;
         if (vv < vend && vv >= ge.vi0 && vv < ge.vi1) io.load(vv, rc[u], ru[u]);
       }
       float first[UV][VN];                              // keys of the first chunk
@@ -253,88 +273,154 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
       int tbj = 0x7fffffff;
 #pragma unroll
       for (int u = 0; u < UV; ++u) {
-        const int vv = base + 32 * u + lane;
-        const bool active = vv < vend;
+        const int vv = vbeg + 32 * u + lane;
         const int j = ge.j0 + vv * VN;
-        float z[VN], key[VN];
+        float z[VN];
 #pragma unroll
-        for (int e = 0; e < VN; ++e) key[e] = -INFINITY;
-        if (active) {
+        for (int e = 0; e < VN; ++e) first[u][e] = -INFINITY;
+        if (vv < vend) {
           if (vv >= ge.vi0 && vv < ge.vi1) {
             io.z(rc[u], ru[u], z);
           } else {                                      // ragged first / last vector of the row
 #pragma unroll
             for (int e = 0; e < VN; ++e) z[e] = (j + e >= ge.alo && j + e < ge.ahi) ? io.z_at(j + e) : -INFINITY;
           }
-          float U[VN];
-          const bool near_one = uniforms(j, U);
+          float F[VN];
+          words(j, F);
+          bool near_one = false;
 #pragma unroll
-          for (int e = 0; e < VN; ++e) key[e] = fast_key(z[e], U[e]);
+          for (int e = 0; e < VN; ++e) {
+            const float U = F[e] - (gum ? 1.f : 0.99999994f);
+            first[u][e] = fast_key(z[e], U);
+            near_one |= U > 0.999f;
+          }
           if (near_one) {                               // rare: one vector in a hundred
 #pragma unroll
             for (int e = 0; e < VN; ++e)
-              if (U[e] > 0.999f) key[e] = careful_key(z[e], U[e]);
+              if (F[e] > 1.998f) first[u][e] = careful_key(z[e], gum ? __ldcs(gum + j + e) : F[e] - 0.99999994f);
           }
           if (want_prob) acc_exp<VN>(z, mx, sx);
         }
-        if (it == 0) {
+#pragma unroll
+        for (int e = 0; e < VN; ++e)
+          if (key_before(first[u][e], j + e, tbk, tbj)) { tbk = first[u][e]; tbj = j + e; }
+      }
+      // the two best of every warp's thread-bests: 2 * SW keys of distinct tokens, whose R-th best is a
+      // lower bound of the row's R-th best key (R <= 12 <= 2 * SW); every warp ranks them for itself
+      float k1 = tbk, k2;
+      int j1 = tbj, j2;
+      warp_key_first(k1, j1);
+      k2 = (tbj == j1) ? -INFINITY : tbk;
+      j2 = (tbj == j1) ? 0x7fffffff : tbj;
+      warp_key_first(k2, j2);
+      if (lane == 0) {
+        s.pk[2 * warp] = make_uint2(__float_as_uint(k1), static_cast<uint32_t>(j1));
+        s.pk[2 * warp + 1] = make_uint2(__float_as_uint(k2), static_cast<uint32_t>(j2));
+      }
+      __syncthreads();
+      {
+        const uint2 en = s.pk[lane & (2 * SW - 1)];
+        const float mk = __uint_as_float(en.x);
+        const int mt = static_cast<int>(en.y);
+        int rank = 0;
+#pragma unroll
+        for (int i = 0; i < 2 * SW; ++i) {
+          const float ok = __shfl_sync(0xffffffffu, mk, i);
+          const int ot = __shfl_sync(0xffffffffu, mt, i);
+          rank += key_before(ok, ot, mk, mt) ? 1 : 0;
+        }
+        const uint32_t hit = __ballot_sync(0xffffffffu, lane < 2 * SW && rank == R - 1 && mt != 0x7fffffff && mk > -INFINITY);
+        if (hit) Tk = __shfl_sync(0xffffffffu, mk, __ffs(hit) - 1);
+      }
+      // (the key at the threshold itself belongs to the R best: >=, so that the first cut finds R entries)
+#pragma unroll
+      for (int u = 0; u < UV; ++u) {
+        const int j = ge.j0 + (vbeg + 32 * u + lane) * VN;
+#pragma unroll
+        for (int e = 0; e < VN; ++e)
+          if (first[u][e] >= Tk && first[u][e] > -INFINITY) append(first[u][e], j + e);
+      }
+    }
+    if (iters > 1) {
+      __syncthreads();
+      raw = min(*s.cnt, kListCap);
+      __syncthreads();                                  // everyone has read the count before it moves again
+      if (mode == 1 && raw > kListCap - kIterElems) {
+        Tk = cut(raw, Tk);
+        raw = R;
+      }
+    }
+    // ---- the other chunks: an element passes when 1 + U > 2 - e^(z - Tk), with room for the roundings of
+    // z L - Tk L (2^-24 of either), of the exponential (2^-22 relative) and of the two sides (2^-24 each)
+    auto cutoff = [](float T) { return fmaf(-(T - kKeyShift), kLog2e, fmaf(fabsf(T), 1e-6f, 4e-5f)); };
+    float c0 = cutoff(Tk);
+    constexpr float kPass = 1.9999995f;
+    for (int it = 1; it < iters; ++it) {
+      const int base = vbeg + it * 32 * UV;
+      uint4 rc[UV], ru[UV];
+      if (base >= ge.vi0 && base + 32 * UV <= min(vend, ge.vi1)) {
+        // whole vectors only (the same decision in every lane): no branch between the vectors, so that their
+        // generator rounds interleave and share the round keys
+        float F[UV][VN];
+#pragma unroll
+        for (int u = 0; u < UV; ++u) io.load(base + 32 * u + lane, rc[u], ru[u]);
+#pragma unroll
+        for (int u = 0; u < UV; ++u) words(ge.j0 + (base + 32 * u + lane) * VN, F[u]);
+        bool any = false;
+#pragma unroll
+        for (int u = 0; u < UV; ++u) {
+          float z[VN];
+          io.z(rc[u], ru[u], z);
 #pragma unroll
           for (int e = 0; e < VN; ++e) {
-            first[u][e] = key[e];
-            if (key_before(key[e], j + e, tbk, tbj)) { tbk = key[e]; tbj = j + e; }
+            F[u][e] += ex2_approx(fmaf(z[e], kLog2e, c0));
+            any |= F[u][e] > kPass;
           }
-        } else {
-          float best = key[0];
+          if (want_prob) acc_exp<VN>(z, mx, sx);
+        }
+        if (any) {                                      // rare, and rarer after the cut
 #pragma unroll
-          for (int e = 1; e < VN; ++e) best = fmaxf(best, key[e]);
-          if (best > Tk) {                              // rare, and rarer after every cut
+          for (int u = 0; u < UV; ++u) {
+            float z[VN];
+            io.z(rc[u], ru[u], z);
 #pragma unroll
             for (int e = 0; e < VN; ++e)
-              if (key[e] > Tk) append(key[e], j + e);
+              if (F[u][e] > kPass && z[e] > -INFINITY) append(z[e], ge.j0 + (base + 32 * u + lane) * VN + e);
+          }
+        }
+      } else {
+#pragma unroll 1
+        for (int u = 0; u < UV; ++u) {
+          const int vv = base + 32 * u + lane;
+          const int j = ge.j0 + vv * VN;
+          if (vv < vend) {
+            float z[VN], F[VN];
+            if (vv >= ge.vi0 && vv < ge.vi1) {
+              io.load(vv, rc[0], ru[0]);
+              io.z(rc[0], ru[0], z);
+            } else {                                    // ragged first / last vector of the row
+#pragma unroll
+              for (int e = 0; e < VN; ++e) z[e] = (j + e >= ge.alo && j + e < ge.ahi) ? io.z_at(j + e) : -INFINITY;
+            }
+            words(j, F);
+#pragma unroll
+            for (int e = 0; e < VN; ++e)
+              if (F[e] + ex2_approx(fmaf(z[e], kLog2e, c0)) > kPass && z[e] > -INFINITY) append(z[e], j + e);
+            if (want_prob) acc_exp<VN>(z, mx, sx);
           }
         }
       }
-      if (it == 0) {
-        // the two best of every warp's thread-bests: 2 * SW keys of distinct tokens, whose R-th best is a
-        // lower bound of the row's R-th best key (R <= 12 <= 2 * SW); every warp ranks them for itself
-        float k1 = tbk, k2;
-        int j1 = tbj, j2;
-        warp_key_first(k1, j1);
-        k2 = (tbj == j1) ? -INFINITY : tbk;
-        j2 = (tbj == j1) ? 0x7fffffff : tbj;
-        warp_key_first(k2, j2);
-        if (lane == 0) {
-          s.pk[2 * warp] = make_uint2(__float_as_uint(k1), static_cast<uint32_t>(j1));
-          s.pk[2 * warp + 1] = make_uint2(__float_as_uint(k2), static_cast<uint32_t>(j2));
-        }
-        __syncthreads();
-        {
-          const uint2 en = s.pk[lane & (2 * SW - 1)];
-          const float mk = __uint_as_float(en.x);
-          const int mt = static_cast<int>(en.y);
-          int rank = 0;
-#pragma unroll
-          for (int i = 0; i < 2 * SW; ++i) {
-            const float ok = __shfl_sync(0xffffffffu, mk, i);
-            const int ot = __shfl_sync(0xffffffffu, mt, i);
-            rank += key_before(ok, ot, mk, mt) ? 1 : 0;
-          }
-          const uint32_t hit = __ballot_sync(0xffffffffu, lane < 2 * SW && rank == R - 1 && mt != 0x7fffffff && mk > -INFINITY);
-          if (hit) Tk = __shfl_sync(0xffffffffu, mk, __ffs(hit) - 1);
-        }
-#pragma unroll
-        for (int u = 0; u < UV; ++u) {
-          const int j = ge.j0 + (base + 32 * u + lane) * VN;
-#pragma unroll
-          for (int e = 0; e < VN; ++e)
-            if (first[u][e] > Tk) append(first[u][e], j + e);
-        }
-      } else if (it == cut_it || mode == 1) {
+      if (it == cut_it || mode == 1) {
         __syncthreads();
         const int cn = *s.cnt;
-        const bool do_cut = mode == 1 ? cn > kListCap - kIterElems : cn > R;
         __syncthreads();                                // everyone has read the count before it moves again
-        if (do_cut) Tk = cn <= 1024 ? cut_small(s, R, Tk) : cut_list(s, R, Tk);
+        if (mode == 1 ? cn > kListCap - kIterElems : cn > R) {
+          if (cn <= kListCap) {                         // (an overflowing list is redone anyway)
+            Tk = cut(raw, Tk);
+            raw = min(cn, R);
+            c0 = cutoff(Tk);
+          }
+        }
       }
     }
     __syncthreads();
@@ -344,6 +430,7 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
     if (tid == 0) *s.cnt = 0;
     __syncthreads();
   }
+  if (c.nrank > 1) cluster_wait();                      // every CTA of the row has started
 
   // ---- softmax denominator of the row (for draft_prob)
   float gm[1] = {0.f}, gs[1] = {0.f};
@@ -355,61 +442,79 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
     combine<1, false>(c, gs);
   }
 
-  // ---- candidates of all CTAs of the row -> CTA 0, exact keys, ranking
-  __syncthreads();
-  const int share = kFinal / static_cast<int>(c.nrank);
-  if (*s.cnt > share) { __syncthreads(); Tk = cut_list(s, min(R, share), Tk); }
-  float tmax[1] = {warp_max(Tk)};
-  combine<1, true>(c, tmax);                          // its barriers also publish the lists
-  if (c.rank == 0) {
-    int nf = 0;
+  // ---- every CTA's R best entries in order; those of all CTAs of the row go to CTA 0
+  Tk = cut(raw, Tk);
+  const int mine = *s.cnt;
+  const uint2* fin = s.list;
+  int nf = mine;
+  float tmax = Tk;
+  if (c.nrank > 1) {
+    if (tid < mine) dsmem_st_u64(dsmem_addr(smem_u32(&s.fin[c.rank * kMaxR + tid]), 0), s.list[tid]);
+    if (tid == 0)
+      dsmem_st_u64(dsmem_addr(smem_u32(&s.rinfo[c.rank]), 0), make_uint2(static_cast<uint32_t>(mine), __float_as_uint(Tk)));
+    cluster_sync();
+    if (c.rank != 0) return;
+    // CTA 0: every entry's place among all of them
+    nf = 0;
     for (uint32_t r = 0; r < c.nrank; ++r) {
-      const uint32_t cnt_r = c.nrank > 1 ? dsmem_ld_u32(dsmem_addr(smem_u32(s.cnt), r)) : static_cast<uint32_t>(*s.cnt);
-      const int m = min(static_cast<int>(cnt_r), share);
-      if (tid < m) {
-        uint32_t tokv;
-        if (c.nrank > 1) tokv = dsmem_ld_u32(dsmem_addr(smem_u32(&s.list[tid]) + 4u, r));
-        else tokv = s.list[tid].y;
-        const int t = static_cast<int>(tokv);
-        float U;
-        if (gum) {
-          U = __ldcs(gum + t);
-        } else {
-          const Philox4 rr = philox_stream(a.seed, a.step, row_id, kStreamGumbel, static_cast<uint32_t>(t >> 2));
-          const uint32_t wv = (t & 3) == 0 ? rr.x : ((t & 3) == 1 ? rr.y : ((t & 3) == 2 ? rr.z : rr.w));
-          U = uniform_open(wv);
+      nf += static_cast<int>(s.rinfo[r].x);
+      tmax = fmaxf(tmax, __uint_as_float(s.rinfo[r].y));
+    }
+    const int r_own = tid / kMaxR, i_own = tid - r_own * kMaxR;
+    if (r_own < static_cast<int>(c.nrank) && i_own < static_cast<int>(s.rinfo[r_own].x)) {
+      const uint2 en = s.fin[tid];
+      int rank = i_own;                                  // the CTAs' lists are in order
+      for (uint32_t r = 0; r < c.nrank; ++r) {
+        if (static_cast<int>(r) == r_own) continue;
+        const int m = static_cast<int>(s.rinfo[r].x);
+#pragma unroll
+        for (int i = 0; i < kMaxR; ++i) {
+          const uint2 o = s.fin[r * kMaxR + i];
+          rank += (i < m && key_before(__uint_as_float(o.x), static_cast<int>(o.y), __uint_as_float(en.x), static_cast<int>(en.y))) ? 1 : 0;
         }
-        const float zt = io.z_at(t);
-        s.fkey[nf + tid] = static_cast<double>(zt) - log(-log(static_cast<double>(U)));
-        s.ftok[nf + tid] = t;
       }
-      nf += m;
+      s.list[rank] = en;                                 // (this CTA's own list has been copied to s.fin)
     }
     __syncthreads();
-    if (tid < nf) {
+  }
+  // ---- exact order: float32 keys decide unless two neighbours in the order, or the last child and the
+  // elements left out, are closer than the keys' errors
+  bool near = false;
+  if (tid < nf && tid < nc) {
+    const float k = __uint_as_float(fin[tid].x);
+    if (tid + 1 < nf) near = k - __uint_as_float(fin[tid + 1].x) <= 2.f * kKeyEps;
+    if (tid == nc - 1) near |= k - tmax <= 2.f * kKeyEps;
+  }
+  const bool exact = __syncthreads_or(near ? 1 : 0) != 0;
+  if (exact && tid < nf)
+    s.fkey[tid] = static_cast<double>(io.z_at(static_cast<int>(fin[tid].y))) -
+                  log(-log(static_cast<double>(uniform_at(static_cast<int>(fin[tid].y)))));
+  if (exact) __syncthreads();
+  if (tid < nf) {
+    const int t = static_cast<int>(fin[tid].y);
+    int rank = tid;
+    if (exact) {
       const double k = s.fkey[tid];
-      const int t = s.ftok[tid];
-      int rank = 0;
+      rank = 0;
       for (int i = 0; i < nf; ++i) {
         const double ki = s.fkey[i];
-        rank += (ki > k || (ki == k && s.ftok[i] < t)) ? 1 : 0;
+        rank += (ki > k || (ki == k && static_cast<int>(fin[i].y) < t)) ? 1 : 0;
       }
-      if (rank < nc) {
-        a.tokens[out_b + fc + rank] = t;
-        if (want_prob) {
-          const float zt = io.z_at(t);
-          a.draft_prob[out_b + fc + rank] = gs[0] > 0.f ? ex2_approx(fmaf(zt, kLog2e, -gm[0] * kLog2e)) / gs[0] : 0.f;
-        }
-        if (rank == nc - 1 && static_cast<double>(tmax[0]) + kKeyEps >= k) vflag(a.status, LANTERN_DEV_KEY_TIES);
+      if (rank == nc - 1 && static_cast<double>(tmax) + kKeyEps >= k + kKeyShift) vflag(a.status, LANTERN_DEV_KEY_TIES);
+    }
+    if (rank < nc) {
+      a.tokens[out_b + fc + rank] = t;
+      if (want_prob) {
+        const float zt = io.z_at(t);
+        a.draft_prob[out_b + fc + rank] = gs[0] > 0.f ? ex2_approx(fmaf(zt, kLog2e, -gm[0] * kLog2e)) / gs[0] : 0.f;
       }
     }
-    if (tid >= nf && tid < nc) {                      // fewer than s tokens with positive probability
-      a.tokens[out_b + fc + tid] = -1;
-      if (want_prob) a.draft_prob[out_b + fc + tid] = 0.f;
-    }
-    if (nf == 0 && tid == 0) vflag(a.status, LANTERN_DEV_EMPTY_ROW);
   }
-  if (c.nrank > 1) cluster_sync();                    // CTA 0 may still be reading this CTA's list
+  if (tid >= nf && tid < nc) {                        // fewer than s tokens with positive probability
+    a.tokens[out_b + fc + tid] = -1;
+    if (want_prob) a.draft_prob[out_b + fc + tid] = 0.f;
+  }
+  if (nf == 0 && tid == 0) vflag(a.status, LANTERN_DEV_EMPTY_ROW);
 }
 
 }  // namespace stream

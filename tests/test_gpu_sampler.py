@@ -199,3 +199,45 @@ def test_streaming_kernel_on_monotone_and_constant_rows(L, shape):
     gum = W.make_gumbel_uniforms(case.B, case.N, V, 99)
     gtok, gprob, _ = _gpu_sample(L, case, gumbel=gum)
     assert _compare(case, gum.numpy(), gtok, gprob) <= 1
+
+
+@pytest.mark.parametrize("kw", [dict(vocab=4096, codebook_size=512), dict(vocab=4099, codebook_size=512, cfg_scale=None),
+                                dict(vocab=16384, codebook_size=512, batch=1, parent=[-1, 0]),
+                                dict(vocab=20011, codebook_size=512, dtype="bf16"),
+                                dict(vocab=65536, codebook_size=512, dtype="bf16", batch=1, parent=[-1, 0, 0, 0, 1], allowed=(4097, 12290)),
+                                dict(vocab=33000, codebook_size=512, batch=1, parent=[-1, 0, 0, 0, 1], allowed=(32990, 33000))])
+@pytest.mark.parametrize("philox", [False, True])
+def test_small_calls_on_the_streaming_kernel(L, kw, philox):
+    """What the library picks by itself for a handful of parents: rows that are one chunk per CTA and rows of several,
+    clusters of up to eight CTAs, allowed ranges that no vector divides and one narrower than a vector per warp."""
+    kw = dict(kw)
+    allowed, parent = kw.pop("allowed", (0, 0)), kw.pop("parent", None)
+    V = kw["vocab"]
+    case = Case(small_config(**kw), parent=parent, seed=31, tokens="random", allowed=allowed, kernels=0, pad=-V % 8)
+    if philox:
+        seed, step = 0xBEEF, 5
+        gum = np.empty((case.B, case.N, V), dtype=np.float32)
+        for b in range(case.B):
+            for n in range(case.N):
+                gum[b, n] = oracle.stream_uniforms(seed, step, b * case.N + n, 0, count=V)
+        gtok, gprob, _ = _gpu_sample(L, case, seed_step=(seed, step))
+    else:
+        gum = W.make_gumbel_uniforms(case.B, case.N, V, 4242).numpy()
+        gtok, gprob, _ = _gpu_sample(L, case, gumbel=torch.from_numpy(gum))
+    assert _compare(case, gum, gtok, gprob) <= 1
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_streaming_kernel_on_wide_ranges_and_nearly_empty_rows(L, dtype):
+    """Logits from -250 to 250 (the exponential of the elements' test overflows and vanishes), and rows of which all
+    but two elements are -inf: fewer candidates than children."""
+    case = Case(small_config(batch=2, vocab=20000, codebook_size=512, dtype=dtype, cfg_scale=None), seed=41, tokens="random", kernels=1)
+    rows = case.padded["draft_cond"]
+    g = torch.Generator().manual_seed(6)
+    rows[0] = ((torch.rand(rows[0].shape, generator=g) * 500.0) - 250.0).to(rows.dtype)
+    rows[1] = -float("inf")
+    rows[1, :, 17] = 1.0
+    rows[1, :, 19999] = 0.5
+    gum = W.make_gumbel_uniforms(case.B, case.N, case.V, 7)
+    gtok, gprob, _ = _gpu_sample(L, case, gumbel=gum)
+    assert _compare(case, gum.numpy(), gtok, gprob) <= 1
