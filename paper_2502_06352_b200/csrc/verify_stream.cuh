@@ -206,7 +206,9 @@ struct StreamSmem {
   float* scan;      // [SW]
   int* misc;        // [32]
   uint32_t* memb;   // [33] greedy-skip rule: bit r = entry r of the neighbour list joined A
+  unsigned long long* wex;   // [kMaxCluster*SW + 1] deterministic drafts: banned mass per warp range and in total
 };
+constexpr float kMassUnits = 1099511627776.f;         // 2^40: banned mass is added in integers, so the order does not matter
 
 // term of every token of vector vv under the current target (exception and masked tokens: 0)
 template <typename IO>
@@ -374,6 +376,8 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
     const int words = (a.V + 31) / 32;
     for (int i = tid; i < words; i += ST) sm.bits[i] = 0u;
   }
+  if (det)
+    for (int i = tid; i < kMaxCluster * SW + 1; i += ST) sm.wex[i] = 0ull;
   if (tid == 32) {
     fm[7] = a.u_res ? a.u_res[out_b + n]
                     : uniform_halfopen(philox_stream(a.seed, a.step, static_cast<uint32_t>(out_b + n), kStreamResample, 0).x);
@@ -579,6 +583,22 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
   float alpha = 0.f, beta = 1.f, ibeta = 1.f, W = 1.f, iW = 1.f;
   int n_dropped = 0;
   int accepted = -1;
+  // Deterministic drafts: the residual after a rejection is q_0 without the banned tokens, so its sum
+  // is the last sum taken over the row less the banned mass, no pass over the row.  It is summed afresh
+  // once half of that sum is gone: until then the subtraction loses at most one bit.
+  // (sums below 1e-20 are always taken afresh: their inverse must stay a float32.)
+  float bsum = 1.f, wscale = rq;           // the sum the banned mass is taken from; sm.wpart * wscale is in its units
+  float unit = 1.f / kMassUnits;           // of sm.wex: bsum 2^-40
+  bool banned = false;
+  auto ban = [&](int t, float q0) {
+    const uint32_t bit = 1u << (t & 31);
+    const uint32_t old = atomicOr(&sm.bits[t >> 5], bit);
+    if (det && !(old & bit) && t >= ge.alo && t < ge.ahi) {
+      const unsigned long long units = static_cast<unsigned long long>(q0 / unit);
+      atomicAdd(&sm.wex[(t - ge.j0) / VN / ge.vw], units);
+      atomicAdd(&sm.wex[kMaxCluster * SW], units);
+    }
+  };
   for (int ci = 0; ci < nc; ++ci) {
     const int child = fc + ci;
     const int x = ctok[ci];
@@ -707,21 +727,32 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
       if (has_code) {
         for (int r = tid; r < a.k; r += ST) {
           const int t = tk[1 + r];
-          if (t >= 0 && ((sm.memb[r >> 5] >> (r & 31)) & 1u)) atomicOr(&sm.bits[t >> 5], 1u << (t & 31));
+          if (t >= 0 && ((sm.memb[r >> 5] >> (r & 31)) & 1u)) ban(t, en[(1 + r) * NOPS]);
         }
       }
     } else {
       for (int r = tid; r < nA; r += ST) {
         const int t = tk[1 + r];
-        if (t >= 0) atomicOr(&sm.bits[t >> 5], 1u << (t & 31));
+        if (t >= 0) ban(t, en[(1 + r) * NOPS]);
       }
     }
     if (tid == 0) {
-      atomicOr(&sm.bits[x >> 5], 1u << (x & 31));
+      ban(x, en[0]);
       if (!x_dropped) dropped[n_dropped] = x;
     }
     if (!x_dropped) ++n_dropped;
     __syncthreads();
+    if (det) {
+      const float left = bsum - static_cast<float>(sm.wex[kMaxCluster * SW]) * unit;
+      if (left > 0.5f * bsum && bsum > 1e-20f) {
+        beta = left;
+        ibeta = 1.f / left;
+        cur.aq = rq;
+        banned = true;
+        __syncthreads();
+        continue;
+      }
+    }
     const float alpha_n = fmaf(beta, iW, alpha);
     Cur nx;
     nx.cq = cur.cq; nx.cp = cur.cp; nx.aq = rq; nx.ap = det ? 0.f : alpha_n * rp; nx.has_p = !det;
@@ -747,6 +778,13 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
         if (lane < SW) sm.wpart[lane] = sm.wtmp[lane];
         if (lane < static_cast<int>(c.nrank)) sm.rtot[lane] = c.gath[lane * 2];
       }
+      if (det) {                             // (every thread has read the banned mass before the combination)
+        for (int i = tid; i < kMaxCluster * SW + 1; i += ST) sm.wex[i] = 0ull;
+        bsum = beta;
+        unit = fmaxf(beta, 1e-20f) / kMassUnits;
+        wscale = 1.f;
+        banned = false;
+      }
     }
     // (beta_{r+1} = 0 cannot follow a rejection in exact arithmetic unless m = 0 and the rows
     // coincide; the target then stays as it is)
@@ -758,6 +796,16 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
   // token order: CTA totals locate the CTA, per-warp sums the warp, whose range is then re-read.
   if (accepted < 0) {
     __syncthreads();
+    if (det && banned) {                     // the ranges' sums without the tokens banned since they were taken
+      if (tid < static_cast<int>(c.nrank)) {
+        unsigned long long gone = 0ull;
+        for (int w2 = 0; w2 < SW; ++w2) gone += sm.wex[tid * SW + w2];
+        sm.rtot[tid] = fmaxf(sm.rtot[tid] * wscale - static_cast<float>(gone) * unit, 0.f);
+      }
+      if (tid < SW)
+        sm.wpart[tid] = fmaxf(sm.wpart[tid] * wscale - static_cast<float>(sm.wex[c.rank * SW + tid]) * unit, 0.f);
+      __syncthreads();
+    }
     const float u = fm[7];
     float total = 0.f;
     for (uint32_t r = 0; r < c.nrank; ++r) total += sm.rtot[r];
@@ -873,7 +921,9 @@ __global__ void __launch_bounds__(ST, LANTERN_STREAM_MINB) verify_stream_kernel(
   sm.scan = sm.rtot + kMaxCluster;     // SW
   sm.misc = reinterpret_cast<int*>(sm.scan + SW);      // 32
   sm.memb = reinterpret_cast<uint32_t*>(sm.misc + 32); // 33
-  static_assert((2 * SW * 4 + 8 + kMaxCluster * 4 + SW + SW + kMaxCluster + SW + 32 + 33) * 4 <= kSmallBytes, "small area");
+  constexpr int kSmallInts = (2 * SW * 4 + 8 + kMaxCluster * 4 + SW + SW + kMaxCluster + SW + 32 + 33 + 1) / 2 * 2;
+  sm.wex = reinterpret_cast<unsigned long long*>(small + kSmallInts);
+  static_assert(kSmallInts * 4 + (kMaxCluster * SW + 1) * 8 <= kSmallBytes, "small area");
   sm.bits = reinterpret_cast<uint32_t*>(stream_smem + kSmallBytes);
   sm.ent = reinterpret_cast<float*>(sm.bits + (a.V + 127) / 128 * 4);
   sm.tok = reinterpret_cast<int*>(sm.ent + static_cast<size_t>(a.max_children) * kp1 * NOPS);

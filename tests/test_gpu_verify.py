@@ -387,6 +387,39 @@ def test_deterministic_draft_mode(L, cs, kw):
         L.set_cluster_size(old)
 
 
+@pytest.mark.parametrize("cs", [0, 1, 4, 16])
+@pytest.mark.parametrize("kw", [dict(logit_std=6.0, k=24), dict(logit_std=1.0, k=40, lam=6.0, dtype="bf16", cfg_scale=None),
+                                dict(vocab=5003, codebook_size=5003, logit_std=9.0, k=12, cfg_scale=None),
+                                dict(logit_std=5.0, k=30, skip=True)])
+def test_deterministic_drafts_that_are_all_rejected(L, cs, kw):
+    """The residual's sum comes from the banned mass while at least half of the last sum is left and is taken
+    afresh below that: flat rows never need a pass, peaked ones do after nearly every child; the draw of every
+    node is from a residual."""
+    kw = dict(kw)
+    skip = kw.pop("skip", False)
+    old = L.set_cluster_size(cs)
+    try:
+        case = Case(small_config(n_nodes=60, **kw), seed=47, det_draft=True, skip=skip, pad=5 if "vocab" in kw else 0)
+        case.u_accept = torch.full_like(case.u_accept, 1.0 - 2.0 ** -24)
+        _run_det(L, case)
+    finally:
+        L.set_cluster_size(old)
+
+
+def _run_det(L, case):
+    g, par, nbr, tok = case.gpu_inputs(L)
+    tree = L.Tree(case.parent)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = L.verify_tree(par, tree, nbr, g["target_cond"], g["target_uncond"], None, None, tok,
+                        case.u_accept.cuda(), case.u_resample.cuda(), debug=True, device_status=status)
+    torch.cuda.synchronize()
+    res = {k: v.cpu().numpy() for k, v in out.items()}
+    assert int(status.item()) == 0
+    orc = case.oracle_verify()
+    stats = compare_verify(res, orc, case.parent, case.u_accept.numpy(), case.seqs, rerun=case.oracle_node)
+    check_walk(res, case.tokens, tree.max_depth, orc, stats["dirty_sequences"], case.seqs, stats["patched"])
+
+
 def test_path_walk_with_a_rule_variant_runs_on_the_streaming_kernel(L):
     case = Case(small_config(k=24, lam=1.8, batch=4, n_nodes=60), seed=45, skip=True)
     g, par, nbr, tok = case.gpu_inputs(L)
