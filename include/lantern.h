@@ -80,6 +80,15 @@ int32_t lantern_tree_max_depth(const lantern_tree* tree);  /* depth of the deepe
  * draft_deterministic = 1).  Destroyed with lantern_tree_destroy.                               */
 lantern_status lantern_forest_create(const int32_t* parent /* host */, const int32_t* n_nodes /* host */,
                                      int32_t batch, int32_t max_nodes, lantern_tree** out);
+/* The same with the handle's device arrays in memory of the caller (a decode loop makes a forest per
+ * step, and allocating and freeing device memory stops the whole GPU each time): `block`, at least
+ * lantern_forest_block() bytes, 16-byte aligned, is filled on `stream` before the call returns (not
+ * inside a stream capture: LANTERN_ERR_CUDA).  It must stay valid for as long as work that uses the
+ * handle is pending, on whatever stream; lantern_tree_destroy does not free it and does not wait. */
+size_t lantern_forest_block(int32_t batch, int32_t max_nodes);
+lantern_status lantern_forest_create_in(const int32_t* parent /* host */, const int32_t* n_nodes /* host */,
+                                        int32_t batch, int32_t max_nodes, void* block, size_t block_bytes,
+                                        void* stream, lantern_tree** out);
 
 /* ---- parameters (App. B "Models": guidance, temperature, top-k; Sec. 4: k, lambda) ---------
  * Row post-processing, identical for target rows (-> q) and drafter rows (-> p):

@@ -3,7 +3,9 @@
 Tensors are torch CUDA tensors (PyTorch supplies device memory and streams);
 pointers, strides and the current stream are handed to the C ABI.
 """
+import array
 import ctypes
+import itertools
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -77,6 +79,10 @@ def _load():
     L.lantern_tree_create.argtypes = [vp, i32, ctypes.POINTER(vp)]
     L.lantern_forest_create.restype = ctypes.c_int
     L.lantern_forest_create.argtypes = [vp, vp, i32, i32, ctypes.POINTER(vp)]
+    L.lantern_forest_block.restype = sz
+    L.lantern_forest_block.argtypes = [i32, i32]
+    L.lantern_forest_create_in.restype = ctypes.c_int
+    L.lantern_forest_create_in.argtypes = [vp, vp, i32, i32, vp, sz, vp, ctypes.POINTER(vp)]
     L.lantern_tree_destroy.restype = ctypes.c_int
     L.lantern_tree_destroy.argtypes = [vp]
     L.lantern_tree_max_depth.restype = i32
@@ -126,11 +132,25 @@ def _check(status, where):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+# Current device and raw stream handle without building device and stream objects: those took a
+# quarter of the host time of a call.
+_current_device = torch._C._cuda_getDevice
+_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
+def _call(fn, where, t, *args):
+    """fn(*args, current stream of t's GPU) with that GPU current."""
+    dev = t.get_device()
+    if dev < 0:
+        raise ValueError("expected CUDA tensors")
+    if dev == _current_device():
+        _check(fn(*args, _raw_stream(dev)), where)
+    else:
+        with torch.cuda.device(dev):
+            _check(fn(*args, _raw_stream(dev)), where)
 
 
 def _dtype_code(t):
@@ -153,6 +173,9 @@ class Tree:
         self.handle = h
         self.max_depth = lib.lantern_tree_max_depth(h)
 
+    def used_by(self, t):
+        pass
+
     def __del__(self):
         h = getattr(self, "handle", None)
         if h is not None and lib is not None:
@@ -160,30 +183,65 @@ class Tree:
             self.handle = None
 
 
+def _flat_parents(parents, n_nodes, width):
+    """The rows' first n_nodes[b] entries, padded to `width` with -1, one after another (a buffer of int32)."""
+    if (isinstance(parents, (list, tuple)) and len(parents) == len(n_nodes) and min(n_nodes, default=0) >= 0 and
+            all(type(r) is list and len(r) == width for r in parents)):
+        try:
+            flat = array.array("i", itertools.chain.from_iterable(parents))
+        except (TypeError, OverflowError):          # entries that are not plain int32 numbers
+            flat = None
+        if flat is not None and flat.itemsize == 4:
+            for b, n in enumerate(n_nodes):
+                if n < width:
+                    flat[b * width + n:(b + 1) * width] = array.array("i", [-1]) * (width - n)
+            return flat
+    flat = []
+    for b in range(len(n_nodes)):
+        row = [int(x) for x in parents[b][:n_nodes[b]]]
+        flat += row + [-1] * (width - len(row))
+    return (ctypes.c_int32 * len(flat))(*flat)
+
+
 class Forest(Tree):
-    """One tree per sequence, padded to max_nodes (lantern_forest_create); used like a Tree."""
+    """One tree per sequence, padded to max_nodes (lantern_forest_create_in); used like a Tree.  Its device arrays
+    live in a tensor, so making and dropping one per decode step neither allocates nor synchronises the GPU."""
 
     def __init__(self, parents, n_nodes, max_nodes=None):
+        n_nodes = [int(n) for n in n_nodes]
         B = len(n_nodes)
-        self.n_nodes = int(max_nodes if max_nodes is not None else max(int(n) for n in n_nodes))
-        flat = []
-        for b in range(B):
-            row = [int(x) for x in parents[b][:int(n_nodes[b])]]
-            flat += row + [-1] * (self.n_nodes - len(row))
-        self.parent = flat
-        arr = (ctypes.c_int32 * len(flat))(*flat)
-        cnt = (ctypes.c_int32 * B)(*[int(n) for n in n_nodes])
+        self.n_nodes = int(max_nodes if max_nodes is not None else max(n_nodes))
+        self._flat = _flat_parents(parents, n_nodes, self.n_nodes)
+        arr = self._flat if isinstance(self._flat, ctypes.Array) else (ctypes.c_int32 * len(self._flat)).from_buffer(self._flat)
+        cnt = (ctypes.c_int32 * B)(*n_nodes)
         h = ctypes.c_void_p()
-        _check(lib.lantern_forest_create(arr, cnt, B, self.n_nodes, ctypes.byref(h)), "lantern_forest_create")
+        device = torch.cuda.current_device()
+        need = lib.lantern_forest_block(B, self.n_nodes)
+        self.block = torch.empty(max(need, 16), dtype=torch.uint8, device="cuda:%d" % device)
+        self.stream = _raw_stream(device)
+        _check(lib.lantern_forest_create_in(arr, cnt, B, self.n_nodes, self.block.data_ptr(), self.block.numel(), self.stream,
+                                            ctypes.byref(h)), "lantern_forest_create_in")
         self.handle = h
         self.max_depth = lib.lantern_tree_max_depth(h)
+
+    @property
+    def parent(self):
+        return list(self._flat)
+
+    def used_by(self, t):
+        """Work on t's GPU's current stream is about to read the arrays: keep their memory until it is done."""
+        if _raw_stream(t.get_device()) != self.stream:
+            self.block.record_stream(torch.cuda.current_stream(t.get_device()))
 
 
 def _rows(t: torch.Tensor, B, N, V):
     """(row_stride, seq_stride) in elements of a [B][N][V] tensor with unit inner stride."""
-    if t.dim() != 3 or t.shape[0] != B or t.shape[1] != N or t.shape[2] != V or t.stride(2) != 1:
+    if t.shape != (B, N, V):
         raise ValueError("expected a [B][N][V] tensor with contiguous rows")
-    return t.stride(1), t.stride(0)
+    seq, row, one = t.stride()
+    if one != 1:
+        raise ValueError("expected a [B][N][V] tensor with contiguous rows")
+    return row, seq
 
 
 def build_neighbors(codebook: torch.Tensor, k: int, return_dist=False):
@@ -196,9 +254,8 @@ def build_neighbors(codebook: torch.Tensor, k: int, return_dist=False):
     dt = _dtype_code(codebook)
     wbytes = lib.lantern_build_neighbors_workspace(dt, L, d, k)
     ws = torch.empty(max(wbytes, 256), dtype=torch.uint8, device=codebook.device)
-    with torch.cuda.device(codebook.device):
-        _check(lib.lantern_build_neighbors(_ptr(codebook), dt, L, d, k, _ptr(idx), _ptr(dist), _ptr(ws),
-                                           ws.numel(), _stream()), "lantern_build_neighbors")
+    _call(lib.lantern_build_neighbors, "lantern_build_neighbors", codebook, _ptr(codebook), dt, L, d, k, _ptr(idx),
+          _ptr(dist), _ptr(ws), ws.numel())
     return (idx, dist) if return_dist else idx
 
 
@@ -245,11 +302,10 @@ def sample_draft_tree(params: Params, tree: Tree, draft_cond, draft_uncond=None,
                                         or tuple(gumbel_uniforms.shape) != (B, N, V)):
         raise ValueError("gumbel_uniforms must be contiguous float32 [B][N][V]")
     cp = params.c()
-    with torch.cuda.device(draft_cond.device):
-        _check(lib.lantern_sample_draft_tree(
-            ctypes.byref(cp), tree.handle, _ptr(draft_cond), _ptr(draft_uncond), _dtype_code(draft_cond), rs, ss,
-            B, parent_begin, N if parent_end is None else parent_end, _ptr(gumbel_uniforms), _ptr(tokens),
-            _ptr(draft_prob), _ptr(device_status), _stream()), "lantern_sample_draft_tree")
+    _call(lib.lantern_sample_draft_tree, "lantern_sample_draft_tree", draft_cond,
+          ctypes.byref(cp), tree.handle, _ptr(draft_cond), _ptr(draft_uncond), _dtype_code(draft_cond), rs, ss,
+          B, parent_begin, N if parent_end is None else parent_end, _ptr(gumbel_uniforms), _ptr(tokens),
+          _ptr(draft_prob), _ptr(device_status))
     return tokens
 
 
@@ -287,13 +343,13 @@ def verify_tree(params: Params, tree: Tree, nbr_idx, target_cond, target_uncond,
         workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
     k_table = 0 if nbr_idx is None else nbr_idx.shape[1]
     cp = params.c()
-    with torch.cuda.device(dev):
-        _check(lib.lantern_verify_tree(
-            ctypes.byref(cp), tree.handle, _ptr(nbr_idx), k_table, _ptr(target_cond), _ptr(target_uncond),
-            _ptr(draft_cond), _ptr(draft_uncond), _dtype_code(target_cond), rs, ss, B, _ptr(tokens),
-            _ptr(u_accept), _ptr(u_resample), _ptr(accept_len), _ptr(out_tokens), _ptr(out_nodes),
-            _ptr(node_next), _ptr(node_token), _ptr(node_mass), _ptr(node_thresh), _ptr(device_status),
-            _ptr(workspace), workspace.numel(), _stream()), "lantern_verify_tree")
+    tree.used_by(target_cond)
+    _call(lib.lantern_verify_tree, "lantern_verify_tree", target_cond,
+          ctypes.byref(cp), tree.handle, _ptr(nbr_idx), k_table, _ptr(target_cond), _ptr(target_uncond),
+          _ptr(draft_cond), _ptr(draft_uncond), _dtype_code(target_cond), rs, ss, B, _ptr(tokens),
+          _ptr(u_accept), _ptr(u_resample), _ptr(accept_len), _ptr(out_tokens), _ptr(out_nodes),
+          _ptr(node_next), _ptr(node_token), _ptr(node_mass), _ptr(node_thresh), _ptr(device_status),
+          _ptr(workspace), workspace.numel())
     return out
 
 
@@ -312,13 +368,12 @@ def verify_tree_static(params: Params, tree: Tree, nbr_idx, target_cond, target_
             raise ValueError("all logit tensors must share strides")
     k_table = 0 if nbr_idx is None else nbr_idx.shape[1]
     cp = params.c()
-    with torch.cuda.device(target_cond.device):
-        _check(lib.lantern_verify_tree_static(
-            ctypes.byref(cp), tree.handle, _ptr(nbr_idx), k_table, _ptr(target_cond), _ptr(target_uncond),
-            _ptr(draft_cond), _ptr(draft_uncond), _dtype_code(target_cond), rs, ss, B, _ptr(tokens),
-            _ptr(u_accept), _ptr(u_resample), _ptr(out["accept_len"]), _ptr(out["out_tokens"]),
-            _ptr(out["out_nodes"]), _ptr(out.get("node_mass")), _ptr(out.get("node_thresh")),
-            _ptr(device_status), _stream()), "lantern_verify_tree_static")
+    tree.used_by(target_cond)
+    _call(lib.lantern_verify_tree_static, "lantern_verify_tree_static", target_cond,
+          ctypes.byref(cp), tree.handle, _ptr(nbr_idx), k_table, _ptr(target_cond), _ptr(target_uncond),
+          _ptr(draft_cond), _ptr(draft_uncond), _dtype_code(target_cond), rs, ss, B, _ptr(tokens),
+          _ptr(u_accept), _ptr(u_resample), _ptr(out["accept_len"]), _ptr(out["out_tokens"]),
+          _ptr(out["out_nodes"]), _ptr(out.get("node_mass")), _ptr(out.get("node_thresh")), _ptr(device_status))
     return out
 
 
@@ -348,11 +403,10 @@ def expand_frontier(params: Params, pool: DraftPool, draft_cond, draft_uncond=No
         raise ValueError("cond and uncond rows must share strides")
     nxt = torch.empty((B, pool.E), dtype=torch.int32, device=draft_cond.device)
     cp = params.c()
-    with torch.cuda.device(draft_cond.device):
-        _check(lib.lantern_expand_frontier(
-            ctypes.byref(cp), _ptr(draft_cond), _ptr(draft_uncond), _dtype_code(draft_cond), rs, ss, B, F, pool.K, pool.E,
-            _ptr(pool.frontier), pool.P, pool.used, pool.n_depths + 1, _ptr(pool.parent), _ptr(pool.token),
-            _ptr(pool.logv), _ptr(pool.depth), _ptr(nxt), _stream()), "lantern_expand_frontier")
+    _call(lib.lantern_expand_frontier, "lantern_expand_frontier", draft_cond,
+          ctypes.byref(cp), _ptr(draft_cond), _ptr(draft_uncond), _dtype_code(draft_cond), rs, ss, B, F, pool.K, pool.E,
+          _ptr(pool.frontier), pool.P, pool.used, pool.n_depths + 1, _ptr(pool.parent), _ptr(pool.token),
+          _ptr(pool.logv), _ptr(pool.depth), _ptr(nxt))
     pool.used += F * pool.K
     pool.n_depths += 1
     pool.frontier = nxt
@@ -367,18 +421,16 @@ def trim_tree(pool: DraftPool, max_nodes: int):
     token = torch.empty_like(parent)
     index = torch.empty_like(parent)
     logv = torch.empty((pool.B, max_nodes), dtype=torch.float64, device=dev)
-    with torch.cuda.device(dev):
-        _check(lib.lantern_trim_tree(pool.B, pool.P, pool.used, pool.n_depths, _ptr(pool.parent), _ptr(pool.token),
-                                     _ptr(pool.logv), _ptr(pool.depth), max_nodes, _ptr(n), _ptr(parent), _ptr(token),
-                                     _ptr(index), _ptr(logv), _stream()), "lantern_trim_tree")
+    _call(lib.lantern_trim_tree, "lantern_trim_tree", pool.parent, pool.B, pool.P, pool.used, pool.n_depths,
+          _ptr(pool.parent), _ptr(pool.token), _ptr(pool.logv), _ptr(pool.depth), max_nodes, _ptr(n), _ptr(parent),
+          _ptr(token), _ptr(index), _ptr(logv))
     return n, parent, token, index, logv
 
 
 def philox_raw(seed, first, c1, c2, c3, n, device="cuda"):
     """lantern_philox_raw: [n][4] raw Philox-4x32-10 words as int64 (values < 2^32)."""
     out = torch.empty((n, 4), dtype=torch.int32, device=device)
-    with torch.cuda.device(out.device):
-        _check(lib.lantern_philox_raw(seed, first, c1, c2, c3, n, _ptr(out), _stream()), "lantern_philox_raw")
+    _call(lib.lantern_philox_raw, "lantern_philox_raw", out, seed, first, c1, c2, c3, n, _ptr(out))
     return out.to(torch.int64) & 0xFFFFFFFF
 
 

@@ -73,8 +73,9 @@ extern "C" lantern_status lantern_tree_create(const int32_t* parent, int32_t n_n
 // A forest: one tree per sequence, all padded to max_nodes (Sec. 2.1, dynamic tree drafting: the
 // shape of the draft tree depends on the sequence).  The device arrays are [batch][max_nodes];
 // padding nodes have no children and an order entry of -1.
-extern "C" lantern_status lantern_forest_create(const int32_t* parent, const int32_t* n_nodes, int32_t batch,
-                                                int32_t max_nodes, lantern_tree** out) {
+// `block`: device memory of the caller for those arrays, filled on `stream`; NULL: allocated here.
+static lantern_status make_forest(const int32_t* parent, const int32_t* n_nodes, int32_t batch, int32_t max_nodes,
+                                  void* block, cudaStream_t stream, lantern_tree** out) {
   if (!parent || !n_nodes || !out || batch < 1 || max_nodes < 1) return LANTERN_ERR_INVALID_ARG;
   if (max_nodes > LANTERN_MAX_NODES || static_cast<int64_t>(batch) * max_nodes > (1 << 24)) return LANTERN_ERR_UNSUPPORTED;
   const size_t BN = static_cast<size_t>(batch) * max_nodes;
@@ -112,10 +113,18 @@ extern "C" lantern_status lantern_forest_create(const int32_t* parent, const int
   if (max_children > LANTERN_MAX_CHILDREN) { free(host); return LANTERN_ERR_UNSUPPORTED; }
   TreeDev* t = static_cast<TreeDev*>(calloc(1, sizeof(TreeDev)));
   if (!t) { free(host); return LANTERN_ERR_CUDA; }
-  void* dev = nullptr;
-  if (cudaMalloc(&dev, sizeof(int32_t) * 3 * BN) != cudaSuccess ||
-      cudaMemcpy(dev, host, sizeof(int32_t) * 3 * BN, cudaMemcpyHostToDevice) != cudaSuccess) {
-    if (dev) cudaFree(dev);
+  void* dev = block;
+  cudaError_t e = cudaSuccess;
+  if (block) {
+    // the arrays are in place when this returns, whatever stream uses the handle
+    e = cudaMemcpyAsync(dev, host, sizeof(int32_t) * 3 * BN, cudaMemcpyHostToDevice, stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+  } else {
+    e = cudaMalloc(&dev, sizeof(int32_t) * 3 * BN);
+    if (e == cudaSuccess) e = cudaMemcpy(dev, host, sizeof(int32_t) * 3 * BN, cudaMemcpyHostToDevice);
+  }
+  if (e != cudaSuccess) {
+    if (!block && dev) cudaFree(dev);
     free(host);
     free(t);
     return LANTERN_ERR_CUDA;
@@ -125,7 +134,7 @@ extern "C" lantern_status lantern_forest_create(const int32_t* parent, const int
   t->max_children = max_children;
   t->n_internal = max_internal;
   t->per_seq = batch;
-  t->d_block = dev;
+  t->d_block = block ? nullptr : dev;
   t->d_first_child = static_cast<int32_t*>(dev);
   t->d_n_child = t->d_first_child + BN;
   t->d_order = t->d_first_child + 2 * BN;
@@ -135,10 +144,33 @@ extern "C" lantern_status lantern_forest_create(const int32_t* parent, const int
   return LANTERN_OK;
 }
 
+extern "C" lantern_status lantern_forest_create(const int32_t* parent, const int32_t* n_nodes, int32_t batch,
+                                                int32_t max_nodes, lantern_tree** out) {
+  return make_forest(parent, n_nodes, batch, max_nodes, nullptr, nullptr, out);
+}
+
+extern "C" size_t lantern_forest_block(int32_t batch, int32_t max_nodes) {
+  if (batch < 1 || max_nodes < 1) return 0;
+  return sizeof(int32_t) * 3 * static_cast<size_t>(batch) * max_nodes;
+}
+
+extern "C" lantern_status lantern_forest_create_in(const int32_t* parent, const int32_t* n_nodes, int32_t batch,
+                                                   int32_t max_nodes, void* block, size_t block_bytes, void* stream,
+                                                   lantern_tree** out) {
+  if (!block || reinterpret_cast<uintptr_t>(block) % 16) return LANTERN_ERR_WORKSPACE;
+  if (batch < 1 || max_nodes < 1) return LANTERN_ERR_INVALID_ARG;
+  if (block_bytes < lantern_forest_block(batch, max_nodes)) return LANTERN_ERR_WORKSPACE;
+  // a copy from this call's own host arrays must not become part of a graph
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+    return LANTERN_ERR_CUDA;
+  return make_forest(parent, n_nodes, batch, max_nodes, block, static_cast<cudaStream_t>(stream), out);
+}
+
 extern "C" lantern_status lantern_tree_destroy(lantern_tree* tree) {
   if (!tree) return LANTERN_OK;
   TreeDev* t = reinterpret_cast<TreeDev*>(tree);
-  cudaError_t e = cudaFree(t->d_block);
+  const cudaError_t e = t->d_block ? cudaFree(t->d_block) : cudaSuccess;
   free(t->h_first_child);   // base of the host block
   free(t);
   return e == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;

@@ -23,7 +23,7 @@ struct TreeDev {
   int32_t* d_first_child;   // [N] first child id, or -1
   int32_t* d_n_child;       // [N]
   int32_t* d_order;         // [N] node ids, internal nodes first (launch order)
-  void* d_block;            // the one allocation behind the arrays above
+  void* d_block;            // the one allocation behind the arrays above, NULL when it belongs to the caller
   int32_t* h_first_child;
   int32_t* h_n_child;
 };

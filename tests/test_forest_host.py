@@ -1,0 +1,46 @@
+"""The host side of a forest handle: the flat parent array that lantern_forest_create_in reads."""
+import numpy as np
+import pytest
+
+from paper_2502_06352_b200 import binding
+
+
+def _want(parents, n_nodes, width):
+    flat = []
+    for b, n in enumerate(n_nodes):
+        row = [int(x) for x in parents[b][:n]]
+        flat += row + [-1] * (width - len(row))
+    return flat
+
+
+@pytest.mark.parametrize("form", ["lists", "ragged", "tuples", "numpy", "numpy_int64", "floats", "numpy_rows", "tensor"])
+def test_flat_parents_of_every_form(form):
+    import torch
+    rows = [[-1, 0, 0, 1], [-1, 0, 7, 9], [-1, 5, 5, 5], [-1, 0, 1, 2]]
+    n_nodes, width = [4, 2, 1, 3], 4
+    if form == "lists":
+        parents = rows
+    elif form == "ragged":
+        parents = [r[:n] for r, n in zip(rows, n_nodes)]
+    elif form == "tuples":
+        parents = tuple(tuple(r) for r in rows)
+    elif form == "numpy":
+        parents = np.array(rows, dtype=np.int32)
+    elif form == "numpy_int64":
+        parents = np.array(rows, dtype=np.int64)
+    elif form == "floats":
+        parents = [[float(x) for x in r] for r in rows]
+    elif form == "numpy_rows":
+        parents = [np.array(r) for r in rows]
+    else:
+        parents = torch.tensor(rows)
+    assert list(binding._flat_parents(parents, n_nodes, width)) == _want(parents, n_nodes, width)
+
+
+def test_flat_parents_of_odd_counts():
+    rows = [[-1, 0, 0], [-1, 0, 1]]
+    for n_nodes in ([0, 3], [3, 5], [-1, 2]):       # refused by the library later, never misread here
+        assert list(binding._flat_parents(rows, n_nodes, 3)) == _want(rows, n_nodes, 3)
+    assert list(binding._flat_parents([[-1, 0, 0, 0], [-1, 0, 1, 1]], [3, 3], 3)) == [-1, 0, 0, -1, 0, 1]
+    big = [[-1, 2 ** 31, 0], [-1, 0, 1]]             # wraps like a C integer, as ctypes does
+    assert len(list(binding._flat_parents(big, [3, 3], 3))) == 6

@@ -218,3 +218,43 @@ def test_argument_errors_are_reported_before_anything_runs(L):
     out = L.verify_tree(par, forest, None, tc, None, None, None, tok, u, u)
     torch.cuda.synchronize()
     assert out["accept_len"].shape == (2,)
+
+
+def test_a_forest_dropped_while_another_stream_still_reads_it(L):
+    """The handle's arrays live in caching-allocator memory: work on a stream other than the one the forest was made on
+    keeps them until it is done, however soon the handle is dropped and its memory asked for again."""
+    B, N, V = 64, 24, 4096
+    g = torch.Generator().manual_seed(5)
+    parents = [[-1] + [(i - 1) // (2 + b % 3) for i in range(1, N)] for b in range(B)]
+    tc = torch.randn((B, N, V), generator=g).cuda()
+    tok = torch.randint(0, V, (B, N), generator=g, dtype=torch.int32).cuda()
+    u = torch.rand((2, B, N), generator=g).cuda()
+    par = L.Params(vocab=V, k=0, draft_deterministic=1)
+    want = L.verify_tree(par, L.Forest(parents, [N] * B, N), None, tc, None, None, None, tok, u[0], u[1], debug=True)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    for _ in range(5):
+        forest = L.Forest(parents, [N] * B, N)
+        ws = torch.empty(L.lib.lantern_verify_tree_workspace(forest.handle, B), dtype=torch.uint8, device="cuda")
+        out = {k: torch.empty_like(v) for k, v in want.items()}
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(2_000_000)
+            L.verify_tree(par, forest, None, tc, None, None, None, tok, u[0], u[1], debug=True, out=out, workspace=ws)
+        size = forest.block.numel()
+        del forest
+        junk = [torch.full((size,), 255, dtype=torch.uint8, device="cuda") for _ in range(8)]
+        torch.cuda.synchronize()
+        for k, v in want.items():
+            assert torch.equal(out[k], v), k
+        del junk
+
+
+def test_a_forest_is_not_made_inside_a_capture(L):
+    graph = torch.cuda.CUDAGraph()
+    x = torch.zeros(4, device="cuda")
+    with pytest.raises(L.LanternError):
+        with torch.cuda.graph(graph):
+            x.add_(1)
+            L.Forest([[-1, 0, 0]], [3], 3)
+    torch.cuda.synchronize()
