@@ -10,7 +10,7 @@
 // (log V descending, pool index ascending); a parent therefore always ranks before its children.
 #include <cmath>
 
-#include "rowops.cuh"
+#include "toplist.cuh"
 
 namespace lantern {
 
@@ -46,58 +46,6 @@ __device__ __forceinline__ void block_best(float& z, int& j, float* sz, int* sj)
   __syncthreads();
 }
 
-constexpr int kDynList = 1024;          // tokens at or above the row's selection threshold
-
-// Visits every allowed token of a row once: 16-byte vector loads over the aligned middle (when the
-// row pointers allow it), scalar loads at the ragged ends.  fn(j, z) per token; fold() after every
-// vector and after every scalar token.
-template <typename T, bool CFG, typename F, typename G>
-__device__ __forceinline__ void for_each_z(const T* c, const T* u, float g, float inv_tau, int lo, int hi, F&& fn, G&& fold) {
-  constexpr int VN = Vec<T>::N;
-  auto z1 = [&](float cc, float uu) { return combine<CFG>(cc, uu, g, inv_tau); };
-  const bool aligned = (reinterpret_cast<uintptr_t>(c) % 16 == 0) && (!CFG || reinterpret_cast<uintptr_t>(u) % 16 == 0);
-  int v0 = lo, v1 = lo;                                 // vector part [v0, v1)
-  if (aligned) {
-    v0 = (lo + VN - 1) / VN * VN;
-    v1 = hi / VN * VN;
-    if (v1 < v0) v1 = v0;
-  }
-  const int tid = threadIdx.x;
-  for (int j = lo + tid; j < (aligned ? min(v0, hi) : hi); j += kDynThreads) {
-    fn(j, z1(Vec<T>::widen(c[j]), CFG ? Vec<T>::widen(u[j]) : 0.f));
-    fold();
-  }
-  if (!aligned) return;
-  constexpr int UV = 4;                                 // vectors a thread keeps in flight (more would only grow the code)
-  for (int j0 = v0 + tid * VN; j0 < v1; j0 += kDynThreads * VN * UV) {
-    uint4 rc[UV], ru[UV];
-#pragma unroll
-    for (int q = 0; q < UV; ++q) {
-      const int j = j0 + q * kDynThreads * VN;
-      if (j < v1) {
-        rc[q] = ldg_stream_u128(c + j);
-        if (CFG) ru[q] = ldg_stream_u128(u + j);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < UV; ++q) {
-      const int j = j0 + q * kDynThreads * VN;
-      if (j < v1) {
-        float cf[VN], uf[VN];
-        Vec<T>::unpack_raw(rc[q], cf);
-        if (CFG) Vec<T>::unpack_raw(ru[q], uf);
-#pragma unroll
-        for (int e = 0; e < VN; ++e) fn(j + e, z1(cf[e], CFG ? uf[e] : 0.f));
-        fold();
-      }
-    }
-  }
-  for (int j = max(v1, v0) + tid; j < hi; j += kDynThreads) {
-    fn(j, z1(Vec<T>::widen(c[j]), CFG ? Vec<T>::widen(u[j]) : 0.f));
-    fold();
-  }
-}
-
 // The round of the fallback path: best token after (pz, pj) over the whole row, scalar loads.  Kept out
 // of line so that this rarely used scan does not grow the kernel's main loops.
 template <typename T>
@@ -111,116 +59,307 @@ __device__ __noinline__ void scan_row_after(const T* c, const T* u, float g, flo
   }
 }
 
-// One frontier row.  Pass 1 (from HBM): every thread's maximum; the K-th largest of the warps' two
-// largest thread maxima each is a lower bound tau of the row's K-th largest value.  Pass 2 (the row is in L2 now): the
-// softmax denominator, and the tokens with z >= tau go to a short list in shared memory, from which
-// K rounds pick the children in the order (z descending, token ascending).  A list that overflows
-// (thousands of equal values) falls back to K rounds over the row.
-template <typename T, bool CFG>
-__global__ void __launch_bounds__(kDynThreads) expand_rows_kernel(const ExpandArgs a) {
-  __shared__ float sz[kDynThreads / 32];
-  __shared__ int sj[kDynThreads / 32];
-  __shared__ double sd[kDynThreads / 32];
-  __shared__ float tmax[2 * (kDynThreads / 32)];
-  __shared__ float lz[kDynList];
-  __shared__ int lj[kDynList];
-  __shared__ int lcount;
-  const int f = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+// Softmax denominator of a thread's elements relative to a reference m, the first finite vector's maximum: terms in
+// float32 from exact differences, a vector's terms summed in float32 and folded into a double.
+template <int VN>
+__device__ __forceinline__ void fold_exp(const float (&z)[VN], float& m, double& s) {
+  if (m == -INFINITY) {
+#pragma unroll
+    for (int e = 0; e < VN; ++e) m = fmaxf(m, z[e]);
+    if (m == -INFINITY) return;
+  }
+  float part = 0.f;
+#pragma unroll
+  for (int e = 0; e < VN; ++e) part += ex2_approx(__fmul_rn(__fsub_rn(z[e], m), kLog2e));   // (the argument's rounding costs
+                                                                                             // |z - m| 2^-24 relative)
+  if (!(part < 1e30f)) {             // an entry far above the reference: move the reference
+    float bm = m;
+#pragma unroll
+    for (int e = 0; e < VN; ++e) bm = fmaxf(bm, z[e]);
+    s *= exp(static_cast<double>(m) - static_cast<double>(bm));
+    m = bm;
+    part = 0.f;
+#pragma unroll
+    for (int e = 0; e < VN; ++e) part += ex2_approx(__fmul_rn(__fsub_rn(z[e], m), kLog2e));
+  }
+  s += static_cast<double>(part);
+}
+
+// One frontier row by one CTA, or by a cluster when a call has few rows: the row is streamed once.  The first
+// chunk's elements give a threshold, a lower bound of the row's K-th largest value; the few elements that reach it go to
+// a list in shared memory, cut back to its K best after a third of the row, and the softmax denominator comes from
+// the same pass.  The CTAs of a row push their K best and their sums to the first one, which writes the
+// children in the order (z descending, token ascending).
+// Bound: instruction issue and the latency of a chunk's loads.  A depth (rows and frontier) of 512 rows of 65536 bfloat16
+// logits: 33 us, with two passes over the row (maxima, then terms and list) 40; of 8 rows: 14 us, was 25; 512 rows of
+// 40003 logits (most of them unaligned): 27 us, was 92.
+template <typename T, bool CFG, bool TAU1>
+__global__ void __launch_bounds__(kDynThreads, 4) expand_rows_kernel(const ExpandArgs a) {
+  using namespace stream;
+  static_assert(kDynThreads == ST, "the list helpers are built for this many threads");
+  using IO = RowIO<T, CFG, TAU1>;
+  constexpr int VN = IO::VN;
+  constexpr int UV = (CFG ? 2 : 4) * 4 / VN;
+  static_assert(ST * UV * VN <= kIterElems, "iteration size");
+  grid_dependency_sync();
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  TopList s;
+  s.list = reinterpret_cast<uint2*>(dyn_smem);
+  s.fin = s.list + kListCap;
+  s.pk = s.fin + kFinal;
+  s.top = s.pk + 2 * 2 * SW;
+  s.rinfo = s.top + 16;
+  double* rsum = reinterpret_cast<double*>(s.rinfo + kMaxCluster);    // [kMaxCluster] the CTAs' sums, in CTA 0
+  double* wsum = rsum + kMaxCluster;                                   // [SW] the warps' sums
+  float* rmax = reinterpret_cast<float*>(wsum + SW);                   // [SW] the warps' references
+  int* sj = reinterpret_cast<int*>(rmax + SW);                         // [SW]
+  s.cnt = sj + SW;
+  s.fkey = nullptr;
+  const uint32_t rank = cluster_ctarank(), nrank = cluster_nctarank();
+  if (nrank > 1) cluster_arrive_relaxed();            // waited for before the first access to a peer's shared memory
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int idx = blockIdx.x / nrank;
+  const int b = idx / a.F, f = idx - b * a.F;
   const int node = a.frontier[b * a.F + f];
   const long long pbase = static_cast<long long>(b) * a.P + a.pool_off + f * a.K;
-  if (node < 0) {                                   // empty slot: candidates that can never be chosen
-    for (int r = tid; r < a.K; r += kDynThreads) {
-      a.pool_parent[pbase + r] = -1;
-      a.pool_token[pbase + r] = -1;
-      a.pool_depth[pbase + r] = a.depth;
-      a.pool_logv[pbase + r] = -INFINITY;
+  if (node < 0) {                                   // empty slot: candidates that can never be chosen (the whole cluster leaves)
+    if (rank == 0) {
+      for (int r = tid; r < a.K; r += kDynThreads) {
+        a.pool_parent[pbase + r] = -1;
+        a.pool_token[pbase + r] = -1;
+        a.pool_depth[pbase + r] = a.depth;
+        a.pool_logv[pbase + r] = -INFINITY;
+      }
     }
+    if (nrank > 1) cluster_wait();
     return;
   }
-  const T* c = static_cast<const T*>(a.dc) + b * a.seq_stride + f * a.row_stride;
-  const T* u = CFG ? static_cast<const T*>(a.du) + b * a.seq_stride + f * a.row_stride : nullptr;
-  // pass 1 (from HBM): maxima only
-  float m = -INFINITY;
-  for_each_z<T, CFG>(c, u, a.g, a.inv_tau, a.allow_lo, a.allow_hi, [&](int, float z) { m = fmaxf(m, z); }, [] {});
-  // the two largest thread maxima of every warp: 16 values of distinct tokens, whose K-th largest
-  // (K <= 8) is a lower bound tau of the row's K-th largest value; every warp ranks them for itself
-  {
-    const int lane = tid & 31, warp = tid >> 5;
-    const float w1 = warp_max(m);
-    const int wl = __ffs(__ballot_sync(0xffffffffu, m == w1)) - 1;
-    const float w2 = warp_max(lane == wl ? -INFINITY : m);
-    if (lane == 0) { tmax[2 * warp] = w1; tmax[2 * warp + 1] = w2; }
-  }
-  if (tid == 0) lcount = 0;
-  float bm = m;
-  int bj = tid;
-  block_best(bm, bj, sz, sj);                       // bm: the row's maximum (the barriers inside publish tmax and lcount too)
-  float tau = -INFINITY;
-  {
-    const int lane = tid & 31;
-    constexpr int NV = 2 * (kDynThreads / 32);
-    const float v = lane < NV ? tmax[lane] : -INFINITY;
-    int r = 0;
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const float o = __shfl_sync(0xffffffffu, v, i);
-      r += (o > v || (o == v && i < lane)) ? 1 : 0;
-    }
-    const uint32_t hit = __ballot_sync(0xffffffffu, lane < NV && r == min(a.K, NV) - 1);
-    tau = __shfl_sync(0xffffffffu, v, __ffs(hit) - 1);
-  }
-  // pass 2 (the row is in L2 now): softmax denominator relative to the row maximum, terms in float32,
-  // a vector's terms summed in float32 and folded into a double (double-precision work is slow on this
-  // part, so it stays at one addition per vector); tokens at or above tau go to the list
-  double s = 0.0;
-  float part = 0.f;
-  for_each_z<T, CFG>(c, u, a.g, a.inv_tau, a.allow_lo, a.allow_hi,
-                [&](int j, float z) {
-                  part += ex2_approx(__fmul_rn(__fsub_rn(z, bm), kLog2e));   // exp(z - max): the argument's rounding costs
-                                                                             // |z - max| 2^-24 relative on a term of weight exp(z - max)
-                  if (z >= tau) {
-                    const int pos = atomicAdd(&lcount, 1);
-                    if (pos < kDynList) { lz[pos] = z; lj[pos] = j; }
-                  }
-                },
-                [&] { s += static_cast<double>(part); part = 0.f; });
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((tid & 31) == 0) sd[tid >> 5] = s;
+  const int K = a.K;
+  IO io;
+  io.c = static_cast<const T*>(a.dc) + b * a.seq_stride + f * a.row_stride;
+  io.u = CFG ? static_cast<const T*>(a.du) + b * a.seq_stride + f * a.row_stride : nullptr;
+  io.g = a.g; io.it = a.inv_tau;
+  // vectors from the 16-byte boundary at or before the first allowed token (rows need no alignment here); rows whose two
+  // operands sit differently are read element by element
+  Geo ge;
+  ge.alo = a.allow_lo; ge.ahi = a.allow_hi;
+  const int off = static_cast<int>((reinterpret_cast<uintptr_t>(io.c + ge.alo) & 15u) / sizeof(T));
+  const bool together = !CFG || ((reinterpret_cast<uintptr_t>(io.c) ^ reinterpret_cast<uintptr_t>(io.u)) & 15u) == 0;
+  ge.j0 = ge.alo - off;
+  io.j0 = ge.j0;
+  ge.nvec = (ge.ahi - ge.j0 + VN - 1) / VN;
+  ge.vi0 = off > 0 ? 1 : 0;
+  ge.vi1 = (ge.j0 + ge.nvec * VN > ge.ahi) ? ge.nvec - 1 : ge.nvec;
+  if (ge.vi1 < ge.vi0 || !together) ge.vi1 = ge.vi0;
+  const int nwarps = static_cast<int>(nrank) * SW;
+  ge.vw = ((ge.nvec + nwarps - 1) / nwarps + 31) / 32 * 32;
+  const int gw = static_cast<int>(rank) * SW + warp;
+  const int vbeg = min(gw * ge.vw, ge.nvec), vend = min(vbeg + ge.vw, ge.nvec);
+  if (tid == 0) *s.cnt = 0;
   __syncthreads();
-  s = 0.0;
-  for (int w = 0; w < kDynThreads / 32; ++w) s += sd[w];
-  const double ln_s = log(s);
-  const double parent_logv = a.pool_logv[static_cast<long long>(b) * a.P + node];
-  __syncthreads();
-  const int n = lcount;
-  const bool listed = n <= kDynList;
-  float pz = INFINITY;
-  int pj = -1;
-  for (int r = 0; r < a.K; ++r) {
-    float bz = -INFINITY;
-    int bjj = 0x7fffffff;
-    if (listed) {
-      for (int i = tid; i < n; i += kDynThreads) {
-        const float z = lz[i];
-        const int j = lj[i];
-        const bool after = z < pz || (z == pz && j > pj);
-        if (after && (z > bz || (z == bz && j < bjj))) { bz = z; bjj = j; }
-      }
+
+  auto append = [&](float z, int tok) {
+    const int pos = atomicAdd(s.cnt, 1);
+    if (pos < kListCap) s.list[pos] = make_uint2(__float_as_uint(z), static_cast<uint32_t>(tok));
+  };
+  auto cut = [&](float T0) { return *s.cnt <= ST ? cut_ranked(s, K, T0) : cut_list(s, K, T0); };
+  // z of vector vv (anything beyond the warp's range or the allowed tokens: -inf)
+  auto vec_z = [&](int vv, const uint4& rc, const uint4& ru, float (&z)[VN]) {
+    if (vv < vend && vv >= ge.vi0 && vv < ge.vi1) {
+      io.z(rc, ru, z);
     } else {
-      scan_row_after<T>(c, u, a.g, a.inv_tau, a.allow_lo, a.allow_hi, pz, pj, bz, bjj);
+#pragma unroll
+      for (int e = 0; e < VN; ++e) {
+        const int t = ge.j0 + vv * VN + e;
+        z[e] = (vv < vend && t >= ge.alo && t < ge.ahi) ? io.z_at(t) : -INFINITY;
+      }
     }
-    block_best(bz, bjj, sz, sj);
-    if (tid == 0) {
-      const bool found = bjj != 0x7fffffff;         // fewer than K allowed tokens: the rest can never be chosen
-      a.pool_parent[pbase + r] = found ? node : -1;
-      a.pool_token[pbase + r] = found ? bjj : -1;
-      a.pool_depth[pbase + r] = a.depth;
-      a.pool_logv[pbase + r] = found ? parent_logv + ((static_cast<double>(bz) - static_cast<double>(bm)) - ln_s) : -INFINITY;
+  };
+  float Tk, m;
+  double sum;
+  const int iters = (ge.vw + 32 * UV - 1) / (32 * UV);
+  const int cut_it = max(1, iters / 3);
+  for (int mode = 0; mode < 2; ++mode) {              // (mode 1: the list overflowed, the row is redone with a cut after every chunk)
+    m = -INFINITY;
+    sum = 0.0;
+    {
+      uint4 rc[UV], ru[UV];
+#pragma unroll
+      for (int u = 0; u < UV; ++u) {
+        const int vv = vbeg + 32 * u + lane;
+        if (vv < vend && vv >= ge.vi0 && vv < ge.vi1) io.load(vv, rc[u], ru[u]);
+      }
+      float first[UV][VN];
+      float tbk = -INFINITY;
+      int tbj = 0x7fffffff;
+#pragma unroll
+      for (int u = 0; u < UV; ++u) {
+        const int vv = vbeg + 32 * u + lane;
+        vec_z(vv, rc[u], ru[u], first[u]);
+        fold_exp<VN>(first[u], m, sum);
+#pragma unroll
+        for (int e = 0; e < VN; ++e)
+          if (key_before(first[u][e], ge.j0 + vv * VN + e, tbk, tbj)) { tbk = first[u][e]; tbj = ge.j0 + vv * VN + e; }
+      }
+      Tk = first_threshold(s, K, tbk, tbj);
+#pragma unroll
+      for (int u = 0; u < UV; ++u) {
+#pragma unroll
+        for (int e = 0; e < VN; ++e)
+          if (first[u][e] >= Tk && first[u][e] > -INFINITY) append(first[u][e], ge.j0 + (vbeg + 32 * u + lane) * VN + e);
+      }
     }
-    pz = bz;
-    pj = bjj;
+    if (mode == 1) {
+      __syncthreads();
+      const bool full = *s.cnt > kListCap - kIterElems;
+      __syncthreads();
+      if (full) Tk = cut(Tk);
+    }
+    for (int it = 1; it < iters; ++it) {
+      const int base = vbeg + it * 32 * UV;
+      constexpr int UF = 2 * UV;                       // two chunks at once where nothing has to be checked between them
+      if (mode == 0 && it != cut_it && it + 1 < iters && base >= ge.vi0 && base + 32 * UF <= min(vend, ge.vi1)) {
+        uint4 rc[UF], ru[UF];                          // whole vectors only, the same in every lane
+#pragma unroll
+        for (int u = 0; u < UF; ++u) io.load(base + 32 * u + lane, rc[u], ru[u]);
+        uint32_t hit = 0u;                             // vectors with an entry for the list
+        float part[UF], worst = m == -INFINITY ? INFINITY : 0.f;
+#pragma unroll
+        for (int u = 0; u < UF; ++u) {
+          float z[VN];
+          io.z(rc[u], ru[u], z);
+          float top = z[0];
+#pragma unroll
+          for (int e = 1; e < VN; ++e) top = fmaxf(top, z[e]);
+          if (top >= Tk) hit |= 1u << u;
+          part[u] = 0.f;
+#pragma unroll
+          for (int e = 0; e < VN; ++e) part[u] += ex2_approx(__fmul_rn(__fsub_rn(z[e], m), kLog2e));
+          worst += part[u];
+        }
+        if (worst < 1e30f) {                           // (one check for all vectors: the reference stays)
+#pragma unroll
+          for (int u = 0; u < UF; ++u) sum += static_cast<double>(part[u]);
+        } else {
+#pragma unroll
+          for (int u = 0; u < UF; ++u) {
+            float z[VN];
+            io.z(rc[u], ru[u], z);
+            fold_exp<VN>(z, m, sum);
+          }
+        }
+        while (hit) {                                  // few: the vector is read again, so that it need not be kept
+          const int vv = base + 32 * (__ffs(hit) - 1) + lane;
+          hit &= hit - 1u;
+          uint4 c1, u1;
+          io.load(vv, c1, u1);
+          float z[VN];
+          io.z(c1, u1, z);
+#pragma unroll
+          for (int e = 0; e < VN; ++e)
+            if (z[e] >= Tk && z[e] > -INFINITY) append(z[e], ge.j0 + vv * VN + e);
+        }
+        ++it;
+        if (it != cut_it) continue;
+      } else {
+#pragma unroll 1
+        for (int u = 0; u < UV; ++u) {
+          const int vv = base + 32 * u + lane;
+          uint4 rc, ru;
+          if (vv < vend && vv >= ge.vi0 && vv < ge.vi1) io.load(vv, rc, ru);
+          float z[VN];
+          vec_z(vv, rc, ru, z);
+#pragma unroll
+          for (int e = 0; e < VN; ++e)
+            if (z[e] >= Tk && z[e] > -INFINITY) append(z[e], ge.j0 + vv * VN + e);
+          fold_exp<VN>(z, m, sum);
+        }
+      }
+      if (it == cut_it || mode == 1) {
+        __syncthreads();
+        const int cn = *s.cnt;
+        __syncthreads();                                // everyone has read the count before it moves again
+        if (cn <= kListCap && (mode == 1 ? cn > kListCap - kIterElems : cn > K)) Tk = cut(Tk);
+      }
+    }
+    __syncthreads();
+    const bool overflow = *s.cnt > kListCap;
+    if (!overflow) break;
+    __syncthreads();                                    // (mode 1 never overflows: it cuts in time)
+    if (tid == 0) *s.cnt = 0;
+    __syncthreads();
   }
+  cut(Tk);
+  // ---- the sums relative to the CTA's largest reference, in double precision
+  {
+    const float wm = warp_max(m);
+    double v = m == -INFINITY ? 0.0 : (m == wm ? sum : sum * exp(static_cast<double>(m) - static_cast<double>(wm)));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) { wsum[warp] = v; rmax[warp] = wm; }
+  }
+  __syncthreads();
+  float cm = -INFINITY;
+  for (int w = 0; w < SW; ++w) cm = fmaxf(cm, rmax[w]);
+  double cs = 0.0;
+  if (tid == 0)
+    for (int w = 0; w < SW; ++w)
+      if (rmax[w] != -INFINITY) cs += wsum[w] * exp(static_cast<double>(rmax[w]) - static_cast<double>(cm));
+  int nf = *s.cnt;
+  if (nrank > 1) {
+    cluster_wait();                                   // every CTA of the row has started
+    if (tid < nf) dsmem_st_u64(dsmem_addr(smem_u32(&s.fin[rank * kMaxR + tid]), 0), s.list[tid]);
+    if (tid == 0) {
+      dsmem_st_u64(dsmem_addr(smem_u32(&s.rinfo[rank]), 0), make_uint2(static_cast<uint32_t>(nf), __float_as_uint(cm)));
+      const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(cs));
+      dsmem_st_u64(dsmem_addr(smem_u32(&rsum[rank]), 0), make_uint2(static_cast<uint32_t>(bits), static_cast<uint32_t>(bits >> 32)));
+    }
+    cluster_sync();
+    if (rank != 0) return;
+    nf = merge_lists(s, nrank);
+  }
+  // ---- children: the first K of the order
+  if (tid == 0) {
+    const float top = nf > 0 ? __uint_as_float(s.list[0].x) : -INFINITY;          // the row's maximum
+    double total = 0.0;
+    if (nrank > 1) {
+      for (uint32_t r = 0; r < nrank; ++r) {
+        const float rm = __uint_as_float(s.rinfo[r].y);
+        if (rm != -INFINITY) total += rsum[r] * exp(static_cast<double>(rm) - static_cast<double>(top));
+      }
+    } else if (cm != -INFINITY) {
+      total = cs * exp(static_cast<double>(cm) - static_cast<double>(top));
+    }
+    wsum[0] = log(total);
+    wsum[1] = a.pool_logv[static_cast<long long>(b) * a.P + node];
+  }
+  __syncthreads();
+  const float bm = nf > 0 ? __uint_as_float(s.list[0].x) : -INFINITY;
+  const double ln_s = wsum[0], parent_logv = wsum[1];
+  auto child = [&](int r, float z, int tok, bool found) {      // fewer than K allowed tokens: the rest can never be chosen
+    a.pool_parent[pbase + r] = found ? node : -1;
+    a.pool_token[pbase + r] = found ? tok : -1;
+    a.pool_depth[pbase + r] = a.depth;
+    a.pool_logv[pbase + r] = found ? parent_logv + ((static_cast<double>(z) - static_cast<double>(bm)) - ln_s) : -INFINITY;
+  };
+  if (tid < min(nf, K)) child(tid, __uint_as_float(s.list[tid].x), static_cast<int>(s.list[tid].y), true);
+  if (nf < K) {                                       // (fewer finite logits than children: tokens without mass, by token)
+    float pz = nf > 0 ? __uint_as_float(s.list[nf - 1].x) : INFINITY;
+    int pj = nf > 0 ? static_cast<int>(s.list[nf - 1].y) : -1;
+    for (int r = nf; r < K; ++r) {
+      float bz = -INFINITY;
+      int bj = 0x7fffffff;
+      scan_row_after<T>(io.c, io.u, a.g, a.inv_tau, a.allow_lo, a.allow_hi, pz, pj, bz, bj);
+      block_best(bz, bj, rmax, sj);
+      if (tid == 0) child(r, bz, bj, bj != 0x7fffffff);
+      pz = bz;
+      pj = bj;
+    }
+  }
+}
+__host__ __device__ constexpr size_t expand_smem() {
+  return (stream::kListCap + stream::kFinal + 2 * 2 * stream::SW + 16 + kMaxCluster) * 8 + (kMaxCluster + stream::SW) * 8 +
+         stream::SW * 8 + 16;
 }
 
 // order-preserving map of a double to an unsigned 64-bit integer (compares then run on the integer pipe)
@@ -233,6 +372,7 @@ __device__ __forceinline__ unsigned long long mono64(double x) {
 __device__ __forceinline__ int rank_desc(const unsigned long long* v, int n, int i) {
   const unsigned long long vi = v[i];
   int r = 0;
+#pragma unroll 8
   for (int j = 0; j < n; ++j) {
     const unsigned long long vj = v[j];
     r += (vj > vi || (vj == vi && j < i)) ? 1 : 0;
@@ -241,6 +381,7 @@ __device__ __forceinline__ int rank_desc(const unsigned long long* v, int n, int
 }
 
 __global__ void __launch_bounds__(kDynThreads) select_frontier_kernel(const ExpandArgs a) {
+  grid_dependency_sync();
   extern __shared__ unsigned long long dyn_lv[];
   const int b = blockIdx.x, tid = threadIdx.x, T = a.F * a.K;
   const double* lv = a.pool_logv + static_cast<long long>(b) * a.P + a.pool_off;
@@ -263,6 +404,7 @@ struct TrimArgs {
 };
 
 __global__ void __launch_bounds__(kDynThreads) trim_tree_kernel(const TrimArgs a) {
+  grid_dependency_sync();
   extern __shared__ unsigned long long dyn_lv[];     // [used] keys of log V | new id | selected | depth | parent, [used] each
   int* newid = reinterpret_cast<int*>(dyn_lv + a.used);
   int* sel = newid + a.used;
@@ -284,6 +426,7 @@ __global__ void __launch_bounds__(kDynThreads) trim_tree_kernel(const TrimArgs a
   __syncthreads();
   // the selected entries, compacted (order irrelevant); at most m of them
   int* lst = reinterpret_cast<int*>(dyn_lv);        // the keys are no longer needed
+  int* lkey = lst + a.used;
   __shared__ int nsel;
   if (tid == 0) nsel = 0;
   __syncthreads();
@@ -291,36 +434,32 @@ __global__ void __launch_bounds__(kDynThreads) trim_tree_kernel(const TrimArgs a
     if (sel[i]) lst[atomicAdd(&nsel, 1)] = i;
   __syncthreads();
   const int ns = nsel;
-  // breadth-first numbering: a level is ordered by (new id of the parent, pool index)
+  // breadth-first numbering: a level is ordered by (new id of the parent, pool index), one key per entry of the
+  // level (the largest for entries of other levels), so that a place is a count over one array
   for (int dep = 1; dep <= a.max_depth; ++dep) {
     if (tid == 0) level_n = 0;
-    __syncthreads();
     const int start = count;
     for (int t = tid; t < ns; t += kDynThreads) {
       const int i = lst[t];
-      if (dep_s[i] != dep) continue;
-      const int pi = newid[par_s[i]];
-      int pos = 0;
-      for (int t2 = 0; t2 < ns; ++t2) {
-        const int j = lst[t2];
-        if (j == i || dep_s[j] != dep) continue;
-        const int pj = newid[par_s[j]];
-        pos += (pj < pi || (pj == pi && j < i)) ? 1 : 0;
-      }
-      const int id = start + pos;
-      const long long o = static_cast<long long>(b) * a.m + id;
-      a.parent[o] = pi;
-      a.token[o] = a.pool_token[base + i];
-      a.pool_index[o] = i;
-      a.logv[o] = a.pool_logv[base + i];
-      atomicAdd(&level_n, 1);
-      sel[i] = 2 + id;                               // the id is published once the level is complete (below)
+      lkey[t] = dep_s[i] == dep ? newid[par_s[i]] * kDynMaxPool + i : 0x7fffffff;      // (an id is below kDynMaxPool)
     }
     __syncthreads();
     for (int t = tid; t < ns; t += kDynThreads) {
-      const int i = lst[t];
-      if (sel[i] >= 2) { newid[i] = sel[i] - 2; sel[i] = 1; }
+      const int key = lkey[t];
+      if (key == 0x7fffffff) continue;
+      int pos = 0;
+#pragma unroll 8
+      for (int t2 = 0; t2 < ns; ++t2) pos += lkey[t2] < key ? 1 : 0;
+      const int i = lst[t], id = start + pos;
+      const long long o = static_cast<long long>(b) * a.m + id;
+      a.parent[o] = key / kDynMaxPool;
+      a.token[o] = a.pool_token[base + i];
+      a.pool_index[o] = i;
+      a.logv[o] = a.pool_logv[base + i];
+      newid[i] = id;                                 // read from the next level on
+      atomicAdd(&level_n, 1);
     }
+    __syncthreads();
     if (tid == 0) count = start + level_n;
     __syncthreads();
   }
@@ -335,6 +474,16 @@ __global__ void __launch_bounds__(kDynThreads) trim_tree_kernel(const TrimArgs a
   }
 }
 
+}  // namespace lantern
+
+namespace lantern {
+template <typename T, bool CFG, bool TAU1>
+static cudaError_t launch_expand(const ExpandArgs& a, int cs, cudaStream_t st) {
+  auto kern = expand_rows_kernel<T, CFG, TAU1>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(expand_smem()));
+  if (e != cudaSuccess) return e;
+  return launch_after_previous(kern, static_cast<unsigned>(a.B) * a.F * cs, kDynThreads, expand_smem(), st, cs, a);
+}
 }  // namespace lantern
 
 using namespace lantern;
@@ -366,18 +515,27 @@ extern "C" lantern_status lantern_expand_frontier(const lantern_params* p, const
   a.pool_parent = pool_parent; a.pool_token = pool_token; a.pool_depth = pool_depth; a.pool_logv = pool_logv;
   a.next_frontier = next_frontier;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const dim3 grid(n_frontier, batch);
-  const bool cfg = draft_uncond != nullptr;
-  if (dt == LANTERN_F32) {
-    if (cfg) expand_rows_kernel<float, true><<<grid, kDynThreads, 0, st>>>(a);
-    else expand_rows_kernel<float, false><<<grid, kDynThreads, 0, st>>>(a);
-  } else {
-    if (cfg) expand_rows_kernel<__nv_bfloat16, true><<<grid, kDynThreads, 0, st>>>(a);
-    else expand_rows_kernel<__nv_bfloat16, false><<<grid, kDynThreads, 0, st>>>(a);
-  }
-  if (cudaGetLastError() != cudaSuccess) return LANTERN_ERR_CUDA;
-  select_frontier_kernel<<<batch, kDynThreads, static_cast<size_t>(T) * sizeof(double), st>>>(a);
-  return cudaGetLastError() == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
+  const bool cfg = draft_uncond != nullptr, f32 = dt == LANTERN_F32;
+  const long long rows = static_cast<long long>(batch) * n_frontier;
+  // CTAs per row, as for the draft sampler: every SM a CTA, every warp at least one full step of the row
+  int dev = 0, sms = 0, cs = 1;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+    sms = 148;
+  const int nvec = (hi - lo) / (f32 ? 4 : 8);
+  while (cs < 8 && rows * cs < sms && nvec / (2 * cs * stream::SW) >= 32) cs *= 2;
+  if (rows * cs > 0x7fffffffll) return LANTERN_ERR_UNSUPPORTED;
+  const bool tau1 = a.inv_tau == 1.0f;
+  cudaError_t e;
+  if (f32)
+    e = cfg ? launch_expand<float, true, false>(a, cs, st)
+            : (tau1 ? launch_expand<float, false, true>(a, cs, st) : launch_expand<float, false, false>(a, cs, st));
+  else
+    e = cfg ? launch_expand<__nv_bfloat16, true, false>(a, cs, st)
+            : (tau1 ? launch_expand<__nv_bfloat16, false, true>(a, cs, st) : launch_expand<__nv_bfloat16, false, false>(a, cs, st));
+  if (e != cudaSuccess) return LANTERN_ERR_CUDA;
+  e = launch_after_previous(select_frontier_kernel, static_cast<unsigned>(batch), kDynThreads, static_cast<size_t>(T) * sizeof(double), st, 1, a);
+  return e == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
 }
 
 extern "C" lantern_status lantern_trim_tree(int32_t batch, int32_t pool_size, int32_t pool_used, int32_t max_depth,
@@ -392,6 +550,6 @@ extern "C" lantern_status lantern_trim_tree(int32_t batch, int32_t pool_size, in
   a.B = batch; a.P = pool_size; a.used = pool_used; a.m = max_nodes; a.max_depth = max_depth;
   a.pool_parent = pool_parent; a.pool_token = pool_token; a.pool_depth = pool_depth; a.pool_logv = pool_logv;
   a.n_nodes = n_nodes; a.parent = parent; a.token = token; a.pool_index = pool_index; a.logv = logv;
-  trim_tree_kernel<<<batch, kDynThreads, static_cast<size_t>(pool_used) * 24, static_cast<cudaStream_t>(stream)>>>(a);
-  return cudaGetLastError() == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
+  return launch_after_previous(trim_tree_kernel, static_cast<unsigned>(batch), kDynThreads, static_cast<size_t>(pool_used) * 24,
+                               static_cast<cudaStream_t>(stream), 1, a) == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
 }
