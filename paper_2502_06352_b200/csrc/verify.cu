@@ -62,9 +62,9 @@ static cudaError_t launch_sparse_any(const VerifyArgs& a, int32_t* redo, int e, 
 }
 
 // ---- launch of the streaming kernel (rows without top-k): one CTA, or a cluster of cs CTAs, per node
-template <typename T, bool CFG, bool TAU1, bool GENERAL>
+template <typename T, bool CFG, bool TAU1, int MODE>
 static cudaError_t launch_stream_k(const VerifyArgs& a, int cs, size_t smem, cudaStream_t st) {
-  auto kern = stream::verify_stream_kernel<T, CFG, TAU1, GENERAL>;
+  auto kern = stream::verify_stream_kernel<T, CFG, TAU1, MODE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   if (cs > 8) {
@@ -76,8 +76,9 @@ static cudaError_t launch_stream_k(const VerifyArgs& a, int cs, size_t smem, cud
 }
 template <typename T, bool CFG, bool TAU1>
 static cudaError_t launch_stream_t(const VerifyArgs& a, int cs, size_t smem, cudaStream_t st) {
-  return (a.lazy || a.skip || a.det || a.tree_stride) ? launch_stream_k<T, CFG, TAU1, true>(a, cs, smem, st)
-                                     : launch_stream_k<T, CFG, TAU1, false>(a, cs, smem, st);
+  if (a.det && !a.lazy && !a.skip) return launch_stream_k<T, CFG, TAU1, 2>(a, cs, smem, st);
+  return (a.lazy || a.skip || a.det || a.tree_stride) ? launch_stream_k<T, CFG, TAU1, 1>(a, cs, smem, st)
+                                                      : launch_stream_k<T, CFG, TAU1, 0>(a, cs, smem, st);
 }
 static cudaError_t launch_stream_any(const VerifyArgs& a, int cs, size_t smem, bool f32, bool cfg, cudaStream_t st) {
   const bool tau1 = a.inv_tau == 1.0f;

@@ -101,6 +101,7 @@ template <typename T, bool CFG, bool TAU1>
 struct RowIO {
   using VT = Vec<T>;
   static constexpr int VN = VT::N;
+  static constexpr bool kGuided = CFG;
   const T* c;
   const T* u;
   float g, it;
@@ -329,8 +330,9 @@ __device__ __forceinline__ void pass_residual(const IO& ioq, const IO& iop, cons
 
 // One tree node (sequence b, node n).  Returns the accepted child or -1, the same value in
 // every thread of the node's CTAs.
-// VAR: the acceptance-rule variants (greedy-skip subset, deterministic drafts) are compiled in.
-template <typename T, bool CFG, bool TAU1, bool VAR>
+// MODE 0: the default acceptance rule, one tree shape.  1: the variants (greedy-skip subset, deterministic drafts,
+// forests) as the arguments say.  2: deterministic drafts with the default subset rule.
+template <typename T, bool CFG, bool TAU1, int MODE>
 __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, const int n, SCtx& c, const StreamSmem& sm) {
   using IO = RowIO<T, CFG, TAU1>;
   constexpr int VN = IO::VN;
@@ -338,15 +340,15 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
   constexpr int U1 = CFG ? 2 : 4;       // vectors in flight per thread and operand, single row
   constexpr int U2 = CFG ? 1 : 2;       // ... when two rows are read together
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int toff = VAR ? b * a.tree_stride : 0;            // a forest keeps one set of tree arrays per sequence
+  const int toff = MODE != 0 ? b * a.tree_stride : 0;            // a forest keeps one set of tree arrays per sequence
   const int fc = a.first_child[toff + n], nc = a.n_child[toff + n];
   const long long row_off = static_cast<long long>(b) * a.seq_stride + static_cast<long long>(n) * a.row_stride;
   const int32_t* tok_b = a.tokens + static_cast<long long>(b) * a.N;
   const long long out_b = static_cast<long long>(b) * a.N;
   const int kp1 = a.k + 1;
   const bool writer = c.rank == 0 && tid == 0;
-  const bool det = VAR && a.det != 0;       // deterministic drafts (Sec. 3): p(x) = 1, no drafter row
-  const bool skip = VAR && a.skip != 0;     // greedy-skip subset rule
+  const bool det = MODE == 2 || (MODE == 1 && a.det != 0);      // deterministic drafts (Sec. 3): p(x) = 1, no drafter row
+  const bool skip = MODE == 1 && a.skip != 0;      // greedy-skip subset rule
   const bool has_p = nc > 0 && !det;
   float* fm = reinterpret_cast<float*>(sm.misc);
   int* dropped = sm.misc + 16;          // [LANTERN_MAX_CHILDREN] rejected draft tokens
@@ -760,9 +762,13 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
     float zs[2];
     {
       float accq, accp;
-      if (det) pass_residual<IO, U1, false, false>(ioq, iop, ge, vbeg, vend, lane, nx, sm.bits, dropped, n_dropped, accq, accp);
-      else if (resum) pass_residual<IO, U2, true>(ioq, iop, ge, vbeg, vend, lane, nx, sm.bits, dropped, n_dropped, accq, accp);
-      else pass_residual<IO, U2, false>(ioq, iop, ge, vbeg, vend, lane, nx, sm.bits, dropped, n_dropped, accq, accp);
+      if constexpr (MODE == 2) {
+        pass_residual<IO, U1, false, false>(ioq, iop, ge, vbeg, vend, lane, nx, sm.bits, dropped, n_dropped, accq, accp);
+      } else {
+        if (det) pass_residual<IO, U1, false, false>(ioq, iop, ge, vbeg, vend, lane, nx, sm.bits, dropped, n_dropped, accq, accp);
+        else if (resum) pass_residual<IO, U2, true>(ioq, iop, ge, vbeg, vend, lane, nx, sm.bits, dropped, n_dropped, accq, accp);
+        else pass_residual<IO, U2, false>(ioq, iop, ge, vbeg, vend, lane, nx, sm.bits, dropped, n_dropped, accq, accp);
+      }
       zs[0] = warp_sum(accq);
       zs[1] = warp_sum(accp);
     }
@@ -901,9 +907,10 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
   return accepted;
 }
 
-// GENERAL = false: one node per CTA (cluster), default acceptance rule (the benchmarked launch).
-// GENERAL = true: the same plus what is decided at run time: the path walk and the rule variants.
-template <typename T, bool CFG, bool TAU1, bool GENERAL>
+// MODE 0 (the benchmarked launch) and 2: one node per CTA (cluster); 1: the path walk too.  The modes are builds of their own
+// because what is decided at run time costs registers: the build with everything spills 1.2 to 1.7 KB per thread,
+// and 3776 nodes of deterministic drafts (65536 bfloat16 logits) took 289 us in it, 143 in mode 2.
+template <typename T, bool CFG, bool TAU1, int MODE>
 __global__ void __launch_bounds__(ST, LANTERN_STREAM_MINB) verify_stream_kernel(const VerifyArgs a) {
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char stream_smem[];
@@ -935,10 +942,10 @@ __global__ void __launch_bounds__(ST, LANTERN_STREAM_MINB) verify_stream_kernel(
   // sequence and walks it (Sec. 2.1): it verifies the root, moves to the accepted child and so
   // on, so only the rows on the accepted path are read and the per-node results of the other
   // nodes are not written.
-  const bool lazy = GENERAL && a.lazy != 0;
+  const bool lazy = MODE == 1 && a.lazy != 0;
   const int b = lazy ? idx : idx % a.B;
-  int cur = lazy ? 0 : a.order[(GENERAL ? b * a.tree_stride : 0) + idx / a.B];
-  if (GENERAL && cur < 0) {            // padding of a forest's shorter tree: nothing to verify (the whole cluster leaves)
+  int cur = lazy ? 0 : a.order[(MODE != 0 ? b * a.tree_stride : 0) + idx / a.B];
+  if (MODE != 0 && cur < 0) {            // padding of a forest's shorter tree: nothing to verify (the whole cluster leaves)
     if (c.rank == 0 && threadIdx.x == 0) {
       const long long o = static_cast<long long>(b) * a.N + idx / a.B;       // padding sits at the end of the order
       a.node_next[o] = -1;
@@ -950,7 +957,7 @@ __global__ void __launch_bounds__(ST, LANTERN_STREAM_MINB) verify_stream_kernel(
   }
   int len = 0;
   for (;;) {
-    const int acc = stream_node<T, CFG, TAU1, GENERAL>(a, b, cur, c, sm);
+    const int acc = stream_node<T, CFG, TAU1, MODE>(a, b, cur, c, sm);
     if (!lazy) break;
     csync(c);     // the next node reuses the shared memory; also orders the store of node_token before the read below
     const bool writer = c.rank == 0 && threadIdx.x == 0;
