@@ -227,11 +227,11 @@ lantern_status lantern_verify_tree(const lantern_params* params, const lantern_t
 /* ---- which kernels a call launches ---------------------------------------------------------------
  * Rows that no top-k truncates are handled by streaming kernels (LANTERN_PATH_STREAM): every row is
  * read from HBM once and never held on chip; a rejection is one more read-only pass over the
- * node's two rows, served by L2.  Rows that App. B's top-k truncation cuts to at most 1280 entries,
- * in vocabularies of at most 16384 tokens, are handled by list-based kernels (LANTERN_PATH_LISTS:
+ * node's two rows, served by L2.  Rows that App. B's top-k truncation cuts to at most 2048 entries,
+ * in vocabularies of at most 131072 tokens, are handled by list-based kernels (LANTERN_PATH_LISTS:
  * the row is compacted to its survivors; everything after works on those), followed by a launch of
  * the dense kernels that redoes the nodes whose rows did not fit the lists' fixed buffers (massive
- * ties; usually none).  All other calls (top-k on wide vocabularies, the path walk) run the dense
+ * ties; usually none).  All other calls (larger k, the path walk of top-k rows) run the dense
  * kernels alone (LANTERN_PATH_DENSE: rows held in shared memory).  So do small calls without top-k
  * whose rows fit the dense kernels: verification of fewer than 128 tree nodes in the whole batch (a
  * handful of nodes is a chain of dependent steps, which shared-memory rows shorten), and drafting of

@@ -39,8 +39,9 @@ struct SampleArgs {
 };
 
 }  // namespace lantern
-#include "sampler_sparse.cuh"
 #include "sampler_stream.cuh"
+#include "sampler_sparse.cuh"
+#include "sampler_wide.cuh"
 namespace lantern {
 
 constexpr float kDenseKeyErr = 2e-5f;     // bound on |float32 key - exact key| (|key| < 64)
@@ -395,6 +396,17 @@ static cudaError_t launch_sample_sparse(const SampleArgs& a, int V, cudaStream_t
 }
 
 
+// ---- the same for wide rows
+template <typename T, bool CFG>
+static cudaError_t launch_sample_wide(const SampleArgs& a, cudaStream_t st) {
+  auto kern = wide::sample_wide_kernel<T, CFG>;
+  const int cap = wide::list_cap(a.topk_d);
+  const size_t smem = wide::sampler_smem_bytes(a.V, cap);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  return launch_after_previous(kern, static_cast<unsigned>(a.B) * a.n_parents, sparse::ST, smem, st, 1, a, cap);
+}
+
 // ---- launch of the streaming kernel (rows without top-k): one CTA, or a cluster, per parent
 template <typename T, bool CFG, bool TAU1>
 static cudaError_t launch_sample_stream_t(const SampleArgs& a, int cs, cudaStream_t st) {
@@ -426,11 +438,13 @@ using namespace lantern;
 extern "C" int32_t lantern_get_cluster_size(void);
 
 namespace {
-// Rows truncated to a moderate top-k can take the list-based kernel.
+// Rows truncated to a moderate top-k can take the list-based kernels: rows that fit the shared-memory buffer the staged
+// one, others (and larger k) the one that streams them.
+bool sampler_stages_rows(const lantern_params* p) { return p->vocab <= sparse::kMaxV && p->top_k_draft <= sparse::kMaxTopK; }
 bool sampler_uses_lists(const lantern_params* p) {
   const int V = p->vocab;
-  const int ov = lantern_get_cluster_size();
-  return ov == 0 && V <= sparse::kMaxV && p->top_k_draft > 0 && p->top_k_draft < V && p->top_k_draft <= sparse::kMaxTopK;
+  if (lantern_get_cluster_size() != 0 || p->top_k_draft <= 0 || p->top_k_draft >= V) return false;
+  return sampler_stages_rows(p) || (V <= wide::kMaxV && p->top_k_draft <= wide::kMaxTopK);
 }
 }  // namespace
 
@@ -540,10 +554,14 @@ extern "C" lantern_status lantern_sample_draft_tree(
   // Rows truncated to a moderate top-k take the list-based kernel; the dense kernel then draws
   // the parents it marked as not fitting (usually none).
   if (sampler_uses_lists(p)) {
-    if (dt == LANTERN_F32)
-      err = cfg ? launch_sample_sparse<float, true>(a, V, st) : launch_sample_sparse<float, false>(a, V, st);
-    else
-      err = cfg ? launch_sample_sparse<__nv_bfloat16, true>(a, V, st) : launch_sample_sparse<__nv_bfloat16, false>(a, V, st);
+    const bool f32 = dt == LANTERN_F32;
+    if (sampler_stages_rows(p)) {
+      if (f32) err = cfg ? launch_sample_sparse<float, true>(a, V, st) : launch_sample_sparse<float, false>(a, V, st);
+      else err = cfg ? launch_sample_sparse<__nv_bfloat16, true>(a, V, st) : launch_sample_sparse<__nv_bfloat16, false>(a, V, st);
+    } else {
+      if (f32) err = cfg ? launch_sample_wide<float, true>(a, st) : launch_sample_wide<float, false>(a, st);
+      else err = cfg ? launch_sample_wide<__nv_bfloat16, true>(a, st) : launch_sample_wide<__nv_bfloat16, false>(a, st);
+    }
     if (err != cudaSuccess) return LANTERN_ERR_CUDA;
     a.repair = 1;
   }

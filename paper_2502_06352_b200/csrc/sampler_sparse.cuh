@@ -16,9 +16,11 @@ constexpr int kRedoToken = -2;
 constexpr int kPerThread = kCap / ST;     // list entries per thread
 constexpr float kKeyErr = 2e-5f;          // bound on |float32 key - exact key| (|key| < 64)
 
+constexpr int kDrawInts = 2 * 2 * SW + 8 + 8 + 8 + 32 + 4;   // words of ListDraw::pk
+
 __host__ __device__ constexpr size_t sampler_smem_bytes(int e) {
   return static_cast<size_t>(ST) * e * 4 + 3 * kCap * 4 + kBins * 4 + kWords * 4 + kCand * 4 + 2 * SW * 2 * 4 +
-         SW * 4 + kMisc * 4 + 2 * 2 * SW * 4 + (8 + 8 + 8 + 32 + 4) * 4;
+         SW * 4 + kMisc * 4 + kDrawInts * 4;
 }
 
 __device__ __forceinline__ bool key_better(float ka, int ia, float kb, int ib) {   // a beats b
@@ -33,75 +35,44 @@ __device__ __forceinline__ void warp_key_best(float& k, int& i) {
   }
 }
 
-template <typename T, bool CFG, int E>
-__global__ void __launch_bounds__(ST, 2) sample_sparse_kernel(const SampleArgs a) {
-  grid_dependency_sync();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Smem s;
-  s.Z = reinterpret_cast<float*>(smem_raw);
-  s.ltok[0] = reinterpret_cast<int*>(s.Z + ST * E);
-  s.lval[0] = reinterpret_cast<float*>(s.ltok[0] + kCap);
-  float* keys = s.lval[0] + kCap;                 // [kCap]
-  s.ltok[1] = nullptr;
-  s.lval[1] = nullptr;
-  s.bins = reinterpret_cast<uint32_t*>(keys + kCap);
-  s.bm[0] = s.bins + kBins;
-  s.bm[1] = nullptr;
-  s.rk = nullptr;
-  s.cand = reinterpret_cast<float*>(s.bm[0] + kWords);
-  Ctx c;
-  c.red = s.cand + kCand;
-  c.last_red = c.red;
-  c.parity = 0;
-  s.wtot = reinterpret_cast<uint32_t*>(c.red + 2 * SW * 2);
-  s.misc = reinterpret_cast<int*>(s.wtot + SW);
-  float* pk = reinterpret_cast<float*>(s.misc + kMisc);    // [2][2*SW] warps' best key and token, two buffers
-  float* wkey = pk + 2 * 2 * SW;                           // [8] keys of the rounds' winners
-  int* wtok = reinterpret_cast<int*>(wkey + 8);            // [8] their tokens (-1: none), [8] their list positions
-  int* wpos = wtok + 8;
-  int* cpos = wpos + 8;                                    // [32] list positions of the entries ranked exactly
-  int* ccnt = cpos + 32;
-
+// A parent's survivors in shared memory, and the draw from them: keys, s selection rounds, exact order of near-ties.
+struct ListDraw {
+  const int* tok;      // [n] token, pre-softmax value (below theta: not a survivor)
+  const float* z;
+  float* keys;         // [n]
+  // [2][2*SW] warps' best key and token, two buffers; [8] keys of the rounds' winners, [8] their tokens (-1: none), [8] their
+  // list positions; [32] list positions of the entries ranked exactly, their number
+  float* pk;           // kDrawInts words
+  int n;
+  float mx, theta;
+};
+// PT: list entries per thread at most
+template <int PT>
+__device__ __forceinline__ void draw_from_list(const SampleArgs& a, Ctx& c, const ListDraw& s, int b, int n, int fc, int nc) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int idx = blockIdx.x;
-  const int b = idx % a.B;
-  const int n = a.order[a.order_begin + idx / a.B];
-  const int fc = a.first_child[n], nc = a.n_child[n];
-  const int len = min(a.V, ST * E);
-  const long long row_off = static_cast<long long>(b) * a.seq_stride + static_cast<long long>(n) * a.row_stride;
+  const int n_list = s.n;
+  const float theta = s.theta;
+  float* keys = s.keys;
+  float* pk = s.pk;
+  float* wkey = pk + 2 * 2 * SW;
+  int* wtok = reinterpret_cast<int*>(wkey + 8);
+  int* wpos = wtok + 8;
+  int* cpos = wpos + 8;
+  int* ccnt = cpos + 32;
   const long long out_b = static_cast<long long>(b) * a.N;
-
-  const bool masked = a.allow_lo > 0 || a.allow_hi < a.V;
-  const T* cond = static_cast<const T*>(a.dc) + row_off;
-  const T* uncond = CFG ? static_cast<const T*>(a.du) + row_off : nullptr;
-  for (int i = tid; i < kBins; i += ST) s.bins[i] = 0;
-  s.bm[0][tid] = 0;
-  float mx[2];
-  mx[0] = load_row<T, CFG, E>(cond, uncond, a.g, a.inv_tau, len, a.allow_lo, a.allow_hi, masked, s.Z);
-  mx[1] = -INFINITY;
-  block_reduce2<true>(c, mx);
-  int n_list = 0;
-  float theta = INFINITY;
-  bool ok = mx[0] != -INFINITY;
-  if (ok) ok = compact_topk<E, true>(s, 0, mx[0], a.topk_d, n_list, theta);
-  if (!ok) {
-    if (tid == 0) a.tokens[out_b + fc] = kRedoToken;
-    return;
-  }
-
   // ---- keys z + G, G = -log(-log U), of the survivors; softmax denominator
   const uint32_t row_id = static_cast<uint32_t>(out_b + n);
   const float* gum = a.gumbel ? a.gumbel + static_cast<long long>(row_id) * a.V : nullptr;
-  const float c0 = -mx[0] * kLog2e;
+  const float c0 = -s.mx * kLog2e;
   float sm[2] = {0.f, 0.f};
   float bk = -INFINITY;
   int bi = 0x7fffffff, bpos = -1;
 #pragma unroll
-  for (int m = 0; m < kPerThread; ++m) {
+  for (int m = 0; m < PT; ++m) {
     const int i = tid + m * ST;
     if (i >= n_list) break;
-    const int t = s.ltok[0][i];
-    const float z = s.lval[0][i];
+    const int t = s.tok[i];
+    const float z = s.z[i];
     float key = -INFINITY;
     if (z >= theta && z != -INFINITY) {
       float u;
@@ -138,17 +109,17 @@ __global__ void __launch_bounds__(ST, 2) sample_sparse_kernel(const SampleArgs a
       wpos[round] = bpos;
       a.tokens[out_b + fc + round] = ci;
       if (a.draft_prob)
-        a.draft_prob[out_b + fc + round] = ex2_approx(fmaf(s.lval[0][bpos], kLog2e, c0)) * inv_sum;
+        a.draft_prob[out_b + fc + round] = ex2_approx(fmaf(s.z[bpos], kLog2e, c0)) * inv_sum;
       keys[bpos] = -INFINITY;
       bk = -INFINITY;
       bi = 0x7fffffff;
       bpos = -1;
 #pragma unroll
-      for (int m = 0; m < kPerThread; ++m) {
+      for (int m = 0; m < PT; ++m) {
         const int i = tid + m * ST;
         if (i >= n_list) break;
         const float key = keys[i];
-        const int t = s.ltok[0][i];
+        const int t = s.tok[i];
         if (key != -INFINITY && key_better(key, t, bk, bi)) { bk = key; bi = t; bpos = i; }
       }
     }
@@ -170,7 +141,7 @@ __global__ void __launch_bounds__(ST, 2) sample_sparse_kernel(const SampleArgs a
   for (int r = 1; r < nv; ++r) close |= wkey[r - 1] - wkey[r] <= 2.f * kKeyErr;
   bool mine = false;
 #pragma unroll
-  for (int m = 0; m < kPerThread; ++m) {
+  for (int m = 0; m < PT; ++m) {
     const int i = tid + m * ST;
     if (i >= n_list) break;
     mine |= keys[i] != -INFINITY && keys[i] >= k_last - 2.f * kKeyErr;
@@ -180,7 +151,7 @@ __global__ void __launch_bounds__(ST, 2) sample_sparse_kernel(const SampleArgs a
   if (tid == 0) *ccnt = nv;
   __syncthreads();
 #pragma unroll
-  for (int m = 0; m < kPerThread; ++m) {
+  for (int m = 0; m < PT; ++m) {
     const int i = tid + m * ST;
     if (i >= n_list) break;
     if (keys[i] != -INFINITY && keys[i] >= k_last - 2.f * kKeyErr) {
@@ -200,8 +171,8 @@ __global__ void __launch_bounds__(ST, 2) sample_sparse_kernel(const SampleArgs a
     float z = 0.f;
     if (lane < ncand) {
       const int i = cpos[lane];
-      t = s.ltok[0][i];
-      z = s.lval[0][i];
+      t = s.tok[i];
+      z = s.z[i];
       float u;
       if (gum) {
         u = __ldcs(gum + t);
@@ -223,6 +194,64 @@ __global__ void __launch_bounds__(ST, 2) sample_sparse_kernel(const SampleArgs a
       if (a.draft_prob) a.draft_prob[out_b + fc + rank] = ex2_approx(fmaf(z, kLog2e, c0)) * inv_sum;
     }
   }
+}
+
+
+template <typename T, bool CFG, int E>
+__global__ void __launch_bounds__(ST, 2) sample_sparse_kernel(const SampleArgs a) {
+  grid_dependency_sync();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Smem s;
+  s.Z = reinterpret_cast<float*>(smem_raw);
+  s.ltok[0] = reinterpret_cast<int*>(s.Z + ST * E);
+  s.lval[0] = reinterpret_cast<float*>(s.ltok[0] + kCap);
+  float* keys = s.lval[0] + kCap;                 // [kCap]
+  s.ltok[1] = nullptr;
+  s.lval[1] = nullptr;
+  s.bins = reinterpret_cast<uint32_t*>(keys + kCap);
+  s.bm[0] = s.bins + kBins;
+  s.bm[1] = nullptr;
+  s.rk = nullptr;
+  s.cand = reinterpret_cast<float*>(s.bm[0] + kWords);
+  Ctx c;
+  c.red = s.cand + kCand;
+  c.last_red = c.red;
+  c.parity = 0;
+  s.wtot = reinterpret_cast<uint32_t*>(c.red + 2 * SW * 2);
+  s.misc = reinterpret_cast<int*>(s.wtot + SW);
+  float* pk = reinterpret_cast<float*>(s.misc + kMisc);    // [2][2*SW] warps' best key and token, two buffers
+
+  const int tid = threadIdx.x;
+  const int idx = blockIdx.x;
+  const int b = idx % a.B;
+  const int n = a.order[a.order_begin + idx / a.B];
+  const int fc = a.first_child[n], nc = a.n_child[n];
+  const int len = min(a.V, ST * E);
+  const long long row_off = static_cast<long long>(b) * a.seq_stride + static_cast<long long>(n) * a.row_stride;
+  const long long out_b = static_cast<long long>(b) * a.N;
+
+  const bool masked = a.allow_lo > 0 || a.allow_hi < a.V;
+  const T* cond = static_cast<const T*>(a.dc) + row_off;
+  const T* uncond = CFG ? static_cast<const T*>(a.du) + row_off : nullptr;
+  for (int i = tid; i < kBins; i += ST) s.bins[i] = 0;
+  s.bm[0][tid] = 0;
+  float mx[2];
+  mx[0] = load_row<T, CFG, E>(cond, uncond, a.g, a.inv_tau, len, a.allow_lo, a.allow_hi, masked, s.Z);
+  mx[1] = -INFINITY;
+  block_reduce2<true>(c, mx);
+  int n_list = 0;
+  float theta = INFINITY;
+  bool ok = mx[0] != -INFINITY;
+  if (ok) ok = compact_topk<E, true>(s, 0, mx[0], a.topk_d, n_list, theta);
+  if (!ok) {
+    if (tid == 0) a.tokens[out_b + fc] = kRedoToken;
+    return;
+  }
+
+  ListDraw ld;
+  ld.tok = s.ltok[0]; ld.z = s.lval[0]; ld.keys = keys; ld.pk = pk;
+  ld.n = n_list; ld.mx = mx[0]; ld.theta = theta;
+  draw_from_list<kPerThread>(a, c, ld, b, n, fc, nc);
 }
 
 }  // namespace sparse

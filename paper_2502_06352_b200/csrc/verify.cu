@@ -34,6 +34,7 @@ static int sm_count() {
 #undef LANTERN_VNS
 #include "verify_sparse.cuh"
 #include "verify_stream.cuh"
+#include "verify_wide.cuh"
 
 namespace lantern {
 
@@ -59,6 +60,22 @@ static cudaError_t launch_sparse_any(const VerifyArgs& a, int32_t* redo, int e, 
   if (f32) return cfg ? launch_sparse<float, true>(a, redo, e, smem, st) : launch_sparse<float, false>(a, redo, e, smem, st);
   return cfg ? launch_sparse<__nv_bfloat16, true>(a, redo, e, smem, st)
              : launch_sparse<__nv_bfloat16, false>(a, redo, e, smem, st);
+}
+
+// ---- the same for wide rows
+template <typename T, bool CFG>
+static cudaError_t launch_wide(const VerifyArgs& a, int32_t* redo, int cap, size_t smem, cudaStream_t st) {
+  auto kern = wide::verify_wide_kernel<T, CFG>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  const int chunk = sm_count();
+  const int nI = a.B * a.n_internal, nL = a.B * (a.N - a.n_internal);
+  const int blocks = (nI + chunk - 1) / chunk + (nL + chunk - 1) / chunk;
+  return launch_after_previous(kern, static_cast<unsigned>(blocks) * chunk, sparse::ST, smem, st, 1, a, redo, chunk, cap);
+}
+static cudaError_t launch_wide_any(const VerifyArgs& a, int32_t* redo, int cap, size_t smem, bool f32, bool cfg, cudaStream_t st) {
+  if (f32) return cfg ? launch_wide<float, true>(a, redo, cap, smem, st) : launch_wide<float, false>(a, redo, cap, smem, st);
+  return cfg ? launch_wide<__nv_bfloat16, true>(a, redo, cap, smem, st) : launch_wide<__nv_bfloat16, false>(a, redo, cap, smem, st);
 }
 
 // ---- launch of the streaming kernel (rows without top-k): one CTA, or a cluster of cs CTAs, per node
@@ -90,14 +107,16 @@ static cudaError_t launch_stream_any(const VerifyArgs& a, int cs, size_t smem, b
   return tau1 ? launch_stream_t<__nv_bfloat16, false, true>(a, cs, smem, st)
               : launch_stream_t<__nv_bfloat16, false, false>(a, cs, smem, st);
 }
-// CTAs per node: one when the nodes alone fill the machine, else the smallest power of two that
-// does, as long as every warp of the wider cluster keeps at least two full 512-byte steps of the row
-// (narrow rows, e.g. an allowed range of 8192 tokens, run faster on fewer, busier CTAs)
+// CTAs per node: one when the nodes alone fill the machine with its four CTAs per SM, else the smallest power of two
+// that does, as long as every warp of the wider cluster keeps at least two full 512-byte steps of the row
+// (narrow rows, e.g. an allowed range of 8192 tokens, run faster on fewer, busier CTAs).  240 nodes of 65536
+// float32 logits with guidance on 1 / 2 / 4 / 8 CTAs: 185 / 112 / 79 / 85 us; 215 nodes of 40003 bfloat16 logits: 108 / 72 /
+// 53 / 62 us.
 static int stream_cluster_size(int nodes, int V, bool f32) {
   if (g_cluster_override > 0) return g_cluster_override;
   const int nvec = V / (f32 ? 4 : 8);
   int cs = 1;
-  while (cs < 16 && static_cast<long long>(nodes) * cs < 8 * sm_count() && nvec / (4 * cs * stream::SW) >= 32) cs *= 2;
+  while (cs < 16 && static_cast<long long>(nodes) * cs < 4 * sm_count() && nvec / (4 * cs * stream::SW) >= 32) cs *= 2;
   return cs;
 }
 
@@ -145,13 +164,23 @@ extern "C" int32_t lantern_get_cluster_size(void) { return g_cluster_override; }
 
 namespace {
 constexpr int kWsTailInts = 64;
-// Rows truncated to a moderate top-k on every side that is read can take the list-based kernel.
+// Rows truncated to a moderate top-k on every side that is read can take the list-based kernels: rows that fit the
+// shared-memory buffer the staged one, others (and larger k) the one that streams them.
+int largest_topk(const lantern_params* p, const TreeDev* t) {
+  return t->n_internal > 0 ? std::max(p->top_k_target, p->top_k_draft) : p->top_k_target;
+}
+bool verify_stages_rows(const lantern_params* p, const TreeDev* t) {
+  return p->vocab <= sparse::kMaxV && largest_topk(p, t) <= sparse::kMaxTopK;
+}
 bool verify_uses_lists(const lantern_params* p, const TreeDev* t) {
-  const int V = p->vocab;
-  auto topk_fits = [&](int k) { return k > 0 && k < V && k <= sparse::kMaxTopK; };
-  return !p->lazy_walk && !p->subset_rule && !p->draft_deterministic && g_cluster_override == 0 &&
-         V <= sparse::kMaxV && topk_fits(p->top_k_target) &&
-         (t->n_internal == 0 || topk_fits(p->top_k_draft)) && t->max_children <= 8;
+  const int V = p->vocab, top = largest_topk(p, t);
+  auto truncates = [&](int k) { return k > 0 && k < V; };
+  if (p->lazy_walk || p->subset_rule || p->draft_deterministic || g_cluster_override != 0 || t->max_children > 8 ||
+      !truncates(p->top_k_target) || (t->n_internal > 0 && !truncates(p->top_k_draft)))
+    return false;
+  return verify_stages_rows(p, t) ||
+         (V <= wide::kMaxV && top <= wide::kMaxTopK &&
+          wide::smem_bytes(V, wide::list_cap(top), t->max_children, (p->k + 3) & ~3) <= 227 * 1024);
 }
 // Can the streaming kernel serve these parameters at all (rows that no top-k truncates)?
 bool stream_applies(const lantern_params* p, const TreeDev* t) {
@@ -280,9 +309,14 @@ extern "C" lantern_status lantern_verify_tree(
   // dense kernel then repairs the nodes it could not hold (a.only) and usually finds none.
   const bool use_sparse = redo && !a.lazy && !t->per_seq && verify_uses_lists(p, t);
   if (use_sparse) {
-    const int se = V <= sparse::ST * 8 ? 8 : (V <= sparse::ST * 16 ? 16 : 32);
-    a.done = redo + static_cast<size_t>(batch) * t->n_nodes;       // the sparse kernel clears it
-    e = launch_sparse_any(a, redo, se, sparse::smem_bytes(se, t->max_children, a.kpad), f32, cfg, st);
+    a.done = redo + static_cast<size_t>(batch) * t->n_nodes;       // the list kernel clears it
+    if (verify_stages_rows(p, t)) {
+      const int se = V <= sparse::ST * 8 ? 8 : (V <= sparse::ST * 16 ? 16 : 32);
+      e = launch_sparse_any(a, redo, se, sparse::smem_bytes(se, t->max_children, a.kpad), f32, cfg, st);
+    } else {
+      const int cap = wide::list_cap(largest_topk(p, t));
+      e = launch_wide_any(a, redo, cap, wide::smem_bytes(V, cap, t->max_children, a.kpad), f32, cfg, st);
+    }
     if (e != cudaSuccess) return LANTERN_ERR_CUDA;
     a.only = redo;
   }

@@ -288,11 +288,12 @@ __device__ __forceinline__ bool compact_topk(const Smem& s, int side, float mx, 
 // Shared memory and identity of the per-node part (union build, sibling loop, draw), which the
 // kernel runs after compacting its two rows.
 struct NodeSmem {
-  int* ut;           // [kUCap]  union arrays: token, target mass, drafter mass
+  int* ut;           // union arrays: token (not with WIDE), target mass, drafter mass
   float* uq;
   float* up;
-  uint32_t* bm[2];   // [kWords] support bitmaps of the two lists
-  uint32_t* rk;      // [kWords] union entries before bitmap word w
+  int words;         // bitmap words (with WIDE; kWords otherwise)
+  uint32_t* bm[2];   // [words]  support bitmaps of the two lists
+  uint32_t* rk;      // [words]  union entries before bitmap word w
   uint32_t* wtot;    // [NT/32]
   int* misc;         // [kMisc]
   uint64_t* mbar;
@@ -378,8 +379,9 @@ __device__ __forceinline__ bool node_prologue(const VerifyArgs& a, const NodeSme
 // The per-node part: merges the two lists (token, unnormalised probability; the bitmaps hold their
 // supports) into the union arrays, runs the sibling loop (Sec. 4; App. A.2 Eq. 1-2) and the
 // inverse-CDF draw, and writes the node's results.  NT threads; a barrier must separate the last
-// write of the bitmaps and lists from the call.
-template <int NT>
+// write of the bitmaps and lists from the call.  WIDE: vocabularies beyond kMaxV, whose tokens at union positions are
+// found through the bitmaps instead of a third array.
+template <int NT, bool WIDE = false>
 __device__ __forceinline__ void node_tail(const VerifyArgs& a, Ctx& c, const NodeSmem& ns, const NodeId& id,
                                           const bool bulk_issued, const int* ltok0, const float* lval0, const int n0,
                                           const int* ltok1, const float* lval1, const int n1) {
@@ -401,12 +403,20 @@ __device__ __forceinline__ void node_tail(const VerifyArgs& a, Ctx& c, const Nod
   float* up = ns.up;
   int n_u;
   {
-    constexpr int WPT = kWords / NT;            // bitmap words per thread
-    int before[WPT], cnt = 0;
+    // consecutive bitmap words of this thread: kWords / NT of them, or with WIDE what the vocabulary takes
+    constexpr int WPT = WIDE ? 1 : kWords / NT;
+    int before[WPT], cnt = 0, w0 = 0, w1 = 0;
+    if constexpr (WIDE) {
+      const int wpt = (ns.words + NT - 1) / NT;
+      w0 = min(tid * wpt, ns.words);
+      w1 = min(w0 + wpt, ns.words);
+      for (int w = w0; w < w1; ++w) cnt += __popc(ns.bm[0][w] | ns.bm[1][w]);
+    } else {
 #pragma unroll
-    for (int j = 0; j < WPT; ++j) {
-      before[j] = cnt;
-      cnt += __popc(ns.bm[0][tid * WPT + j] | ns.bm[1][tid * WPT + j]);
+      for (int j = 0; j < WPT; ++j) {
+        before[j] = cnt;
+        cnt += __popc(ns.bm[0][tid * WPT + j] | ns.bm[1][tid * WPT + j]);
+      }
     }
     int incl = cnt;
 #pragma unroll
@@ -422,9 +432,16 @@ __device__ __forceinline__ void node_tail(const VerifyArgs& a, Ctx& c, const Nod
       const int t = __shfl_up_sync(0xffffffffu, wincl, o);
       if (lane >= o) wincl += t;
     }
-    const int base = __shfl_sync(0xffffffffu, wincl - wt, warp) + incl - cnt;
+    int base = __shfl_sync(0xffffffffu, wincl - wt, warp) + incl - cnt;
+    if constexpr (WIDE) {
+      for (int w = w0; w < w1; ++w) {
+        ns.rk[w] = static_cast<uint32_t>(base);
+        base += __popc(ns.bm[0][w] | ns.bm[1][w]);
+      }
+    } else {
 #pragma unroll
-    for (int j = 0; j < WPT; ++j) ns.rk[tid * WPT + j] = static_cast<uint32_t>(base + before[j]);
+      for (int j = 0; j < WPT; ++j) ns.rk[tid * WPT + j] = static_cast<uint32_t>(base + before[j]);
+    }
     n_u = __shfl_sync(0xffffffffu, wincl, NW - 1);
   }
   // ---- neighbour rows must have landed
@@ -456,7 +473,7 @@ __device__ __forceinline__ void node_tail(const VerifyArgs& a, Ctx& c, const Nod
     const int nl = side ? n1 : n0;
     for (int i = tid; i < nl; i += NT) {
       const int t = lt[i], u = uidx(t);
-      ut[u] = t;
+      if (!WIDE) ut[u] = t;
       mine[u] = lv[i];
       if (!((obm[t >> 5] >> (t & 31)) & 1u)) other[u] = 0.f;
     }
@@ -643,7 +660,20 @@ __device__ __forceinline__ void node_tail(const VerifyArgs& a, Ctx& c, const Nod
       lastp = __reduce_max_sync(0xffffffffu, lane < NW ? misc[80 + lane] : -1);
       if (lane == 0) {
         const int found = cand != 0x7fffffff ? cand : lastp;
-        a.node_token[out_b + n] = found >= 0 ? ut[found] : -1;
+        int tok = -1;
+        if constexpr (!WIDE) {
+          tok = found >= 0 ? ut[found] : -1;
+        } else if (found >= 0) {                // the token at a position: its bitmap word, then its bit
+          int lo = 0, hi = ns.words - 1;        // the last word with rk <= found
+          while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (static_cast<int>(ns.rk[mid]) <= found) lo = mid; else hi = mid - 1;
+          }
+          uint32_t bits = ns.bm[0][lo] | ns.bm[1][lo];
+          for (int skip = found - static_cast<int>(ns.rk[lo]); skip > 0; --skip) bits &= bits - 1u;
+          tok = lo * 32 + __ffs(bits) - 1;
+        }
+        a.node_token[out_b + n] = tok;
         if (found < 0) vflag(a.status, LANTERN_DEV_EMPTY_ROW);
       }
     }

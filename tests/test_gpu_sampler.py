@@ -241,3 +241,18 @@ def test_streaming_kernel_on_wide_ranges_and_nearly_empty_rows(L, dtype):
     gum = W.make_gumbel_uniforms(case.B, case.N, case.V, 7)
     gtok, gprob, _ = _gpu_sample(L, case, gumbel=gum)
     assert _compare(case, gum.numpy(), gtok, gprob) <= 1
+
+
+@pytest.mark.parametrize("kw", [dict(vocab=16385, codebook_size=500, top_k=50), dict(vocab=20001, codebook_size=500, top_k=2048, cfg_scale=None),
+                                dict(vocab=65536, codebook_size=500, top_k=2000, dtype="bf16"), dict(vocab=4096, codebook_size=500, top_k=6),
+                                dict(vocab=33000, codebook_size=500, top_k=1000, allowed=(4099, 12290)),
+                                dict(vocab=33000, codebook_size=500, top_k=300, allowed=(32001, 32100))])
+def test_topk_rows_of_every_width(L, kw):
+    kw = dict(kw)
+    allowed = kw.pop("allowed", (0, 0))
+    case = Case(small_config(batch=1, **kw), seed=33, tokens="random", allowed=allowed, pad=-kw["vocab"] % 8)
+    gum = W.make_gumbel_uniforms(case.B, case.N, case.V, 515)
+    gtok, gprob, _ = _gpu_sample(L, case, gumbel=gum)
+    assert _compare(case, gum.numpy(), gtok, gprob) <= 1
+    again, prob, _ = _gpu_sample(L, case, gumbel=gum)
+    assert np.array_equal(again, gtok) and np.array_equal(prob, gprob)          # bit for bit

@@ -80,6 +80,62 @@ def test_topk_rows_on_every_path(L, cs, kw):
         L.set_cluster_size(old)
 
 
+@pytest.mark.parametrize("kw", [
+    dict(vocab=16385, codebook_size=1000, top_k=50, k=12),                                       # just past the rows that fit one dense CTA
+    dict(vocab=20001, codebook_size=1000, code_offset=7, top_k=2048, k=40, cfg_scale=None),      # the largest k of the lists
+    dict(vocab=20001, codebook_size=1000, top_k=2049, k=8, cfg_scale=None),                      # one more: dense kernels
+    dict(vocab=65536, codebook_size=2000, code_offset=4096, top_k=2000, k=20, dtype="bf16"),
+    dict(vocab=70003, codebook_size=500, top_k=1, k=4, temperature=0.7),
+    dict(vocab=4096, codebook_size=500, top_k=100, k=8),                                         # as many entries as skip the sample
+    dict(vocab=4104, codebook_size=500, top_k=100, k=8, dtype="bf16"),
+    dict(vocab=33000, codebook_size=500, top_k=1000, k=8, allowed=(4099, 12290)),
+    dict(vocab=33000, codebook_size=500, top_k=300, k=8, allowed=(32001, 32100)),                # k above the number of allowed tokens
+])
+def test_topk_rows_of_every_width_on_the_lists(L, kw):
+    kw = dict(kw)
+    allowed = kw.pop("allowed", (0, 0))
+    V = kw["vocab"]
+    case = Case(small_config(batch=1, **kw), seed=51, pad=-V % 8, allowed=allowed, tokens="random")
+    for b in range(case.B):          # draft tokens that can be accepted: the largest logits' tokens for every other child
+        for n in range(1, case.N, 2):
+            p = case.parent[n]
+            lo, hi = case.params["allowed_begin"], case.params["allowed_end"]
+            top = torch.topk(case.logits["target_cond"][b, p, lo:hi].float(), 4).indices + lo
+            sib = [int(case.tokens[b, m]) for m in range(1, case.N) if case.parent[m] == p and m != n]
+            pick = [int(x) for x in top if int(x) not in sib]
+            if pick:
+                case.tokens[b, n] = pick[0]
+    _run(L, case)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("shape", ["block", "rising", "periodic", "few"])
+def test_topk_rows_whose_sample_misleads(L, shape, dtype):
+    """The largest entries in one short block, in order, at the period of the sample, or fewer finite entries than k:
+    whatever the sample says, the truncation is exact (the dense kernel redoes what does not fit the lists)."""
+    V = 40000
+    case = Case(small_config(batch=1, vocab=V, codebook_size=500, top_k=700, k=8, cfg_scale=None, dtype=dtype), seed=52, tokens="random")
+    for v in case.padded.values():
+        if v is None:
+            continue
+        base = v.float()
+        if shape == "block":
+            base[:, :, 20000:20800] += 12.0
+        elif shape == "rising":
+            base += torch.linspace(-8.0, 8.0, V)
+        elif shape == "periodic":
+            base[:, :, ::64] += 9.0
+        else:
+            keep = base[:, :, 1000:1400].clone()
+            base[:] = -float("inf")
+            base[:, :, 1000:1400] = keep
+        v.copy_(base.to(v.dtype))
+    kids = [m for m in range(1, case.N)]
+    for m in kids:                    # tokens that have mass
+        case.tokens[0, m] = 1000 + 3 * m if shape == "few" else 20000 + 7 * m
+    _run(L, case)
+
+
 def test_topk_target_only_and_leaf_only_tree(L):
     # top-k on the target side only: the drafter rows are dense, so the dense kernel runs
     case = Case(small_config(top_k=0), seed=14, top_k_target=60, top_k_draft=0)
