@@ -583,7 +583,7 @@ def dynamic_tree_entry(torch, L, dev, peak):
             "us_median": round(1e3 * med, 1), "us_min": round(1e3 * times[0], 1), "algorithmic_bytes": alg,
             "gbs": round(alg / (med * 1e-3) / 1e9, 1), "frac_measured": round(alg / (med * 1e-3) / 1e9 / peak, 4),
             "mean_nodes": float(n.float().mean()), "mean_node_depth": round(depth_mean, 3),
-            "note": "two passes per row (HBM, then L2); about 10 instructions per logit and pass, latency-bound chain per row"}
+            "note": "one pass per row"}
 
 
 def c1_three_numbers(torch, L, W, dev, peak, use_graph=True):
