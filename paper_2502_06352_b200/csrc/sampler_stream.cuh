@@ -45,6 +45,8 @@ __device__ __forceinline__ float fast_key(float z, float U) {
 __device__ __noinline__ float careful_key(float z, float U) {
   return fmaf(-0.6931471805599453f, lg2_approx(-logf(U) * kLog2e), z);
 }
+// ... and where U is below the smallest normal number, which lg2.approx takes for 0 (supplied uniforms only)
+__device__ __forceinline__ bool wants_care(float U) { return U > 0.999f || U < 1.17549435e-38f; }
 
 template <typename T, bool CFG, bool TAU1>
 __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a) {
@@ -106,9 +108,10 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
   if (tid == 0) *s.cnt = 0;
   __syncthreads();
 
-  // 1 + U of tokens j .. j+VN-1 (j a multiple of VN).  Philox words become floats without an integer
-  // conversion: the 23 mantissa bits under the exponent of 1.0 give F = 1 + i 2^-23, and subtracting
-  // 1 - 2^-24 leaves U = (i + 1/2) 2^-23 exactly.
+  // 1 + U of tokens j .. j+VN-1 (j a multiple of VN), to 2^-24: enough for the test of the later chunks.  Philox words
+  // become floats without an integer conversion: the 23 mantissa bits under the exponent of 1.0 give F = 1 + i 2^-23, and
+  // subtracting 1 - 2^-24 leaves U = (i + 1/2) 2^-23 exactly.  Supplied uniforms lie on no such grid: keys are
+  // made from `uniforms`, which hands them on as they are.
   auto words = [&](int j, float (&F)[VN]) {
     if (gum) {
 #pragma unroll
@@ -124,6 +127,16 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
       }
     }
   };
+  auto uniforms = [&](int j, float (&U)[VN]) {
+    if (gum) {
+#pragma unroll
+      for (int e = 0; e < VN; ++e) U[e] = (j + e < a.V) ? __ldcs(gum + j + e) : 0.5f;
+    } else {
+      words(j, U);
+#pragma unroll
+      for (int e = 0; e < VN; ++e) U[e] -= 0.99999994f;
+    }
+  };
   auto uniform_at = [&](int t) -> float {
     if (gum) return __ldcs(gum + t);
     const Philox4 r = philox4x32_10_keys(static_cast<uint32_t>(t >> 2), row_id, static_cast<uint32_t>(a.step),
@@ -136,7 +149,7 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
     for (int i = raw + tid; i < n; i += ST) {
       const uint2 en = s.list[i];
       const float U = uniform_at(static_cast<int>(en.y)), z = __uint_as_float(en.x);
-      s.list[i].x = __float_as_uint(U > 0.999f ? careful_key(z, U) : fast_key(z, U));
+      s.list[i].x = __float_as_uint(wants_care(U) ? careful_key(z, U) : fast_key(z, U));
     }
     __syncthreads();
     return n <= ST ? cut_ranked(s, R, T) : cut_list(s, R, T);
@@ -188,19 +201,18 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
 #pragma unroll
             for (int e = 0; e < VN; ++e) z[e] = (j + e >= ge.alo && j + e < ge.ahi) ? io.z_at(j + e) : -INFINITY;
           }
-          float F[VN];
-          words(j, F);
-          bool near_one = false;
+          float U[VN];
+          uniforms(j, U);
+          bool care = false;
 #pragma unroll
           for (int e = 0; e < VN; ++e) {
-            const float U = F[e] - (gum ? 1.f : 0.99999994f);
-            first[u][e] = fast_key(z[e], U);
-            near_one |= U > 0.999f;
+            first[u][e] = fast_key(z[e], U[e]);
+            care |= wants_care(U[e]);
           }
-          if (near_one) {                               // rare: one vector in a hundred
+          if (care) {                                   // rare: one vector in a hundred
 #pragma unroll
             for (int e = 0; e < VN; ++e)
-              if (F[e] > 1.998f) first[u][e] = careful_key(z[e], gum ? __ldcs(gum + j + e) : F[e] - 0.99999994f);
+              if (wants_care(U[e])) first[u][e] = careful_key(z[e], U[e]);
           }
           if (want_prob) acc_exp<VN>(z, mx, sx);
         }

@@ -256,3 +256,38 @@ def test_topk_rows_of_every_width(L, kw):
     assert _compare(case, gum.numpy(), gtok, gprob) <= 1
     again, prob, _ = _gpu_sample(L, case, gumbel=gum)
     assert np.array_equal(again, gtok) and np.array_equal(prob, gprob)          # bit for bit
+
+
+@pytest.mark.parametrize("V,cs", [(4096, 0), (16384, 0), (65536, 1)])       # one chunk per CTA; the same on a cluster; sixteen chunks
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_supplied_uniforms_of_any_size_are_used_as_given(L, V, cs, dtype):
+    """Uniforms that no 2^-23 grid holds, down to the smallest float32, on a token that dominates its row, at the row's
+    start and far behind it; a second token's key lies 1e-3 above or below, so that a key that is off by more shows."""
+    us = [2.0 ** -24, 1e-8, 1e-7, 1e-6, 1e-5, 3e-5, 1e-30, 1e-42, 1.0 - 2.0 ** -24]
+    parent = [-1] + [0] * 4
+    kw = dict(vocab=V, codebook_size=512, batch=2 * len(us), dtype=dtype, cfg_scale=None)
+    case = Case(small_config(**kw), parent=parent, seed=61, tokens="random", kernels=1)
+    gum = W.make_gumbel_uniforms(case.B, case.N, V, 17)
+    rows = case.padded["draft_cond"]
+    for i, u in enumerate(us):
+        for j in range(2):
+            b = 2 * i + j
+            a = 5 if j == 0 else V - 99
+            gum[b, 0, a] = u
+            rows[b, 0, a] = 40.0
+            key = float(rows[b, 0, a].float()) - np.log(-np.log(np.float64(gum[b, 0, a].item())))
+            t = (a + 1234) % V                         # a token of the same height whose uniform puts its key beside that one
+            rows[b, 0, t] = rows[b, 0, a]
+            for step in (1e-3, -1e-3):
+                want = np.exp(-np.exp(-(key + step - float(rows[b, 0, t].float()))))
+                if 0.0 < np.float32(want) < 1.0:
+                    gum[b, 0, t] = float(np.float32(want))
+                    break
+    old = L.set_cluster_size(cs)
+    try:
+        gtok, gprob, _ = _gpu_sample(L, case, gumbel=gum)
+    finally:
+        L.set_cluster_size(old)
+    assert _compare(case, gum.numpy(), gtok, gprob) == 0
+    dominant = [5 if b % 2 == 0 else V - 99 for b in range(case.B)]
+    assert all(dominant[b] in gtok[b, 1:] for b in range(case.B))
