@@ -12,7 +12,8 @@
 // one and T) are closer than the keys' errors, by keys recomputed in double precision (ties: lower
 // token id); the result is the exact ranking as long as the s-th exact key clears T by kKeyEps, which
 // is checked (LANTERN_DEV_KEY_TIES otherwise: more than s+4 keys within 2.5e-4 of each other at the
-// top).  The softmax denominator for draft_prob comes from the same pass.
+// top, or within a few units in the last place of logits so large that those are more).  The softmax
+// denominator for draft_prob comes from the same pass.
 //
 // Bound: instruction issue; the generator alone is 10 to 12 of about 20 instructions per element.  3200 rows of
 // 65536 bfloat16 logits: 244 us (two logarithms per element and branches between the vectors: 320); 144 rows of
@@ -24,7 +25,10 @@
 namespace lantern {
 namespace stream {
 
-constexpr float kKeyEps = 2.5e-4f;               // bound on |fast key - exact key| (up to the constant below)
+// bound on |fast key - exact key| (up to the constant below): the logarithms' error, and the key's own rounding, which is
+// what counts for logits in the thousands and above (2^-24 of the key, doubled)
+constexpr float kKeyEps = 2.5e-4f;
+__device__ __forceinline__ float key_eps(float k) { return fmaf(fabsf(k), 1.1920929e-7f, kKeyEps); }
 constexpr float kKeyShift = -0.36651292f;        // ln(ln 2): fast keys are z + G + ln(ln 2)
 
 __host__ __device__ constexpr size_t sampler_stream_smem() {
@@ -346,8 +350,11 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
   bool near = false;
   if (tid < nf && tid < nc) {
     const float k = __uint_as_float(fin[tid].x);
-    if (tid + 1 < nf) near = k - __uint_as_float(fin[tid + 1].x) <= 2.f * kKeyEps;
-    if (tid == nc - 1) near |= k - tmax <= 2.f * kKeyEps;
+    if (tid + 1 < nf) {
+      const float next = __uint_as_float(fin[tid + 1].x);
+      near = k - next <= key_eps(k) + key_eps(next);
+    }
+    if (tid == nc - 1) near |= tmax > -INFINITY && k - tmax <= key_eps(k) + key_eps(tmax);
   }
   const bool exact = __syncthreads_or(near ? 1 : 0) != 0;
   if (exact && tid < nf)
@@ -364,7 +371,7 @@ __global__ void __launch_bounds__(ST, 4) sample_stream_kernel(const SampleArgs a
         const double ki = s.fkey[i];
         rank += (ki > k || (ki == k && static_cast<int>(fin[i].y) < t)) ? 1 : 0;
       }
-      if (rank == nc - 1 && static_cast<double>(tmax) + kKeyEps >= k + kKeyShift) vflag(a.status, LANTERN_DEV_KEY_TIES);
+      if (rank == nc - 1 && static_cast<double>(tmax) + key_eps(tmax) >= k + kKeyShift) vflag(a.status, LANTERN_DEV_KEY_TIES);
     }
     if (rank < nc) {
       a.tokens[out_b + fc + rank] = t;

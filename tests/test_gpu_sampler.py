@@ -291,3 +291,36 @@ def test_supplied_uniforms_of_any_size_are_used_as_given(L, V, cs, dtype):
     assert _compare(case, gum.numpy(), gtok, gprob) == 0
     dominant = [5 if b % 2 == 0 else V - 99 for b in range(case.B)]
     assert all(dominant[b] in gtok[b, 1:] for b in range(case.B))
+
+
+@pytest.mark.parametrize("z", [20000.0, -300000.0])
+def test_large_logits_are_ordered_by_exact_keys(L, z):
+    """Logits so large that a float32 step (2e-3, 3e-2) is far above the keys' own error: two tokens of the same height whose
+    noise lies on either side of a rounding boundary, closer together than that error, where their float32 keys are a
+    whole step apart and say nothing about the order."""
+    V, B = 4096, 64
+    case = Case(small_config(vocab=V, codebook_size=512, batch=B, n_nodes=26, cfg_scale=None), seed=62, tokens="random", kernels=1)
+    rng = np.random.default_rng(12)
+    step = abs(float(np.spacing(np.float32(z))))
+    case.padded["draft_cond"][:] = z - 60.0 * max(1.0, step)
+    gum = W.make_gumbel_uniforms(B, case.N, V, 18)
+    pair = {}
+    for b in range(B):
+        for n in range(case.N):
+            edge = (round((6.4 + 0.1 * rng.random()) / step) + 0.5) * step
+            t = rng.choice(V, 2, replace=False)
+            for i, off in enumerate((-2e-5, 2e-5)):
+                gum[b, n, t[i]] = float(np.float32(np.exp(-np.exp(-(edge + off)))))
+                case.padded["draft_cond"][b, n, t[i]] = z
+            key = -np.log(-np.log(gum[b, n, torch.from_numpy(t)].double().numpy()))
+            if abs(key[0] - key[1]) > 1e-6:
+                pair[b, n] = [int(x) for x in (t if key[0] > key[1] else t[::-1])]
+    g, par, _, _ = case.gpu_inputs(L)
+    tok = L.sample_draft_tree(par, L.Tree(case.parent), g["draft_cond"], None, gumbel_uniforms=gum.cuda()).cpu().numpy()
+    kids = oracle.tree_children(case.parent)
+    seen = 0
+    for (b, n), want in pair.items():
+        if len(kids[n]) >= 2:
+            seen += 1
+            assert [int(tok[b, c]) for c in kids[n][:2]] == want, (b, n)
+    assert seen > 200
