@@ -961,10 +961,29 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
       if (!any) {
         // last positive entry of the range
         if (lastpos >= 0) atomicMax(&sm.misc[3], lastpos);
+        if (tid == 0) { sm.misc[4] = 0x7fffffff; sm.misc[5] = -1; }
         __syncthreads();
+        int found = sm.misc[3];
+        if (det && banned && found < 0) {
+          // Nothing in the range has mass: its sum was what rounding left of a difference.  The first token with mass
+          // behind it, else the last before it, by this CTA over the whole row.
+          for (int vv = tid; vv < ge.nvec; vv += ST) {
+            float tv[VN];
+            vec_terms(ioq, iop, ge, cur, sm.bits, vv, tv);
+#pragma unroll
+            for (int e = 0; e < VN; ++e) {
+              if (tv[e] > 0.f) {
+                if (vv >= oe) atomicMin(&sm.misc[4], ge.j0 + vv * VN + e);
+                else atomicMax(&sm.misc[5], ge.j0 + vv * VN + e);
+              }
+            }
+          }
+          __syncthreads();
+          found = sm.misc[4] != 0x7fffffff ? sm.misc[4] : sm.misc[5];
+        }
         if (tid == 0) {
-          a.node_token[out_b + n] = sm.misc[3];
-          if (sm.misc[3] < 0) vflag(a.status, LANTERN_DEV_EMPTY_ROW);
+          a.node_token[out_b + n] = found;
+          if (found < 0) vflag(a.status, LANTERN_DEV_EMPTY_ROW);
         }
       }
     } else if (owner < 0 && writer) {

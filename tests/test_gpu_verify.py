@@ -476,6 +476,31 @@ def _run_det(L, case):
     check_walk(res, case.tokens, tree.max_depth, orc, stats["dirty_sequences"], case.seqs, stats["patched"])
 
 
+@pytest.mark.parametrize("cs", [1, 2, 4, 16])
+@pytest.mark.parametrize("where", ["first", "last"])
+def test_deterministic_drafts_that_empty_a_stretch_of_the_row(L, cs, where):
+    """The only tokens with mass in one stretch of the row are all rejected, and the uniform points into that stretch
+    (u = 0 at the row's start, u just below 1 at its end): the draw is the nearest token that still has mass."""
+    V, B = 8192, 48
+    parent = [-1] + [0] * 5
+    case = Case(small_config(vocab=V, codebook_size=512, batch=B, k=0, cfg_scale=None), parent=parent, seed=48, det_draft=True, tokens="random")
+    g = torch.Generator().manual_seed(9)
+    at = V - 40 if where == "last" else 40                  # six tokens: five are drafted, one has no mass
+    rest = torch.arange(3000, 5000)
+    rows = case.padded["target_cond"]
+    rows[:] = -float("inf")
+    rows[:, :, rest] = torch.randn((B, case.N, len(rest)), generator=g)
+    rows[:, :, at:at + 5] = torch.randn((B, case.N, 5), generator=g) + 4.0       # about a fifth of the mass
+    case.tokens[:, 1:] = torch.stack([torch.randperm(5, generator=g) for _ in range(B)]).numpy() + at
+    case.u_accept = torch.full_like(case.u_accept, 1.0 - 2.0 ** -24)
+    case.u_resample = torch.full_like(case.u_resample, 1.0 - 2.0 ** -24 if where == "last" else 0.0)
+    old = L.set_cluster_size(cs)
+    try:
+        _run_det(L, case)
+    finally:
+        L.set_cluster_size(old)
+
+
 def test_path_walk_with_a_rule_variant_runs_on_the_streaming_kernel(L):
     case = Case(small_config(k=24, lam=1.8, batch=4, n_nodes=60), seed=45, skip=True)
     g, par, nbr, tok = case.gpu_inputs(L)
