@@ -62,12 +62,12 @@ constexpr int kT5MaxK = 320;
 constexpr int kT5Items = 148;       // CTAs per chunk (one per SM)
 constexpr int kT5MaxSplit = 8;      // shares of the candidates
 constexpr int kT5MaxGroups = 1024;  // group minima per query
-constexpr float kT5Huge = 1e37f;    // rows with a squared norm from here on never enter the contraction's bounds
+constexpr float kT5Huge = 1e37f;    // rows with a squared norm from here on (or NaN) never enter the bounds or the lists
 
 struct KnnT5Args {
   // operand tiles of 128 rows in the layout the tensor core reads, [dpad/8 chunks][16 row groups][8 rows][16 bytes]:
   const unsigned char *qm, *cm;     // query side, and candidate side (the sampled rows in the sample pass)
-  const float* cn;                  // squared norms of the candidate side's rows, +inf for rows that are none
+  const float* cn;                  // squared norms of the candidate side's rows, +inf for rows that are none and from kT5Huge on
   const float* nrm;                 // [L] squared norms, nrm[L] = the largest below kT5Huge
   float* minima;                    // [tiles][kT5Q][groups] (sample pass)
   const float* bound;               // [tiles][kT5Q] knn_bound_kernel's result
@@ -504,7 +504,8 @@ __global__ void __launch_bounds__(256) knn_prep_kernel(const KnnPrepArgs a) {
   odd = __any_sync(0xffffffffu, odd);
   if (lane == 0) {
     if (odd && !sample && in) a.nrm[a.L + 1] = 1.f;
-    (sample ? a.sn : a.cn)[tr] = in ? s : INFINITY;
+    // (a row whose norm the error bound does not cover is no candidate: a query that needs it finds too few others)
+    (sample ? a.sn : a.cn)[tr] = in && s < kT5Huge ? s : INFINITY;
     if (!sample && in) {
       a.nrm[row] = s;
       unsigned int* top = reinterpret_cast<unsigned int*>(a.nrm + a.L);      // s >= 0: bit order = value order

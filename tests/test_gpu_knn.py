@@ -242,3 +242,33 @@ def test_float32_codebook_without_a_workspace_takes_the_brute_force_kernel(L):
     # a bfloat16 shape that has always needed its workspace is still refused
     b = W.make_codebook(600, 32, "bf16", seed=2).cuda()
     assert lib.lantern_build_neighbors(p(b), 1, 600, 32, k, p(idx), p(dist), None, 0, None) == 3
+
+
+@pytest.mark.parametrize("dt", ["f32", "bf16"])
+def test_rows_of_huge_norm_among_the_neighbours(L, dt):
+    """Squared norms that float32 still holds (1e37 to 3.4e38) beside ordinary rows, and k reaching past those: what the
+    contraction's error bound does not cover is ranked without it."""
+    n, d, k = 300, 16, 150
+    g = torch.Generator().manual_seed(31)
+    dtype = torch.float32 if dt == "f32" else torch.bfloat16
+    cb = torch.randn((n, d), generator=g)
+    # two hundred rows of nearly the same norm: the same magnitudes, five decades of them, in another order in every row, the
+    # small ones a few per cent apart
+    base = 4e18 * 10.0 ** (-5.0 * torch.arange(d) / (d - 1))
+    for i in range(100, n):
+        row = base * torch.where(torch.arange(d) > 9, 1.0 + 0.1 * torch.rand(d, generator=g), 1.0)
+        cb[i] = (row * torch.sign(torch.rand(d, generator=g) - 0.5))[torch.randperm(d, generator=g)]
+    cb = cb[torch.randperm(n, generator=g)].to(dtype)
+    norms = (cb.double() ** 2).sum(1)
+    assert ((norms > 1.1e37) & (norms < 3.4e38)).sum() == 200
+    idx, dist = L.build_neighbors(cb.cuda(), k, return_dist=True)
+    idx, dist = idx.cpu().numpy(), dist.cpu().numpy()
+    x = cb.to(torch.float64).numpy()
+    for i in range(n):
+        D = ((x - x[i]) ** 2).sum(axis=1)
+        D[i] = np.inf
+        want = np.lexsort((np.arange(n), D))[:k]
+        # (the double sums differ in their last bits between the two sides: only distances closer than that may swap)
+        assert np.all((idx[i] == want) | (np.abs(D[idx[i]] - D[want]) <= 1e-13 * D[want])), i
+        with np.errstate(over="ignore"):
+            assert np.allclose(dist[i], D[idx[i]].astype(np.float32), rtol=1e-6, atol=0)
