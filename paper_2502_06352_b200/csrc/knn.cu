@@ -24,9 +24,11 @@ struct KnnArgs {
   const void* cb;
   int L, d, k, QT, CAP, q_double;
   int f32acc;        // filter distances accumulated in float32 with an error margin (small d)
-  float margin;      // 1 + 3 (d + 2) 2^-24: the filter keeps everything within this factor of tau
+  float margin;      // 1 + 3 (d + 2) 2^-24: the filter keeps everything within this factor of tau ...
+  float slack;       // ... and this much more: the rounding of sums below the normal range
   int32_t* nbr_idx;
   float* nbr_dist;
+  const int *queries, *n_queries;   // LISTED: the query rows, in any order, and their number
 };
 
 template <typename T> __device__ __forceinline__ float widen(T x);
@@ -202,9 +204,9 @@ __device__ __forceinline__ void rank_query(const T* __restrict__ cb, int L, int 
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kKnnThreads) knn_kernel(const KnnArgs a) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+// Queries [q0, q0 + QT) of `total`: the rows themselves, or with LISTED the entries of a list.
+template <typename T, bool LISTED>
+__device__ __forceinline__ void knn_tile(const KnnArgs& a, const int q0, const int total, unsigned char* smem_raw) {
   const int QT = a.QT, CAP = a.CAP, d = a.d, L = a.L, k = a.k;
   const T* cb = static_cast<const T*>(a.cb);
   // layout: buf[QT][CAP] u64 | sortd[CAP] f64 | sorti[CAP] i32 | cand[256][kDC+1] f32 | tau[QT] f32 |
@@ -226,19 +228,19 @@ __global__ void __launch_bounds__(kKnnThreads) knn_kernel(const KnnArgs a) {
   float* qf = reinterpret_cast<float*>(qraw);
 
   const int tid = threadIdx.x;
-  const int q0 = blockIdx.x * QT;
-  const int nq = min(QT, L - q0);
+  const int nq = min(QT, total - q0);
+  auto row_of = [&](int q) { return LISTED ? a.queries[q0 + q] : q0 + q; };
 
   const int dpad = (d + 7) & ~7;
   if (a.f32acc) {
     for (int i = tid; i < QT * dpad; i += kKnnThreads) {
       int q = i / dpad, t = i - q * dpad;
-      qf[i] = (q < nq && t < d) ? widen<T>(cb[static_cast<long long>(q0 + q) * d + t]) : 0.f;
+      qf[i] = (q < nq && t < d) ? widen<T>(cb[static_cast<long long>(row_of(q)) * d + t]) : 0.f;
     }
   } else {
     for (int i = tid; i < QT * d; i += kKnnThreads) {
       int q = i / d, t = i - q * d;
-      float v = (q < nq) ? widen<T>(cb[static_cast<long long>(q0 + q) * d + t]) : 0.f;
+      float v = (q < nq) ? widen<T>(cb[static_cast<long long>(row_of(q)) * d + t]) : 0.f;
       if (a.q_double) qd[i] = static_cast<double>(v); else qf[i] = v;
     }
   }
@@ -246,6 +248,9 @@ __global__ void __launch_bounds__(kKnnThreads) knn_kernel(const KnnArgs a) {
   __syncthreads();
 
   constexpr int MAXQT = 8;
+  int own[MAXQT];                                     // (a query is no candidate of its own)
+#pragma unroll
+  for (int q = 0; q < MAXQT; ++q) own[q] = q < nq ? row_of(q) : -1;
   // d <= 8 (one chunk of dimensions): the candidate row of the next tile is fetched while this
   // tile is being processed
   float cnext[8];
@@ -323,7 +328,7 @@ __global__ void __launch_bounds__(kKnnThreads) knn_kernel(const KnnArgs a) {
       const int j = base + tid;
 #pragma unroll
       for (int q = 0; q < MAXQT; ++q) {
-        if (q < nq && j != q0 + q) {
+        if (q < nq && j != own[q]) {
           float f = static_cast<float>(acc[q]);
           if (f <= tau[q]) {
             int pos = atomicAdd(&cnt[q], 1);
@@ -341,9 +346,9 @@ __global__ void __launch_bounds__(kKnnThreads) knn_kernel(const KnnArgs a) {
       unsigned long long* bq = buf + static_cast<size_t>(q) * CAP;
       // keep everything up to the k-th smallest filter distance (times the margin in float32 mode)
       uint32_t limit;
-      const float margin = a.f32acc ? a.margin : 1.0f;
+      const float margin = a.f32acc ? a.margin : 1.0f, slack = a.f32acc ? a.slack : 0.0f;
       const int m = radix_cut(bq, min(n, CAP), k, reinterpret_cast<unsigned long long*>(sortd), hist, sel,
-                              [&](uint32_t kth) { return __float_as_uint(__fmul_ru(__uint_as_float(kth), margin)); }, &limit);
+                              [&](uint32_t kth) { return __float_as_uint(__fadd_ru(__fmul_ru(__uint_as_float(kth), margin), slack)); }, &limit);
       if (tid == 0) {
         tau[q] = __uint_as_float(limit);      // (non-negative floats order as their bits)
         cnt[q] = m;
@@ -355,10 +360,29 @@ __global__ void __launch_bounds__(kKnnThreads) knn_kernel(const KnnArgs a) {
 
   // final ranking per query
   for (int q = 0; q < nq; ++q) {
-    const int qi = q0 + q;
+    const int qi = row_of(q);
     rank_query<T>(cb, L, d, k, qi, buf + static_cast<size_t>(q) * CAP, cnt[q], ovf[q] != 0, CAP, sortd, sorti, redd, redi,
                   a.nbr_idx + static_cast<long long>(qi) * k,
                   a.nbr_dist ? a.nbr_dist + static_cast<long long>(qi) * k : nullptr);
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kKnnThreads) knn_kernel(const KnnArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  knn_tile<T, false>(a, blockIdx.x * a.QT, a.L, smem_raw);
+}
+
+// The queries that the tcgen05 kernels gave up (usually none: the list is made on the device, so this is always launched,
+// on about the CTAs that are resident at once).  Rows that crowd within the contraction's absolute error
+// bound differ by far more than the relative margin here.
+template <typename T>
+__global__ void __launch_bounds__(kKnnThreads) knn_rest_kernel(const KnnArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int total = *a.n_queries;
+  for (int q0 = blockIdx.x * a.QT; q0 < total; q0 += gridDim.x * a.QT) {
+    knn_tile<T, true>(a, q0, total, smem_raw);
+    __syncthreads();                                  // the next queries overwrite the shared memory
   }
 }
 
@@ -382,7 +406,7 @@ struct T5Plan {
   bool ok, sampled;                 // sampled: the sample is a proper part of the codebook, with tiles of its own
   int dp, tiles, nst, gshift, groups;
   int first_tiles;                  // query tiles of the first (largest) chunk
-  size_t off_cn, off_sn, off_counts, off_bound, off_qm, off_cm, off_sm, off_minima, off_lists, bytes;
+  size_t off_cn, off_sn, off_rest, off_counts, off_bound, off_qm, off_cm, off_sm, off_minima, off_lists, bytes;
 };
 size_t round256(size_t x) { return (x + 255) / 256 * 256; }
 int t5_split(int tiles, int L) {    // CTAs per query tile of a chunk
@@ -425,7 +449,8 @@ T5Plan t5_plan(lantern_dtype dt, int L, int d, int k) {
   const size_t tile = static_cast<size_t>(kT5Q) * p.dp * 2, side = p.tiles * tile;
   p.off_cn = round256((static_cast<size_t>(L) + 64) * sizeof(float));
   p.off_sn = p.off_cn + static_cast<size_t>(p.tiles) * kT5C * sizeof(float);
-  p.off_counts = p.off_sn + static_cast<size_t>(p.sampled ? p.nst : 0) * kT5C * sizeof(float);
+  p.off_rest = p.off_sn + static_cast<size_t>(p.sampled ? p.nst : 0) * kT5C * sizeof(float);
+  p.off_counts = p.off_rest + round256(static_cast<size_t>(L) * sizeof(int));
   p.off_bound = p.off_counts + segs * sizeof(int);
   p.off_qm = p.off_bound + static_cast<size_t>(kT5Items) * kT5Q * sizeof(float);
   p.off_cm = p.off_qm + (dt == LANTERN_F32 ? side : 0);
@@ -437,11 +462,31 @@ T5Plan t5_plan(lantern_dtype dt, int L, int d, int k) {
   return p;
 }
 
+// Arguments of the brute-force kernels; returns their shared memory.
+size_t brute_shape(KnnArgs& a, const void* codebook, int L, int d, int k, int32_t* nbr_idx, float* nbr_dist) {
+  a.cb = codebook; a.L = L; a.d = d; a.k = k; a.nbr_idx = nbr_idx; a.nbr_dist = nbr_dist;
+  int cap = 512;
+  while (cap < k + 2 * kKnnThreads) cap *= 2;
+  a.CAP = cap;
+  a.QT = cap <= 1024 ? 8 : 4;
+  auto smem_for = [&](int qt, int qdouble) {
+    return static_cast<size_t>(qt) * cap * 8 + static_cast<size_t>(cap) * 12 + 8 * 12 +
+           static_cast<size_t>(kKnnThreads) * (kDC + 1) * 4 + static_cast<size_t>(qt) * 12 + 16 + 260 * 4 +
+           static_cast<size_t>(qt) * ((d + 7) & ~7) * (qdouble ? 8 : 4);
+  };
+  a.f32acc = d <= 64 ? 1 : 0;
+  a.margin = 1.0f + 3.0f * static_cast<float>(d + 2) * 5.9604644775390625e-8f;
+  a.slack = static_cast<float>(d + 2) * 2.8025969e-45f;          // two roundings of 2^-150 per term, doubled
+  a.q_double = (!a.f32acc && smem_for(a.QT, 1) <= 160 * 1024) ? 1 : 0;
+  while (a.QT > 1 && smem_for(a.QT, a.q_double) > 220 * 1024) a.QT /= 2;
+  return smem_for(a.QT, a.q_double);
+}
+
 template <typename T>
 lantern_status build_t5(const T5Plan& p, const T* cb, int L, int d, int k, int32_t* nbr_idx, float* nbr_dist,
                         unsigned char* ws, cudaStream_t st) {
   float* nrm = reinterpret_cast<float*>(ws);
-  if (cudaMemsetAsync(nrm + L, 0, 2 * sizeof(float), st) != cudaSuccess) return LANTERN_ERR_CUDA;
+  if (cudaMemsetAsync(nrm + L, 0, 3 * sizeof(float), st) != cudaSuccess) return LANTERN_ERR_CUDA;
   KnnPrepArgs g;
   g.cb = cb; g.L = L; g.d = d; g.dp = p.dp;
   g.rows = p.tiles * kT5C;
@@ -469,13 +514,19 @@ lantern_status build_t5(const T5Plan& p, const T* cb, int L, int d, int k, int32
   KnnRankArgs r;
   r.cb = cb; r.nrm = nrm; r.lists = a.lists; r.counts = a.counts;
   r.L = L; r.d = d; r.k = k; r.eps1 = a.eps1; r.eps0 = a.eps0; r.nbr_idx = nbr_idx; r.nbr_dist = nbr_dist;
+  r.rest = reinterpret_cast<int*>(ws + p.off_rest);
+  r.n_rest = reinterpret_cast<int*>(nrm + L + 2);
   r.lanes = 0;
   if (d % 8 == 0 && reinterpret_cast<uintptr_t>(cb) % 16 == 0) {
     r.lanes = 1;
     while (r.lanes < 8 && r.lanes * 2 <= d / 8) r.lanes *= 2;
   }
+  KnnArgs b = {};
+  const size_t smb = brute_shape(b, cb, L, d, k, nbr_idx, nbr_dist);
+  b.queries = r.rest; b.n_queries = r.n_rest;
   const size_t sm5 = knn_t5_smem(p.dp), smr = knn_rank_smem(d);
-  if (cudaFuncSetAttribute(knn_t5_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm5)) != cudaSuccess ||
+  if (cudaFuncSetAttribute(knn_rest_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smb)) != cudaSuccess ||
+      cudaFuncSetAttribute(knn_t5_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm5)) != cudaSuccess ||
       cudaFuncSetAttribute(knn_t5_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm5)) != cudaSuccess)
     return LANTERN_ERR_CUDA;
   for (a.tile0 = 0; a.tile0 < p.tiles; a.tile0 += kT5Items) {
@@ -493,6 +544,8 @@ lantern_status build_t5(const T5Plan& p, const T* cb, int L, int d, int k, int32
     const int queries = L - r.q0 < n * kT5Q ? L - r.q0 : n * kT5Q;
     knn_rank_kernel<T><<<queries, kRankThreads, smr, st>>>(r);
   }
+  const int groups = (L + b.QT - 1) / b.QT, resident = smb <= 113 * 1024 ? 2 * kT5Items : kT5Items;
+  knn_rest_kernel<T><<<groups < resident ? groups : resident, kKnnThreads, smb, st>>>(b);
   return cudaGetLastError() == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
 }
 
@@ -530,22 +583,8 @@ extern "C" lantern_status lantern_build_neighbors(const void* codebook, lantern_
                                : build_t5(p, static_cast<const __nv_bfloat16*>(codebook), L, d, k, nbr_idx, nbr_dist, ws, st);
     }
   }
-  KnnArgs a;
-  a.cb = codebook; a.L = L; a.d = d; a.k = k; a.nbr_idx = nbr_idx; a.nbr_dist = nbr_dist;
-  int cap = 512;
-  while (cap < k + 2 * kKnnThreads) cap *= 2;
-  a.CAP = cap;
-  a.QT = cap <= 1024 ? 8 : 4;
-  auto smem_for = [&](int qt, int qdouble) {
-    return static_cast<size_t>(qt) * cap * 8 + static_cast<size_t>(cap) * 12 + 8 * 12 +
-           static_cast<size_t>(kKnnThreads) * (kDC + 1) * 4 + static_cast<size_t>(qt) * 12 + 16 + 260 * 4 +
-           static_cast<size_t>(qt) * ((d + 7) & ~7) * (qdouble ? 8 : 4);
-  };
-  a.f32acc = d <= 64 ? 1 : 0;
-  a.margin = 1.0f + 3.0f * static_cast<float>(d + 2) * 5.9604644775390625e-8f;
-  a.q_double = (!a.f32acc && smem_for(a.QT, 1) <= 160 * 1024) ? 1 : 0;
-  while (a.QT > 1 && smem_for(a.QT, a.q_double) > 220 * 1024) a.QT /= 2;
-  size_t smem = smem_for(a.QT, a.q_double);
+  KnnArgs a = {};
+  const size_t smem = brute_shape(a, codebook, L, d, k, nbr_idx, nbr_dist);
   if (smem > 227 * 1024) return LANTERN_ERR_UNSUPPORTED;
   const int grid = (L + a.QT - 1) / a.QT;
   cudaError_t e;

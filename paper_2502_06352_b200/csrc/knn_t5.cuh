@@ -21,7 +21,8 @@
 //                          sample is representative.  A list that would overflow all the same is cut
 //                          back by its warp.
 //   knn_rank_kernel        one CTA per query: cuts the lists down to the k-th smallest g + 2 eps and
-//                          ranks the survivors by (exact distance in double precision, index).
+//                          ranks the survivors by (exact distance in double precision, index).  Queries whose
+//                          survivors are too many (rows closer together than eps) or too few go to knn_rest_kernel.
 // Measured on 65536 x 256, k = 200 (5.5 ms; one kernel that streamed from an open threshold, cut lists back
 // and ranked behind the contraction took 19.7): per chunk of 18944 queries 0.22 ms sample pass, 0.06 ms bounds,
 // 0.75 ms contraction, 0.64 ms ranking; the tensor rate alone would be 0.39 ms per chunk.  The contraction's
@@ -549,12 +550,13 @@ struct KnnRankArgs {
   int q0;                           // first query of the chunk
   int lanes;                        // lanes that share one candidate's distance (power of two); 0: rows read element by element
   float eps1, eps0;
+  int *rest, *n_rest;               // queries left to the brute-force kernel, and their number
   int32_t* nbr_idx;
   float* nbr_dist;
 };
 constexpr int kRankThreads = 128;
 __host__ __device__ constexpr size_t knn_rank_smem(int d) {
-  return kT5Sort * (8 + 8 + 4) + 256 * 4 + static_cast<size_t>((d + 7) / 8 * 8) * 8 + 16 * 8 + 64;
+  return kT5Sort * (8 + 8 + 4) + 256 * 4 + static_cast<size_t>((d + 7) / 8 * 8) * 8 + 16;
 }
 
 // Eight elements to double.  For normal bfloat16 numbers the double's high word is the sign, the exponent rebiased by
@@ -619,10 +621,9 @@ __global__ void __launch_bounds__(kRankThreads) knn_rank_kernel(const KnnRankArg
   unsigned long long* st = reinterpret_cast<unsigned long long*>(rank_smem);     // [kT5Sort] survivors
   unsigned long long* sortd = st + kT5Sort;                                      // [kT5Sort] bits of doubles >= 0
   double* qd = reinterpret_cast<double*>(sortd + kT5Sort);                       // [d] the query row
-  double* redd = qd + (a.d + 7) / 8 * 8;                                         // [4]
-  int* sorti = reinterpret_cast<int*>(redd + 16);                                // [kT5Sort]
+  int* sorti = reinterpret_cast<int*>(qd + (a.d + 7) / 8 * 8);                   // [kT5Sort]
   uint32_t* hist = reinterpret_cast<uint32_t*>(sorti + kT5Sort);                 // [256]
-  int* misc = reinterpret_cast<int*>(hist + 256);                                // [0] survivors, [1..4] minima, [5..8] maxima, [9..12] counts, [12..15] redi
+  int* misc = reinterpret_cast<int*>(hist + 256);                                // [0] survivors
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const T* cb = static_cast<const T*>(a.cb);
   const int ql = blockIdx.x, qi = a.q0 + ql, k = a.k, d = a.d;
@@ -712,8 +713,8 @@ __global__ void __launch_bounds__(kRankThreads) knn_rank_kernel(const KnnRankArg
   } else {
     __syncthreads();
   }
-  if (!whole) {                                      // too few or too many rows under the bound: duplicated rows, huge norms
-    argmin_rounds<T, kRankThreads>(cb, a.L, d, k, qi, redd, misc + 12, out_i, out_d);
+  if (!whole) {                                      // too few or too many rows under the bound: crowded rows, huge norms
+    if (tid == 0) a.rest[atomicAdd(a.n_rest, 1)] = qi;
     return;
   }
   int p2 = 32;

@@ -272,3 +272,38 @@ def test_rows_of_huge_norm_among_the_neighbours(L, dt):
         assert np.all((idx[i] == want) | (np.abs(D[idx[i]] - D[want]) <= 1e-13 * D[want])), i
         with np.errstate(over="ignore"):
             assert np.allclose(dist[i], D[idx[i]].astype(np.float32), rtol=1e-6, atol=0)
+
+
+def _crowded(kind, n, d, dt):
+    g = torch.Generator().manual_seed(41)
+    cb = torch.randn((n, d), generator=g)
+    if kind == "unused":                 # two thirds of the codes still near their initial value
+        cb[: 2 * n // 3] = cb[: 2 * n // 3] * 1e-3 + 0.25
+    elif kind == "offset":               # a common offset: every distance is far below the norms
+        cb += 2000.0
+    else:                                # one row so large that the others' norms vanish beside it
+        cb[n // 2] *= 1e6
+    cb = cb[torch.randperm(n, generator=g)]
+    return cb.to(torch.float32 if dt == "f32" else torch.bfloat16)
+
+
+@pytest.mark.parametrize("kind", ["unused", "offset", "outlier"])
+@pytest.mark.parametrize("n,d,k,dt", [(2500, 8, 100, "f32"), (1300, 64, 50, "f32"), (2000, 80, 33, "f32"), (1400, 100, 320, "bf16"),
+                                      (2200, 32, 64, "bf16"), (64, 8, 10, "f32")])
+def test_codebooks_whose_rows_crowd_within_the_error_bound(L, kind, n, d, k, dt):
+    """Rows that the contraction cannot tell apart (more of them than a query's survivors may be) are ranked by a pass over
+    all rows with a margin relative to the distance."""
+    cb = _crowded(kind, n, d, dt)
+    idx, dist = L.build_neighbors(cb.cuda(), k, return_dist=True)
+    idx, dist = idx.cpu().numpy(), dist.cpu().numpy()
+    x = cb.to(torch.float64).numpy()
+    rows = range(0, n, max(1, n // 60))
+    for i in rows:
+        D = ((x - x[i]) ** 2).sum(axis=1)
+        D[i] = np.inf
+        want = np.lexsort((np.arange(n), D))[:k]
+        assert np.all((idx[i] == want) | (np.abs(D[idx[i]] - D[want]) <= 1e-13 * D[want])), i
+        assert np.allclose(dist[i], D[idx[i]].astype(np.float32), rtol=1e-6, atol=0)
+    assert idx.min() >= 0 and idx.max() < n and not np.any(idx == np.arange(n)[:, None])
+    s = np.sort(idx, axis=1)
+    assert np.all(s[:, 1:] != s[:, :-1])
