@@ -84,7 +84,9 @@ lantern_status lantern_forest_create(const int32_t* parent /* host */, const int
  * step, and allocating and freeing device memory stops the whole GPU each time): `block`, at least
  * lantern_forest_block() bytes, 16-byte aligned, is filled on `stream` before the call returns (not
  * inside a stream capture: LANTERN_ERR_CUDA).  It must stay valid for as long as work that uses the
- * handle is pending, on whatever stream; lantern_tree_destroy does not free it and does not wait. */
+ * handle is pending, on whatever stream; lantern_tree_destroy does not free it and does not wait.
+ * What is wrong with the trees is reported before the block is looked at; lantern_forest_block() is 0 for
+ * sizes that are refused.                                                                         */
 size_t lantern_forest_block(int32_t batch, int32_t max_nodes);
 lantern_status lantern_forest_create_in(const int32_t* parent /* host */, const int32_t* n_nodes /* host */,
                                         int32_t batch, int32_t max_nodes, void* block, size_t block_bytes,

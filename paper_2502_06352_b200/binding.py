@@ -215,10 +215,14 @@ class Forest(Tree):
         arr = self._flat if isinstance(self._flat, ctypes.Array) else (ctypes.c_int32 * len(self._flat)).from_buffer(self._flat)
         cnt = (ctypes.c_int32 * B)(*n_nodes)
         h = ctypes.c_void_p()
-        device = torch.cuda.current_device()
         need = lib.lantern_forest_block(B, self.n_nodes)
-        self.block = torch.empty(max(need, 16), dtype=torch.uint8, device="cuda:%d" % device)
-        self.stream = _raw_stream(device)
+        try:
+            device = torch.cuda.current_device()
+            self.block = torch.empty(max(need, 16), dtype=torch.uint8, device="cuda:%d" % device)
+            self.stream = _raw_stream(device)
+        except (RuntimeError, AssertionError) as e:     # no GPU, or no room on it: what is wrong with the trees comes first
+            status = lib.lantern_forest_create_in(arr, cnt, B, self.n_nodes, None, 0, None, ctypes.byref(h))
+            raise LanternError(4 if status == 3 else status, "lantern_forest_create_in") from e
         _check(lib.lantern_forest_create_in(arr, cnt, B, self.n_nodes, self.block.data_ptr(), self.block.numel(), self.stream,
                                             ctypes.byref(h)), "lantern_forest_create_in")
         self.handle = h

@@ -73,11 +73,14 @@ extern "C" lantern_status lantern_tree_create(const int32_t* parent, int32_t n_n
 // A forest: one tree per sequence, all padded to max_nodes (Sec. 2.1, dynamic tree drafting: the
 // shape of the draft tree depends on the sequence).  The device arrays are [batch][max_nodes];
 // padding nodes have no children and an order entry of -1.
-// `block`: device memory of the caller for those arrays, filled on `stream`; NULL: allocated here.
+// `own`: the arrays are allocated here; otherwise they go to `block`, device memory of the caller, filled on `stream`.
+static bool forest_fits(int32_t batch, int32_t max_nodes) {
+  return max_nodes <= LANTERN_MAX_NODES && static_cast<int64_t>(batch) * max_nodes <= (1 << 24);
+}
 static lantern_status make_forest(const int32_t* parent, const int32_t* n_nodes, int32_t batch, int32_t max_nodes,
-                                  void* block, cudaStream_t stream, lantern_tree** out) {
+                                  bool own, void* block, size_t block_bytes, cudaStream_t stream, lantern_tree** out) {
   if (!parent || !n_nodes || !out || batch < 1 || max_nodes < 1) return LANTERN_ERR_INVALID_ARG;
-  if (max_nodes > LANTERN_MAX_NODES || static_cast<int64_t>(batch) * max_nodes > (1 << 24)) return LANTERN_ERR_UNSUPPORTED;
+  if (!forest_fits(batch, max_nodes)) return LANTERN_ERR_UNSUPPORTED;
   const size_t BN = static_cast<size_t>(batch) * max_nodes;
   int32_t* host = static_cast<int32_t*>(malloc(sizeof(int32_t) * 4 * BN));
   if (!host) return LANTERN_ERR_CUDA;
@@ -111,11 +114,23 @@ static lantern_status make_forest(const int32_t* parent, const int32_t* n_nodes,
     if (internal > max_internal) max_internal = internal;
   }
   if (max_children > LANTERN_MAX_CHILDREN) { free(host); return LANTERN_ERR_UNSUPPORTED; }
+  if (!own) {
+    if (!block || reinterpret_cast<uintptr_t>(block) % 16 || block_bytes < sizeof(int32_t) * 3 * BN) {
+      free(host);
+      return LANTERN_ERR_WORKSPACE;
+    }
+    // a copy from this call's own host arrays must not become part of a graph
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      free(host);
+      return LANTERN_ERR_CUDA;
+    }
+  }
   TreeDev* t = static_cast<TreeDev*>(calloc(1, sizeof(TreeDev)));
   if (!t) { free(host); return LANTERN_ERR_CUDA; }
-  void* dev = block;
+  void* dev = own ? nullptr : block;
   cudaError_t e = cudaSuccess;
-  if (block) {
+  if (!own) {
     // the arrays are in place when this returns, whatever stream uses the handle
     e = cudaMemcpyAsync(dev, host, sizeof(int32_t) * 3 * BN, cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -124,7 +139,7 @@ static lantern_status make_forest(const int32_t* parent, const int32_t* n_nodes,
     if (e == cudaSuccess) e = cudaMemcpy(dev, host, sizeof(int32_t) * 3 * BN, cudaMemcpyHostToDevice);
   }
   if (e != cudaSuccess) {
-    if (!block && dev) cudaFree(dev);
+    if (own && dev) cudaFree(dev);
     free(host);
     free(t);
     return LANTERN_ERR_CUDA;
@@ -134,7 +149,7 @@ static lantern_status make_forest(const int32_t* parent, const int32_t* n_nodes,
   t->max_children = max_children;
   t->n_internal = max_internal;
   t->per_seq = batch;
-  t->d_block = block ? nullptr : dev;
+  t->d_block = own ? dev : nullptr;
   t->d_first_child = static_cast<int32_t*>(dev);
   t->d_n_child = t->d_first_child + BN;
   t->d_order = t->d_first_child + 2 * BN;
@@ -146,25 +161,18 @@ static lantern_status make_forest(const int32_t* parent, const int32_t* n_nodes,
 
 extern "C" lantern_status lantern_forest_create(const int32_t* parent, const int32_t* n_nodes, int32_t batch,
                                                 int32_t max_nodes, lantern_tree** out) {
-  return make_forest(parent, n_nodes, batch, max_nodes, nullptr, nullptr, out);
+  return make_forest(parent, n_nodes, batch, max_nodes, true, nullptr, 0, nullptr, out);
 }
 
 extern "C" size_t lantern_forest_block(int32_t batch, int32_t max_nodes) {
-  if (batch < 1 || max_nodes < 1) return 0;
+  if (batch < 1 || max_nodes < 1 || !forest_fits(batch, max_nodes)) return 0;
   return sizeof(int32_t) * 3 * static_cast<size_t>(batch) * max_nodes;
 }
 
 extern "C" lantern_status lantern_forest_create_in(const int32_t* parent, const int32_t* n_nodes, int32_t batch,
                                                    int32_t max_nodes, void* block, size_t block_bytes, void* stream,
                                                    lantern_tree** out) {
-  if (!block || reinterpret_cast<uintptr_t>(block) % 16) return LANTERN_ERR_WORKSPACE;
-  if (batch < 1 || max_nodes < 1) return LANTERN_ERR_INVALID_ARG;
-  if (block_bytes < lantern_forest_block(batch, max_nodes)) return LANTERN_ERR_WORKSPACE;
-  // a copy from this call's own host arrays must not become part of a graph
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
-    return LANTERN_ERR_CUDA;
-  return make_forest(parent, n_nodes, batch, max_nodes, block, static_cast<cudaStream_t>(stream), out);
+  return make_forest(parent, n_nodes, batch, max_nodes, false, block, block_bytes, static_cast<cudaStream_t>(stream), out);
 }
 
 extern "C" lantern_status lantern_tree_destroy(lantern_tree* tree) {

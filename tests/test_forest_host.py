@@ -44,3 +44,22 @@ def test_flat_parents_of_odd_counts():
     assert list(binding._flat_parents([[-1, 0, 0, 0], [-1, 0, 1, 1]], [3, 3], 3)) == [-1, 0, 0, -1, 0, 1]
     big = [[-1, 2 ** 31, 0], [-1, 0, 1]]             # wraps like a C integer, as ctypes does
     assert len(list(binding._flat_parents(big, [3, 3], 3))) == 6
+
+
+def test_a_forest_of_refused_arguments_says_so_before_any_device_memory_is_asked_for():
+    """Sizes the library refuses and trees that are none: LanternError with the library's status, on a host without a
+    GPU too, and no request for an absurd amount of device memory."""
+    import torch
+    from paper_2502_06352_b200 import Forest, LanternError
+    assert binding.lib.lantern_forest_block(2, 60) == 3 * 2 * 60 * 4
+    assert binding.lib.lantern_forest_block(1, 1025) == 0 and binding.lib.lantern_forest_block(1 << 22, 1000) == 0
+    unsupported, invalid = 2, 1
+    for parents, n_nodes, width, status in ([[[-1]], [1], 1025, unsupported], [[[-1, 0, 1, 0]], [4], 4, invalid],
+                                            [[[-1, 0]], [3], 3, invalid], [[], [], 4, invalid]):
+        with pytest.raises(LanternError) as e:
+            Forest(parents, n_nodes, width)
+        assert e.value.status == status, (n_nodes, width)
+    if not torch.cuda.is_available():
+        with pytest.raises(LanternError) as e:           # nothing wrong with the tree: the host has no GPU
+            Forest([[-1, 0, 0]], [3])
+        assert e.value.status == 4
