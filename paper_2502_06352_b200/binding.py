@@ -136,9 +136,9 @@ def _ptr(t: Optional[torch.Tensor]):
 
 
 # Current device and raw stream handle without building device and stream objects: those took a
-# quarter of the host time of a call.
-_current_device = torch._C._cuda_getDevice
-_raw_stream = torch._C._cuda_getCurrentRawStream
+# quarter of the host time of a call.  (Private functions of torch: without them, the public ones.)
+_current_device = getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
 
 
 def _call(fn, where, t, *args):

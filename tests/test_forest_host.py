@@ -63,3 +63,20 @@ def test_a_forest_of_refused_arguments_says_so_before_any_device_memory_is_asked
         with pytest.raises(LanternError) as e:           # nothing wrong with the tree: the host has no GPU
             Forest([[-1, 0, 0]], [3])
         assert e.value.status == 4
+
+
+def test_the_package_imports_without_torchs_private_device_functions():
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = ("import torch\n"
+            "for n in ('_cuda_getDevice', '_cuda_getCurrentRawStream'):\n"
+            "    if hasattr(torch._C, n): delattr(torch._C, n)\n"
+            "class S: cuda_stream = 7\n"
+            "torch.cuda.current_device = lambda: 3\n"
+            "torch.cuda.current_stream = lambda dev: S\n"
+            "import paper_2502_06352_b200.binding as b\n"
+            "assert b._current_device() == 3 and b._raw_stream(3) == 7\n")
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-2000:]
