@@ -59,30 +59,28 @@ __device__ __noinline__ void scan_row_after(const T* c, const T* u, float g, flo
   }
 }
 
-// Softmax denominator of a thread's elements relative to a reference m, the first finite vector's maximum: terms in
-// float32 from exact differences, a vector's terms summed in float32 and folded into a double.
+// Softmax denominator of a thread's elements relative to a reference m (-inf: none yet): terms in float32 from exact
+// differences, a vector's terms summed in float32 and folded into a double.  A term's argument is rounded to |z - m| 2^-24,
+// which for z far above m is lost accuracy of a term that makes up the sum: an element more than kRefSlack above the
+// reference becomes the reference, so that its own term is 1.
+constexpr float kRefSlack = 1.f;
 template <int VN>
-__device__ __forceinline__ void fold_exp(const float (&z)[VN], float& m, double& s) {
-  if (m == -INFINITY) {
-#pragma unroll
-    for (int e = 0; e < VN; ++e) m = fmaxf(m, z[e]);
-    if (m == -INFINITY) return;
-  }
+__device__ __forceinline__ float sum_terms(const float (&z)[VN], float m) {
   float part = 0.f;
 #pragma unroll
-  for (int e = 0; e < VN; ++e) part += ex2_approx(__fmul_rn(__fsub_rn(z[e], m), kLog2e));   // (the argument's rounding costs
-                                                                                             // |z - m| 2^-24 relative)
-  if (!(part < 1e30f)) {             // an entry far above the reference: move the reference
-    float bm = m;
+  for (int e = 0; e < VN; ++e) part += ex2_approx(__fmul_rn(__fsub_rn(z[e], m), kLog2e));
+  return part;
+}
+template <int VN>
+__device__ __forceinline__ void fold_exp(const float (&z)[VN], float& m, double& s) {
+  float top = z[0];
 #pragma unroll
-    for (int e = 0; e < VN; ++e) bm = fmaxf(bm, z[e]);
-    s *= exp(static_cast<double>(m) - static_cast<double>(bm));
-    m = bm;
-    part = 0.f;
-#pragma unroll
-    for (int e = 0; e < VN; ++e) part += ex2_approx(__fmul_rn(__fsub_rn(z[e], m), kLog2e));
+  for (int e = 1; e < VN; ++e) top = fmaxf(top, z[e]);
+  if (top > m + kRefSlack) {
+    if (m > -INFINITY) s *= exp(static_cast<double>(m) - static_cast<double>(top));
+    m = top;
   }
-  s += static_cast<double>(part);
+  s += static_cast<double>(sum_terms<VN>(z, m > -INFINITY ? m : 0.f));    // (no finite element so far: 0, or NaN for a NaN)
 }
 
 // One frontier row by one CTA, or by a cluster when a call has few rows: the row is streamed once.  The first
@@ -196,14 +194,15 @@ __global__ void __launch_bounds__(kDynThreads, 4) expand_rows_kernel(const Expan
       for (int u = 0; u < UV; ++u) {
         const int vv = vbeg + 32 * u + lane;
         vec_z(vv, rc[u], ru[u], first[u]);
-        fold_exp<VN>(first[u], m, sum);
 #pragma unroll
         for (int e = 0; e < VN; ++e)
           if (key_before(first[u][e], ge.j0 + vv * VN + e, tbk, tbj)) { tbk = first[u][e]; tbj = ge.j0 + vv * VN + e; }
       }
       Tk = first_threshold(s, K, tbk, tbj);
+      m = first_best(s);                               // the chunk's maximum: few elements of the row lie above it
 #pragma unroll
       for (int u = 0; u < UV; ++u) {
+        sum += static_cast<double>(sum_terms<VN>(first[u], m > -INFINITY ? m : 0.f));
 #pragma unroll
         for (int e = 0; e < VN; ++e)
           if (first[u][e] >= Tk && first[u][e] > -INFINITY) append(first[u][e], ge.j0 + (vbeg + 32 * u + lane) * VN + e);
@@ -223,7 +222,7 @@ __global__ void __launch_bounds__(kDynThreads, 4) expand_rows_kernel(const Expan
 #pragma unroll
         for (int u = 0; u < UF; ++u) io.load(base + 32 * u + lane, rc[u], ru[u]);
         uint32_t hit = 0u;                             // vectors with an entry for the list
-        float part[UF], worst = m == -INFINITY ? INFINITY : 0.f;
+        float part[UF], above = -INFINITY;
 #pragma unroll
         for (int u = 0; u < UF; ++u) {
           float z[VN];
@@ -232,12 +231,10 @@ __global__ void __launch_bounds__(kDynThreads, 4) expand_rows_kernel(const Expan
 #pragma unroll
           for (int e = 1; e < VN; ++e) top = fmaxf(top, z[e]);
           if (top >= Tk) hit |= 1u << u;
-          part[u] = 0.f;
-#pragma unroll
-          for (int e = 0; e < VN; ++e) part[u] += ex2_approx(__fmul_rn(__fsub_rn(z[e], m), kLog2e));
-          worst += part[u];
+          above = fmaxf(above, top);
+          part[u] = sum_terms<VN>(z, m);
         }
-        if (worst < 1e30f) {                           // (one check for all vectors: the reference stays)
+        if (above <= m + kRefSlack && m > -INFINITY) {  // (one check for all vectors: the reference stays)
 #pragma unroll
           for (int u = 0; u < UF; ++u) sum += static_cast<double>(part[u]);
         } else {
@@ -293,7 +290,7 @@ __global__ void __launch_bounds__(kDynThreads, 4) expand_rows_kernel(const Expan
   // ---- the sums relative to the CTA's largest reference, in double precision
   {
     const float wm = warp_max(m);
-    double v = m == -INFINITY ? 0.0 : (m == wm ? sum : sum * exp(static_cast<double>(m) - static_cast<double>(wm)));
+    double v = m == wm || m == -INFINITY ? sum : sum * exp(static_cast<double>(m) - static_cast<double>(wm));   // (-inf: 0 or NaN)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (lane == 0) { wsum[warp] = v; rmax[warp] = wm; }
@@ -304,7 +301,7 @@ __global__ void __launch_bounds__(kDynThreads, 4) expand_rows_kernel(const Expan
   double cs = 0.0;
   if (tid == 0)
     for (int w = 0; w < SW; ++w)
-      if (rmax[w] != -INFINITY) cs += wsum[w] * exp(static_cast<double>(rmax[w]) - static_cast<double>(cm));
+      cs += rmax[w] != -INFINITY ? wsum[w] * exp(static_cast<double>(rmax[w]) - static_cast<double>(cm)) : wsum[w];
   int nf = *s.cnt;
   if (nrank > 1) {
     cluster_wait();                                   // every CTA of the row has started
@@ -325,12 +322,14 @@ __global__ void __launch_bounds__(kDynThreads, 4) expand_rows_kernel(const Expan
     if (nrank > 1) {
       for (uint32_t r = 0; r < nrank; ++r) {
         const float rm = __uint_as_float(s.rinfo[r].y);
-        if (rm != -INFINITY) total += rsum[r] * exp(static_cast<double>(rm) - static_cast<double>(top));
+        total += rm != -INFINITY ? rsum[r] * exp(static_cast<double>(rm) - static_cast<double>(top)) : rsum[r];
       }
-    } else if (cm != -INFINITY) {
-      total = cs * exp(static_cast<double>(cm) - static_cast<double>(top));
+    } else {
+      total = cm != -INFINITY ? cs * exp(static_cast<double>(cm) - static_cast<double>(top)) : cs;
     }
-    wsum[0] = log(total);
+    // at least the top's own term, 1: its float32 stand-in may have lost a few units, and a child's log V never
+    // rises above its parent's (which trimming relies on).  (A NaN stays one.)
+    wsum[0] = total < 1.0 ? 0.0 : log(total);
     wsum[1] = a.pool_logv[static_cast<long long>(b) * a.P + node];
   }
   __syncthreads();

@@ -136,6 +136,14 @@ __device__ __forceinline__ float first_threshold(const TopList& s, int R, float 
   return hit ? __shfl_sync(0xffffffffu, mk, __ffs(hit) - 1) : -INFINITY;
 }
 
+// The best key of the CTA, after first_threshold and before the buffer is written again; -inf when there is none.
+__device__ __forceinline__ float first_best(const TopList& s) {
+  float best = -INFINITY;
+#pragma unroll
+  for (int w = 0; w < SW; ++w) best = fmaxf(best, __uint_as_float(s.pk[2 * w].x));
+  return best;
+}
+
 // CTA 0: the ordered lists that the CTAs of a row pushed (s.fin, lengths in s.rinfo[].x) -> s.list in order; returns
 // their total length.  A barrier separates the result from its readers.
 __device__ __forceinline__ int merge_lists(const TopList& s, uint32_t nrank) {

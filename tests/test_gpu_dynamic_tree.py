@@ -258,3 +258,51 @@ def test_a_forest_is_not_made_inside_a_capture(L):
             x.add_(1)
             L.Forest([[-1, 0, 0]], [3], 3)
     torch.cuda.synchronize()
+
+
+def _trimmed_of_its_own_pool(gpu, m):
+    """The trimmed trees against the host's trimming and numbering of the device's own pool: no near-ties to excuse."""
+    for b in range(gpu["n"].shape[0]):
+        keep = DT.trim(gpu["pool_parent"][b], gpu["pool_logv"][b], m)
+        parent, index = DT.breadth_first(gpu["pool_parent"][b], gpu["pool_depth"][b], keep)
+        n = int(gpu["n"][b])
+        assert n == len(index)
+        assert np.array_equal(gpu["index"][b][:n], index) and np.array_equal(gpu["parent"][b][:n], parent)
+
+
+@pytest.mark.parametrize("V,dtype", [(65536, torch.bfloat16), (16384, torch.float32), (5003, torch.float32)])
+def test_peaked_rows_keep_a_parent_before_its_children(L, V, dtype):
+    """Nearly greedy drafters: the top logit lies 2 to 69 nats above the rest, outside any thread's first vector.  The top's
+    share of the row is 1 to the last bit, so log V must not rise from a node to its child (trimming counts on it)."""
+    D, E, K, m = 6, 8, 8, 59
+    gaps = [2.0, 5.0, 9.0, 15.0, 20.0, 25.0, 27.0, 28.5, 30.0, 31.0, 33.0, 36.0, 40.0, 45.0, 50.0, 57.0, 63.0, 65.0, 68.0, 69.0]
+    B = len(gaps)
+    g = torch.Generator().manual_seed(V)
+    data = torch.randn((D, B, E, V), generator=g)
+    at = torch.randint(V // 2, V - 8, (D, B, E, 1), generator=g)
+    top = data.amax(-1, keepdim=True) + torch.tensor(gaps).view(1, B, 1, 1) + torch.rand((D, B, E, 1), generator=g)
+    data.scatter_(-1, at, top)
+    gpu, orc = _draft(L, data, None, K, E, m, dtype)
+    for b, t in enumerate(orc):
+        par, lv = gpu["pool_parent"][b], gpu["pool_logv"][b]
+        live = np.nonzero(np.isfinite(lv) & (par >= 0))[0]
+        assert np.all(lv[live] <= lv[par[live]]), (gaps[b], float(np.max(lv[live] - lv[par[live]])))
+        Pn = len(t["pool_parent"])
+        if np.array_equal(par[:Pn], t["pool_parent"]) and np.array_equal(gpu["pool_token"][b][:Pn], t["pool_token"]):
+            # Six levels.  A vector's terms are summed in float32: the one with the top, a sum between 1 and 2, is rounded by
+            # up to 2^-24 (3.6e-7 in all); below a gap of 15 nats the other terms' own rounding, 2^-22 of their share, adds as much.
+            assert np.allclose(lv[:Pn], t["pool_logv"], rtol=0, atol=6e-7 if gaps[b] < 15.0 else 6 * 2.0 ** -24), gaps[b]
+    _trimmed_of_its_own_pool(gpu, m)
+
+
+def test_rows_with_nan_logits_give_nan_confidences(L):
+    """One NaN anywhere in a row makes its softmax NaN, also where the thread that meets it has seen nothing else yet."""
+    V = 4096
+    rows = torch.randn((3, 1, V), generator=torch.Generator().manual_seed(1))
+    rows[0, 0, 8:16] = float("nan")
+    rows[1, 0, 3001] = float("nan")
+    pool = L.DraftPool(3, 1, 4, 4)
+    L.expand_frontier(L.Params(vocab=V), pool, rows.cuda())
+    torch.cuda.synchronize()
+    lv = pool.logv.cpu().numpy()[:, 1:5]
+    assert np.all(np.isnan(lv[:2])) and np.all(np.isfinite(lv[2]))
