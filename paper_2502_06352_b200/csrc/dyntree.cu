@@ -434,13 +434,15 @@ __global__ void __launch_bounds__(kDynThreads) trim_tree_kernel(const TrimArgs a
   __syncthreads();
   const int ns = nsel;
   // breadth-first numbering: a level is ordered by (new id of the parent, pool index), one key per entry of the
-  // level (the largest for entries of other levels), so that a place is a count over one array
+  // level (the largest for entries of other levels), so that a place is a count over one array.  An entry whose parent
+  // has no id (in a pool where a child outranks its parent) gets none either.
   for (int dep = 1; dep <= a.max_depth; ++dep) {
     if (tid == 0) level_n = 0;
     const int start = count;
     for (int t = tid; t < ns; t += kDynThreads) {
       const int i = lst[t];
-      lkey[t] = dep_s[i] == dep ? newid[par_s[i]] * kDynMaxPool + i : 0x7fffffff;      // (an id is below kDynMaxPool)
+      const int pi = dep_s[i] == dep && static_cast<unsigned>(par_s[i]) < static_cast<unsigned>(n) ? newid[par_s[i]] : -1;
+      lkey[t] = pi >= 0 ? pi * kDynMaxPool + i : 0x7fffffff;      // (an id is below kDynMaxPool)
     }
     __syncthreads();
     for (int t = tid; t < ns; t += kDynThreads) {

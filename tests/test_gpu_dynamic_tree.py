@@ -295,6 +295,38 @@ def test_peaked_rows_keep_a_parent_before_its_children(L, V, dtype):
     _trimmed_of_its_own_pool(gpu, m)
 
 
+def _trim(L, parent, depth, logv, m):
+    """lantern_trim_tree on pools given by the caller ([B][P] arrays)."""
+    B, P = parent.shape
+    dev = lambda x, dt: torch.as_tensor(np.ascontiguousarray(x)).to(dt).cuda()
+    pp, pd, pl = dev(parent, torch.int32), dev(depth, torch.int32), dev(logv, torch.float64)
+    pt = torch.arange(P, dtype=torch.int32, device="cuda").repeat(B, 1).contiguous()
+    n = torch.empty(B, dtype=torch.int32, device="cuda")
+    out = [torch.full((B, m), -9, dtype=torch.int32, device="cuda") for _ in range(3)]
+    lv = torch.empty((B, m), dtype=torch.float64, device="cuda")
+    p = lambda t: t.data_ptr()
+    st = L.lib.lantern_trim_tree(B, P, P, int(depth.max()), p(pp), p(pt), p(pl), p(pd), m, p(n), p(out[0]), p(out[1]), p(out[2]),
+                                 p(lv), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    return st, n.cpu().numpy(), out[0].cpu().numpy(), out[1].cpu().numpy(), out[2].cpu().numpy(), lv.cpu().numpy()
+
+
+def test_trimming_drops_a_node_whose_parent_was_not_kept(L):
+    """Pools in which a child outranks its parent (no drafting makes them): the child goes with its parent, and so do
+    the child's own children, instead of being hung on another node."""
+    inf = np.inf
+    #          0     1     2     3     4     5     6     7     8    (2 and 5 do not make the cut; 4 under 2, 6 under 4, 8 under 5)
+    parent = [[-1, 0, 0, 0, 2, 1, 4, 1, 5], [-1, 0, 0, 0, 2, 1, 4, 1, 5]]
+    depth = [[0, 1, 1, 1, 2, 2, 3, 2, 3], [0, 1, 1, 1, 2, 2, 3, 2, 3]]
+    logv = [[0, -1.0, -9.0, -2.0, -1.5, -8.0, -1.6, -3.0, -2.5], [0, -1.0, -inf, -2.0, np.nan, -inf, -1.6, -3.0, -inf]]
+    st, n, par, tok, idx, lv = _trim(L, np.array(parent), np.array(depth), np.array(logv), 7)
+    assert st == 0
+    assert list(n) == [4, 4]
+    for b in range(2):
+        assert list(idx[b]) == [0, 1, 3, 7, -1, -1, -1] and list(par[b]) == [-1, 0, 0, 1, -1, -1, -1]
+        assert list(tok[b][:4]) == [-1, 1, 3, 7] and np.array_equal(lv[b][:4], np.array(logv)[b][[0, 1, 3, 7]])
+
+
 def test_rows_with_nan_logits_give_nan_confidences(L):
     """One NaN anywhere in a row makes its softmax NaN, also where the thread that meets it has seen nothing else yet."""
     V = 4096
