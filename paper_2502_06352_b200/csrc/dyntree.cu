@@ -551,6 +551,11 @@ extern "C" lantern_status lantern_trim_tree(int32_t batch, int32_t pool_size, in
   a.B = batch; a.P = pool_size; a.used = pool_used; a.m = max_nodes; a.max_depth = max_depth;
   a.pool_parent = pool_parent; a.pool_token = pool_token; a.pool_depth = pool_depth; a.pool_logv = pool_logv;
   a.n_nodes = n_nodes; a.parent = parent; a.token = token; a.pool_index = pool_index; a.logv = logv;
-  return launch_after_previous(trim_tree_kernel, static_cast<unsigned>(batch), kDynThreads, static_cast<size_t>(pool_used) * 24,
-                               static_cast<cudaStream_t>(stream), 1, a) == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
+  // (a full pool's 48 KB and the kernel's few static bytes are more than a launch gets unasked)
+  const size_t smem = static_cast<size_t>(pool_used) * 24;
+  if (smem > 40 * 1024 &&
+      cudaFuncSetAttribute(trim_tree_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynMaxPool * 24) != cudaSuccess)
+    return LANTERN_ERR_CUDA;
+  return launch_after_previous(trim_tree_kernel, static_cast<unsigned>(batch), kDynThreads, smem, static_cast<cudaStream_t>(stream),
+                               1, a) == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
 }

@@ -327,6 +327,29 @@ def test_trimming_drops_a_node_whose_parent_was_not_kept(L):
         assert list(tok[b][:4]) == [-1, 1, 3, 7] and np.array_equal(lv[b][:4], np.array(logv)[b][[0, 1, 3, 7]])
 
 
+@pytest.mark.parametrize("P,m", [(2047, 300), (2048, 1024), (2048, 7)])
+def test_trimming_the_largest_pools(L, P, m):
+    B = 3
+    rng = np.random.default_rng(P + m)
+    parent = np.full((B, P), -1)
+    depth = np.zeros((B, P), dtype=np.int64)
+    logv = np.zeros((B, P))
+    for b in range(B):
+        for i in range(1, P):
+            q = int(rng.integers(max(0, i - 400), i))
+            while depth[b, q] >= 12:
+                q = parent[b, q]
+            parent[b, i], depth[b, i] = q, depth[b, q] + 1
+            logv[b, i] = logv[b, q] - rng.exponential()
+    st, n, par, tok, idx, lv = _trim(L, parent, depth, logv, m)
+    assert st == 0
+    for b in range(B):
+        want_par, want_idx = DT.breadth_first(parent[b], depth[b], DT.trim(parent[b], logv[b], m))
+        assert int(n[b]) == len(want_idx)
+        assert np.array_equal(idx[b][:n[b]], want_idx) and np.array_equal(par[b][:n[b]], want_par)
+        assert np.array_equal(lv[b][:n[b]], logv[b][want_idx])
+
+
 def test_rows_with_nan_logits_give_nan_confidences(L):
     """One NaN anywhere in a row makes its softmax NaN, also where the thread that meets it has seen nothing else yet."""
     V = 4096
