@@ -205,7 +205,12 @@ def _flat_parents(parents, n_nodes, width):
 
 class Forest(Tree):
     """One tree per sequence, padded to max_nodes (lantern_forest_create_in); used like a Tree.  Its device arrays
-    live in a tensor, so making and dropping one per decode step neither allocates nor synchronises the GPU."""
+    live in a tensor, so making and dropping one per decode step allocates and frees no device memory.  Making one copies
+    the arrays on the current stream and waits for that stream.  Dropping one waits for nothing, the arrays are kept for the
+    streams whose calls have read them; only where a call went into a CUDA graph, whose replays may be on
+    any stream, does dropping wait for the GPU (outside a capture).  A graph must not be replayed after that."""
+
+    captured = False
 
     def __init__(self, parents, n_nodes, max_nodes=None):
         n_nodes = [int(n) for n in n_nodes]
@@ -236,6 +241,13 @@ class Forest(Tree):
         """Work on t's GPU's current stream is about to read the arrays: keep their memory until it is done."""
         if _raw_stream(t.get_device()) != self.stream:
             self.block.record_stream(torch.cuda.current_stream(t.get_device()))
+        if not self.captured and torch.cuda.is_current_stream_capturing():
+            self.captured = True
+
+    def __del__(self):
+        if self.captured and not torch.cuda.is_current_stream_capturing():
+            torch.cuda.synchronize(self.block.device)
+        super().__del__()
 
 
 def _rows(t: torch.Tensor, B, N, V):

@@ -250,6 +250,41 @@ def test_a_forest_dropped_while_another_stream_still_reads_it(L):
         del junk
 
 
+def test_a_forest_dropped_while_a_captured_graph_still_reads_it(L):
+    """A graph replayed on a stream the handle has never seen: dropping the handle waits for the replay, as freeing device
+    memory does."""
+    B, N, V = 64, 24, 4096
+    g = torch.Generator().manual_seed(6)
+    parents = [[-1] + [(i - 1) // (2 + b % 3) for i in range(1, N)] for b in range(B)]
+    tc = torch.randn((B, N, V), generator=g).cuda()
+    tok = torch.randint(0, V, (B, N), generator=g, dtype=torch.int32).cuda()
+    u = torch.rand((2, B, N), generator=g).cuda()
+    par = L.Params(vocab=V, k=0, draft_deterministic=1)
+    forest = L.Forest(parents, [N] * B, N)
+    want = L.verify_tree(par, forest, None, tc, None, None, None, tok, u[0], u[1], debug=True)
+    ws = torch.empty(L.lib.lantern_verify_tree_workspace(forest.handle, B), dtype=torch.uint8, device="cuda")
+    out = {k: torch.full_like(v, -5) for k, v in want.items()}
+    torch.cuda.synchronize()
+    assert not forest.captured
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        L.verify_tree(par, forest, None, tc, None, None, None, tok, u[0], u[1], debug=True, out=out, workspace=ws)
+    assert forest.captured
+    done = torch.cuda.Event()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        torch.cuda._sleep(2_000_000)
+        graph.replay()
+        done.record()
+    size = forest.block.numel()
+    del forest
+    assert done.query()
+    junk = [torch.full((size,), 255, dtype=torch.uint8, device="cuda") for _ in range(8)]
+    torch.cuda.synchronize()
+    for k, v in want.items():
+        assert torch.equal(out[k], v), k
+    del junk
+
+
 def test_a_forest_is_not_made_inside_a_capture(L):
     graph = torch.cuda.CUDAGraph()
     x = torch.zeros(4, device="cuda")
