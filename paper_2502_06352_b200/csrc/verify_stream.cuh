@@ -364,7 +364,8 @@ __device__ __forceinline__ void pass_residual(const IO& ioq, const IO& iop, cons
 // One tree node (sequence b, node n).  Returns the accepted child or -1, the same value in
 // every thread of the node's CTAs.
 // MODE 0: the default acceptance rule, one tree shape.  1: the variants (greedy-skip subset, deterministic drafts,
-// forests) as the arguments say.  2: deterministic drafts with the default subset rule.
+// forests) as the arguments say.  2: deterministic drafts with the default subset rule, whose residual sums come from the
+// banned mass (the general build, short of registers, takes them from the row).
 template <typename T, bool CFG, bool TAU1, int MODE>
 __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, const int n, SCtx& c, const StreamSmem& sm) {
   using IO = RowIO<T, CFG, TAU1>;
@@ -380,6 +381,9 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
   const long long out_b = static_cast<long long>(b) * a.N;
   const int kp1 = a.k + 1;
   const bool writer = c.rank == 0 && tid == 0;
+  constexpr bool kByMass = MODE == 2;       // residual sums from the banned mass
+  // one check for several vectors of the pass; the general build has no registers for it when a vector holds eight elements
+  constexpr bool kBatched = !CFG && (MODE != 1 || VN == 4);
   const bool det = MODE == 2 || (MODE == 1 && a.det != 0);      // deterministic drafts (Sec. 3): p(x) = 1, no drafter row
   const bool skip = MODE == 1 && a.skip != 0;      // greedy-skip subset rule
   const bool has_p = nc > 0 && !det;
@@ -411,7 +415,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
     const int words = (a.V + 31) / 32;
     for (int i = tid; i < words; i += ST) sm.bits[i] = 0u;
   }
-  if (det)
+  if constexpr (kByMass)
     for (int i = tid; i < kMaxCluster * SW + 1; i += ST) sm.wex[i] = 0ull;
   if (tid == 32) {
     fm[7] = a.u_res ? a.u_res[out_b + n]
@@ -477,7 +481,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
     const int hb = max(vbeg, ge.vi0), he = min(vend, ge.vi1);
     if (has_p) {
       // the two rows alternate in the instruction stream so that both are in flight
-      if constexpr (!CFG) {
+      if constexpr (kBatched) {
         float cq = 0.f, cp = 0.f;
         int base = hb;
         for (; base + 32 * U2 <= he; base += 32 * U2) {
@@ -518,7 +522,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
           }
         }
       }
-    } else if constexpr (!CFG) {
+    } else if constexpr (kBatched) {
       float cq = 0.f;
       int base = hb;
       for (; base + 32 * U1 <= he; base += 32 * U1) {
@@ -656,7 +660,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
   float alpha = 0.f, beta = 1.f, ibeta = 1.f, W = 1.f, iW = 1.f;
   int n_dropped = 0;
   int accepted = -1;
-  // Deterministic drafts: the residual after a rejection is q_0 without the banned tokens, so its sum
+  // Deterministic drafts (MODE 2): the residual after a rejection is q_0 without the banned tokens, so its sum
   // is the last sum taken over the row less the banned mass, no pass over the row.  It is summed afresh
   // once half of that sum is gone: until then the subtraction loses at most one bit.
   // (sums below 1e-20 are always taken afresh: their inverse must stay a float32.)
@@ -666,10 +670,12 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
   auto ban = [&](int t, float q0) {
     const uint32_t bit = 1u << (t & 31);
     const uint32_t old = atomicOr(&sm.bits[t >> 5], bit);
-    if (det && !(old & bit) && t >= ge.alo && t < ge.ahi) {
-      const unsigned long long units = static_cast<unsigned long long>(q0 / unit);
-      atomicAdd(&sm.wex[(t - ge.j0) / VN / ge.vw], units);
-      atomicAdd(&sm.wex[kMaxCluster * SW], units);
+    if constexpr (kByMass) {
+      if (!(old & bit) && t >= ge.alo && t < ge.ahi) {
+        const unsigned long long units = static_cast<unsigned long long>(q0 / unit);
+        atomicAdd(&sm.wex[(t - ge.j0) / VN / ge.vw], units);
+        atomicAdd(&sm.wex[kMaxCluster * SW], units);
+      }
     }
   };
   for (int ci = 0; ci < nc; ++ci) {
@@ -815,7 +821,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
     }
     if (!x_dropped) ++n_dropped;
     __syncthreads();
-    if (det) {
+    if constexpr (kByMass) {
       const float left = bsum - static_cast<float>(sm.wex[kMaxCluster * SW]) * unit;
       if (left > 0.5f * bsum && bsum > 1e-20f) {
         beta = left;
@@ -855,7 +861,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
         if (lane < SW) sm.wpart[lane] = sm.wtmp[lane];
         if (lane < static_cast<int>(c.nrank)) sm.rtot[lane] = c.gath[lane * 2];
       }
-      if (det) {                             // (every thread has read the banned mass before the combination)
+      if constexpr (kByMass) {               // (every thread has read the banned mass before the combination)
         for (int i = tid; i < kMaxCluster * SW + 1; i += ST) sm.wex[i] = 0ull;
         bsum = beta;
         unit = fmaxf(beta, 1e-20f) / kMassUnits;
@@ -873,7 +879,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
   // token order: CTA totals locate the CTA, per-warp sums the warp, whose range is then re-read.
   if (accepted < 0) {
     __syncthreads();
-    if (det && banned) {                     // the ranges' sums without the tokens banned since they were taken
+    if (kByMass && banned) {                 // the ranges' sums without the tokens banned since they were taken
       if (tid < static_cast<int>(c.nrank)) {
         unsigned long long gone = 0ull;
         for (int w2 = 0; w2 < SW; ++w2) gone += sm.wex[tid * SW + w2];
@@ -964,7 +970,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
         if (tid == 0) { sm.misc[4] = 0x7fffffff; sm.misc[5] = -1; }
         __syncthreads();
         int found = sm.misc[3];
-        if (det && banned && found < 0) {
+        if (kByMass && banned && found < 0) {
           // Nothing in the range has mass: its sum was what rounding left of a difference.  The first token with mass
           // behind it, else the last before it, by this CTA over the whole row.
           for (int vv = tid; vv < ge.nvec; vv += ST) {
@@ -998,8 +1004,8 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
 }
 
 // MODE 0 (the benchmarked launch) and 2: one node per CTA (cluster); 1: the path walk too.  The modes are builds of their own
-// because what is decided at run time costs registers: the build with everything spills 1.2 to 1.7 KB per thread,
-// and 3776 nodes of deterministic drafts (65536 bfloat16 logits) took 289 us in it, 143 in mode 2.
+// because what is decided at run time costs registers: mode 1 spills 0.4 to 0.9 KB per thread, and 3776 nodes of deterministic
+// drafts (65536 bfloat16 logits) that took 289 us with the banned mass in it (and up to 1.7 KB of spills) take 143 in mode 2.
 template <typename T, bool CFG, bool TAU1, int MODE>
 __global__ void __launch_bounds__(ST, LANTERN_STREAM_MINB) verify_stream_kernel(const VerifyArgs a) {
   grid_dependency_sync();
