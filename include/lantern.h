@@ -147,15 +147,19 @@ typedef struct {
  *   codebook  [L][d] row-major, dt = F32 or BF16            nbr_idx  [L][k] int32
  *   nbr_dist  [L][k] float32 squared distances, or NULL
  *   workspace device scratch of at least lantern_build_neighbors_workspace() bytes, 256-B aligned
- *             (row norms, operand tiles, bounds and candidate lists of the tcgen05 kernels: at most about
- *             300 MB + 7 * L * d bytes; 0 bytes for the brute-force kernel)
+ *             (row norms, operand tiles, bounds and candidate lists of the tcgen05 kernels; with L' = L rounded
+ *             up to a multiple of 128, S = max(1024, L / 4) likewise, d' = d (bfloat16) or 3 d (float32) rounded
+ *             up to a multiple of 16: at most 390 MB + 2 L' d' (float32: 4 L' d') + 2 S d' + 16 (L' + S) bytes;
+ *             0 bytes for the brute-force kernel)
  * 64 <= L, k <= 320 and d <= 256 (bfloat16) or d <= 85 (float32): approximate distances from tcgen05
- * MMAs select a superset of the neighbours (with a proven error margin), which is then ranked exactly.
+ * MMAs select a superset of the neighbours (with a proven error margin), which is then ranked exactly; rows
+ * with more candidates within the margin than are ranked go through the brute-force kernel in the same call.
  * bfloat16 codebooks with d a multiple of 16 in [32, 256], or with L >= 8192 and d a multiple of 8, must
  * be 16-byte aligned and come with the workspace; for the other codebooks of that range a call without
  * it takes the brute-force kernel, which serves everything else too.  The table is the same whichever
- * kernel builds it.  Every wait inside the tcgen05 kernel is bounded; should one run out, the rows of the
- * affected query tiles are written as -1 (never observed; callers may check nbr_idx[i][0] >= 0).
+ * kernel builds it, up to the order of the double-precision additions.  Every wait inside the tcgen05 kernel
+ * is bounded; should one run out, the rows of the affected query tiles are written as -1 (never observed;
+ * callers may check nbr_idx[i][0] >= 0).
  * Requires 1 <= k <= min(L-1, 1024), 1 <= d <= 4096.                                            */
 size_t lantern_build_neighbors_workspace(lantern_dtype dt, int32_t L, int32_t d, int32_t k);
 lantern_status lantern_build_neighbors(const void* codebook, lantern_dtype dt, int32_t L, int32_t d,

@@ -66,3 +66,19 @@ def test_neighbour_table_file_round_trip_and_checksums(tmp_path):
     np.savez(path, **d)
     with pytest.raises(ValueError):
         L.load_neighbors(path, device="cpu")
+
+
+def test_the_stated_bound_of_the_table_workspace_holds():
+    """What include/lantern.h says a caller may budget for lantern_build_neighbors, over sizes at and between the steps of the plan."""
+    up = lambda x, m: -(-x // m) * m
+    for dt, parts, width in ((0, 3, 85), (1, 1, 256)):
+        for n in (64, 127, 128, 1000, 1025, 1153, 2000, 4096, 4097, 8192, 16384, 18944, 18945, 65536, 131073, 500000, 1 << 20, 1 << 22):
+            for d in (1, 5, 8, 16, 33, 64, 85, 100, 256):
+                for k in (1, 10, 100, 200, 320):
+                    got = L.lib.lantern_build_neighbors_workspace(dt, n, d, k)
+                    if d > width:
+                        assert got == 0
+                        continue
+                    rows, sample, wide = up(n, 128), up(max(1024, n // 4), 128), up(parts * d, 16)
+                    bound = 390e6 + (4 if dt == 0 else 2) * rows * wide + 2 * sample * wide + 16 * (rows + sample)
+                    assert 0 < got <= bound, (dt, n, d, k, got, bound)
