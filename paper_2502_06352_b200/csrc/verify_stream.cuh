@@ -563,14 +563,19 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
     }
   }
   // one combination for both rows: per-warp (reference, sum) pairs -> CTA -> cluster; the sums are
-  // rescaled to the common reference in a fixed order, so every thread gets the same values
+  // rescaled to the common reference in a fixed order, so every thread gets the same values.  Where the banned mass is
+  // taken from the sum, the factors are those between the references' offsets in the exponent as they are rounded, so
+  // that the sum is that of the q_0 terms and not off by what those have in common.
   float gm[2], ws[2];
+  auto rescale = [](float m, float ref) {
+    return ex2_approx(kByMass ? __fsub_rn(__fmul_rn(-ref, kLog2e), __fmul_rn(-m, kLog2e)) : (m - ref) * kLog2e);
+  };
   {
     float wm[2] = {warp_max(mx[0]), warp_max(mx[1])};
     float wsum[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-      wsum[i] = warp_sum(mx[i] == -INFINITY ? 0.f : sx[i] * ex2_approx((mx[i] - wm[i]) * kLog2e));
+      wsum[i] = warp_sum(mx[i] == -INFINITY ? 0.f : sx[i] * rescale(mx[i], wm[i]));
     float* red = c.red + c.parity * (SW * 4);
     if (lane == 0) { red[warp * 4] = wm[0]; red[warp * 4 + 1] = wsum[0]; red[warp * 4 + 2] = wm[1]; red[warp * 4 + 3] = wsum[1]; }
     __syncthreads();
@@ -580,7 +585,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const float m2 = red[w2 * 4 + 2 * i];
-        if (m2 != -INFINITY) cs2[i] += red[w2 * 4 + 2 * i + 1] * ex2_approx((m2 - cm[i]) * kLog2e);
+        if (m2 != -INFINITY) cs2[i] += red[w2 * 4 + 2 * i + 1] * rescale(m2, cm[i]);
       }
     }
     gm[0] = cm[0]; gm[1] = cm[1]; ws[0] = cs2[0]; ws[1] = cs2[1];
@@ -597,21 +602,21 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
       for (uint32_t r = 0; r < c.nrank; ++r) {
         const uint32_t base = dsmem_addr(smem_u32(&c.xch[c.parity * 4]), r);
         const float v0 = dsmem_ld_f32(base), v1 = dsmem_ld_f32(base + 4), v2 = dsmem_ld_f32(base + 8), v3 = dsmem_ld_f32(base + 12);
-        if (v0 != -INFINITY) rs[0] += v1 * ex2_approx((v0 - rm[0]) * kLog2e);
-        if (v2 != -INFINITY) rs[1] += v3 * ex2_approx((v2 - rm[1]) * kLog2e);
+        if (v0 != -INFINITY) rs[0] += v1 * rescale(v0, rm[0]);
+        if (v2 != -INFINITY) rs[1] += v3 * rescale(v2, rm[1]);
       }
       gm[0] = rm[0]; gm[1] = rm[1]; ws[0] = rs[0]; ws[1] = rs[1];
     }
     // commit: the current target is q_0 (unnormalised, relative to gm[0])
     if (tid < SW) {
       const float m2 = red[tid * 4];
-      sm.wpart[tid] = m2 == -INFINITY ? 0.f : red[tid * 4 + 1] * ex2_approx((m2 - gm[0]) * kLog2e);
+      sm.wpart[tid] = m2 == -INFINITY ? 0.f : red[tid * 4 + 1] * rescale(m2, gm[0]);
     }
     if (tid < static_cast<int>(c.nrank)) {
       if (c.nrank > 1) {
         const uint32_t base = dsmem_addr(smem_u32(&c.xch[c.parity * 4]), tid);
         const float v0 = dsmem_ld_f32(base), v1 = dsmem_ld_f32(base + 4);
-        sm.rtot[tid] = v0 == -INFINITY ? 0.f : v1 * ex2_approx((v0 - gm[0]) * kLog2e);
+        sm.rtot[tid] = v0 == -INFINITY ? 0.f : v1 * rescale(v0, gm[0]);
       } else {
         sm.rtot[0] = ws[0];
       }
@@ -664,7 +669,10 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
   // is the last sum taken over the row less the banned mass, no pass over the row.  It is summed afresh
   // once half of that sum is gone: until then the subtraction loses at most one bit.
   // (sums below 1e-20 are always taken afresh: their inverse must stay a float32.)
+  // The first of these sums is 1 but for the rounding of the reciprocal rq, which the terms q_0 have in common and a pass
+  // over the row would count.
   float bsum = 1.f, wscale = rq;           // the sum the banned mass is taken from; sm.wpart * wscale is in its units
+  float excess = fmaf(ws[0], rq, -1.f);
   float unit = 1.f / kMassUnits;           // of sm.wex: bsum 2^-40
   bool banned = false;
   auto ban = [&](int t, float q0) {
@@ -822,7 +830,8 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
     if (!x_dropped) ++n_dropped;
     __syncthreads();
     if constexpr (kByMass) {
-      const float left = bsum - static_cast<float>(sm.wex[kMaxCluster * SW]) * unit;
+      const double gone = static_cast<double>(sm.wex[kMaxCluster * SW]) * static_cast<double>(unit);
+      const float left = static_cast<float>(static_cast<double>(bsum) + static_cast<double>(excess) - gone);
       if (left > 0.5f * bsum && bsum > 1e-20f) {
         beta = left;
         ibeta = 1.f / left;
@@ -864,6 +873,7 @@ __device__ __forceinline__ int stream_node(const VerifyArgs& a, const int b, con
       if constexpr (kByMass) {               // (every thread has read the banned mass before the combination)
         for (int i = tid; i < kMaxCluster * SW + 1; i += ST) sm.wex[i] = 0ull;
         bsum = beta;
+        excess = 0.f;
         unit = fmaxf(beta, 1e-20f) / kMassUnits;
         wscale = 1.f;
         banned = false;
