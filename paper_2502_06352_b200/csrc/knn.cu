@@ -379,6 +379,7 @@ __global__ void __launch_bounds__(kKnnThreads) knn_kernel(const KnnArgs a) {
 template <typename T>
 __global__ void __launch_bounds__(kKnnThreads) knn_rest_kernel(const KnnArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  grid_dependency_sync();
   const int total = *a.n_queries;
   for (int q0 = blockIdx.x * a.QT; q0 < total; q0 += gridDim.x * a.QT) {
     knn_tile<T, true>(a, q0, total, smem_raw);
@@ -545,7 +546,9 @@ lantern_status build_t5(const T5Plan& p, const T* cb, int L, int d, int k, int32
     knn_rank_kernel<T><<<queries, kRankThreads, smr, st>>>(r);
   }
   const int groups = (L + b.QT - 1) / b.QT, resident = smb <= 113 * 1024 ? 2 * kT5Items : kT5Items;
-  knn_rest_kernel<T><<<groups < resident ? groups : resident, kKnnThreads, smb, st>>>(b);
+  if (launch_after_previous(knn_rest_kernel<T>, static_cast<unsigned>(groups < resident ? groups : resident), kKnnThreads, smb, st, 1, b) !=
+      cudaSuccess)
+    return LANTERN_ERR_CUDA;
   return cudaGetLastError() == cudaSuccess ? LANTERN_OK : LANTERN_ERR_CUDA;
 }
 
