@@ -90,7 +90,8 @@ __device__ __forceinline__ void fold_exp(const float (&z)[VN], float& m, double&
 // children in the order (z descending, token ascending).
 // Bound: instruction issue and the latency of a chunk's loads.  A depth (rows and frontier) of 512 rows of 65536 bfloat16
 // logits: 33 us, with two passes over the row (maxima, then terms and list) 40; of 8 rows: 14 us, was 25; 512 rows of
-// 40003 logits (most of them unaligned): 27 us, was 92.
+// 40003 logits (most of them unaligned): 27 us, was 92.  (Six depths of 64 sequences and the trimming: 203 us; 199 with
+// the terms relative to a thread's first maximum, which cost accuracy.)
 template <typename T, bool CFG, bool TAU1>
 __global__ void __launch_bounds__(kDynThreads, 4) expand_rows_kernel(const ExpandArgs a) {
   using namespace stream;

@@ -15,7 +15,7 @@
 // top, or within a few units in the last place of logits so large that those are more).  The softmax
 // denominator for draft_prob comes from the same pass.
 //
-// Bound: instruction issue; the generator alone is 10 to 12 of about 20 instructions per element.  3200 rows of
+// Bound: instruction issue; the generator alone is 10 to 12 of about 27 instructions per element.  3200 rows of
 // 65536 bfloat16 logits: 244 us (two logarithms per element and branches between the vectors: 320); 144 rows of
 // 65536 float32 logits with guidance: 28 us, was 40; a row whose elements are one chunk per CTA is a chain of
 // barriers, 8 us on 8 CTAs.
